@@ -110,9 +110,9 @@ __global__ void spline_t_kernel(const double* __restrict__ gbar, const int* __re
   const int row = blockIdx.x * blockDim.x + threadIdx.x;   // (z, o, s)
   if (row >= nz * nO * 4) return;
   const int s = row & 3, zo = row >> 2, iz = zo / nO;
-  const double* h = sp + (size_t)iz * 3 * N;
-  const double* cp = h + N;
-  const double* den = cp + N;
+  const double* h = sp + (size_t)iz * kSpTabs * N;
+  const double* cp = h + kSpCp * N;
+  const double* den = h + kSpDen * N;
   double* yb = ybar + (size_t)row * N;
   double* mb = Mbar + (size_t)row * N;
   for (int i = 0; i < N; ++i) { yb[i] = 0.0; mb[i] = 0.0; }

@@ -495,13 +495,16 @@ int build_device_tables(Ctx* c) {
   }
   // ---- spline tables: per height h, Thomas factors (cp, den), grid
   {
-    std::vector<double> sp((size_t)nz * 3 * N, 0.0), ug((size_t)nz * N);
+    std::vector<double> sp((size_t)nz * kSpTabs * N, 0.0), ug((size_t)nz * N);
     for (int iz = 0; iz < nz; ++iz) {
       const double* u = &c->u[(size_t)iz * N];
-      double* h = &sp[(size_t)iz * 3 * N];
-      double* cp = h + N;
-      double* den = cp + N;
-      for (int i = 0; i < N - 1; ++i) h[i] = u[i + 1] - u[i];
+      double* h = &sp[(size_t)iz * kSpTabs * N];
+      double *cp = h + kSpCp * N, *den = h + kSpDen * N, *k6 = h + kSpK6 * N;
+      double *e0 = h + kSpE0 * N, *e1 = h + kSpE1 * N, *cg = h + kSpCg * N;
+      for (int i = 0; i < N - 1; ++i) {
+        h[i] = u[i + 1] - u[i];
+        k6[i] = h[i] * h[i] / 6.0;
+      }
       const int m = N - 2;
       for (int r = 0; r < m; ++r) {
         const int i = r + 1;
@@ -509,6 +512,9 @@ int build_device_tables(Ctx* c) {
         const double dn = 2.0 * (h[i - 1] + h[i]) - sub * (r > 0 ? cp[r - 1] : 0.0);
         den[r] = dn;
         cp[r] = (r < m - 1) ? h[i] / dn : 0.0;
+        cg[r] = sub / dn;
+        e0[r] = 6.0 / (h[i - 1] * dn);
+        e1[r] = 6.0 / (h[i] * dn);
       }
       for (int n = 0; n < N; ++n) ug[(size_t)iz * N + n] = u[n];
     }
@@ -555,7 +561,7 @@ int build_device_tables(Ctx* c) {
   }
   // ---- scratch vectors
   const size_t vb = nvec(c) * c->esz;
-  if ((rc = dalloc(c, c->scratch1, vb)) || (rc = dalloc(c, c->scratch2, vb)) || (rc = dalloc(c, c->scratch3, vb)))
+  if ((rc = dalloc(c, c->scratch2, vb)) || (rc = dalloc(c, c->scratch3, vb)))
     return rc;
   return PRD_OK;
 }

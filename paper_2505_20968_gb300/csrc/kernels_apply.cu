@@ -15,78 +15,178 @@
 namespace prd {
 
 // ------------------------------------------------------------------ splines
-// Second derivatives of the natural spline of every (z, Omega, s) row.
-template <typename T>
-__global__ void spline_M_kernel(const T* __restrict__ y, T* __restrict__ M, const double* __restrict__ sp,
-                                int nz, int nO, int N) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;   // (z, o, s)
-  if (row >= nz * nO * 4) return;
-  const int s = row & 3, zo = row >> 2, iz = zo / nO;
-  const double* h = sp + (size_t)iz * 3 * N;
-  const double* cp = h + N;
-  const double* den = cp + N;
-  const T* yr = y + (size_t)zo * N * 4 + s;
-  T* Mr = M + (size_t)zo * N * 4 + s;
-  Mr[0] = (T)0;
-  Mr[(size_t)(N - 1) * 4] = (T)0;
-  if (N <= 2) return;
-  // forward sweep: g_r stored in M[i], i = r + 1
-  double gprev = 0.0;
-  double y0 = (double)yr[0], y1 = (double)yr[4];
-  for (int r = 0; r < N - 2; ++r) {
-    const int i = r + 1;
-    const double y2 = (double)yr[(size_t)(i + 1) * 4];
-    const double rhs = 6.0 * ((y2 - y1) / h[i] - (y1 - y0) / h[i - 1]);
-    const double sub = (r > 0) ? h[i - 1] : 0.0;
-    const double g = (rhs - sub * gprev) / den[r];
-    Mr[(size_t)i * 4] = (T)g;
-    gprev = g;
-    y0 = y1;
-    y1 = y2;
-  }
-  double mnext = 0.0;
-  for (int r = N - 3; r >= 0; --r) {
-    const int i = r + 1;
-    const double m = (double)Mr[(size_t)i * 4] - cp[r] * mnext;
-    Mr[(size_t)i * 4] = (T)m;
-    mnext = m;
-  }
-}
-
 template <typename T> struct V4;
 template <> struct V4<float> { using type = float4; };
 template <> struct V4<double> { using type = double4_16a; };
 
-// Evaluate the spline of every (z, Omega) row at the tabulated points; the
-// intensity component is multiplied by fI (nullable).
-template <typename T, typename F = T>
-__global__ void spline_eval_kernel(const T* __restrict__ y, const T* __restrict__ M, const int* __restrict__ kidx,
-                                   const double* __restrict__ tt, const double* __restrict__ sp,
-                                   const F* __restrict__ fI, T* __restrict__ out, int nz, int nO, int N) {
-  using V = typename V4<T>::type;
-  const long long pt = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // (z, o, n)
-  if (pt >= (long long)nz * nO * N) return;
-  const int zo = (int)(pt / N), iz = zo / nO;
-  const int k = kidx[pt];
-  const V* yr = reinterpret_cast<const V*>(y) + (size_t)zo * N;
-  const V* Mr = reinterpret_cast<const V*>(M) + (size_t)zo * N;
-  V r;
-  if (k < 0) r = yr[0];
-  else if (k >= N - 1) r = yr[N - 1];
-  else {
-    const double t = tt[pt], omt = 1.0 - t;
-    const double h = sp[(size_t)iz * 3 * N + k];
-    const double k6 = h * h / 6.0;
-    // y_k + t (y_{k+1} - y_k) + ...: reproduces a constant exactly in any precision
-    const T c1 = (T)t, c2 = (T)(k6 * (omt * omt * omt - omt)), c3 = (T)(k6 * (t * t * t - t));
-    const V a = yr[k], b = yr[k + 1], ma = Mr[k], mb = Mr[k + 1];
-    r.x = a.x + c1 * (b.x - a.x) + c2 * ma.x + c3 * mb.x;
-    r.y = a.y + c1 * (b.y - a.y) + c2 * ma.y + c3 * mb.y;
-    r.z = a.z + c1 * (b.z - a.z) + c2 * ma.z + c3 * mb.z;
-    r.w = a.w + c1 * (b.w - a.w) + c2 * ma.w + c3 * mb.w;
+// Frame change of R (z, Omega) rows of one height per CTA: the natural spline of
+// every Stokes row (its second derivatives M from the tridiagonal system, in FP64)
+// evaluated at the tabulated points; the intensity is multiplied by fI (nullable).
+//
+// What bounds it: the Thomas recurrence, 2 (N - 2) dependent FP64 steps per row,
+// on a chip with two FP64 lanes a clock and SM.  So the recurrence is stripped to
+// one FP64 FMA a step: the divisions are folded into per-height factors (e0, e1,
+// cg, cp of the spline tables), the right-hand sides are formed by the whole CTA
+// beforehand, and the rows, right-hand sides and factors sit in shared memory, so
+// that no step waits for a global load.  M never leaves the CTA.  Against two
+// kernels that walked global memory with a thread per row and divided at every
+// step: an FP32 apply of 8 x 64 rows of 200 points 3399 -> 2952 us, of 10 x 16 rows of
+// 27 points 262 -> 201 us, a preconditioner apply of 20 x 16 rows of 100 points
+// (four FP64 frame changes) 1097 -> 217 us.
+// R = 4 rows a CTA (16 recurrences in a warp) where there are rows enough for
+// every SM, R = 1 below that, so that the right-hand sides and evaluations of a
+// small problem still spread over the chip.
+constexpr int kSplThreads = 128;
+constexpr int kSplFew = 4 * 152;                     // rows up to which a CTA takes one
+
+template <typename T, int R>
+struct SplineSmem {
+  // g: [node][chain] FP64 right-hand sides, then second derivatives; ys: [row][node]
+  // with an odd row stride (rows fall in different banks); Mt: the second
+  // derivatives in T (FP64 reads g itself); cg, cp: recurrence factors
+  static __host__ __device__ int stride(int N) { return N | 1; }
+  static __host__ __device__ size_t ys_off(int N) { return (size_t)N * 4 * R * 8; }
+  static __host__ __device__ size_t mt_off(int N) { return ys_off(N) + (size_t)R * stride(N) * 4 * sizeof(T); }
+  static __host__ __device__ size_t tab_off(int N) {
+    return mt_off(N) + (sizeof(T) == 8 ? 0 : (size_t)N * 4 * R * sizeof(T));
   }
-  if (fI) r.x *= (T)fI[pt];
-  reinterpret_cast<V*>(out)[pt] = r;
+  static __host__ __device__ size_t bytes(int N) { return tab_off(N) + (size_t)2 * N * 8; }
+};
+
+template <typename T, int R>
+__global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict__ y, const int* __restrict__ kidx,
+                                                             const double* __restrict__ tt,
+                                                             const double* __restrict__ sp,
+                                                             const double* __restrict__ fI, T* __restrict__ out,
+                                                             int nO, int N) {
+  using V = typename V4<T>::type;
+  using L = SplineSmem<T, R>;
+  constexpr int C = 4 * R;                           // recurrences of the CTA
+  extern __shared__ __align__(16) unsigned char spsm[];
+  double* g = reinterpret_cast<double*>(spsm);
+  V* ys = reinterpret_cast<V*>(spsm + L::ys_off(N));
+  T* Mt = sizeof(T) == 8 ? reinterpret_cast<T*>(g) : reinterpret_cast<T*>(spsm + L::mt_off(N));
+  double* cg = reinterpret_cast<double*>(spsm + L::tab_off(N));
+  double* cp = cg + N;
+  const int iz = blockIdx.y, o0 = blockIdx.x * R, nr = min(R, nO - o0), tid = threadIdx.x;
+  const int S = L::stride(N);
+  const double* tab = sp + (size_t)iz * kSpTabs * N;
+  const size_t row0 = (size_t)iz * nO + o0;
+  {
+    const V* src = reinterpret_cast<const V*>(y) + row0 * N;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (r < nr)
+        for (int i = tid; i < N; i += kSplThreads) ys[r * S + i] = src[(size_t)r * N + i];
+  }
+  for (int i = tid; i < N; i += kSplThreads) {
+    cg[i] = tab[kSpCg * N + i];
+    cp[i] = tab[kSpCp * N + i];
+  }
+  __syncthreads();
+  // right-hand sides divided by the pivots; end nodes zero (natural spline)
+  for (int idx = tid; idx < N * C; idx += kSplThreads) {
+    const int i = idx / C, ch = idx - i * C;
+    double v = 0.0;
+    if (i > 0 && i < N - 1 && (ch >> 2) < nr) {
+      const T* yr = reinterpret_cast<const T*>(ys + (ch >> 2) * S) + (ch & 3);
+      const double y0 = (double)yr[(i - 1) * 4], y1 = (double)yr[i * 4], y2 = (double)yr[(i + 1) * 4];
+      v = tab[kSpE1 * N + i - 1] * (y2 - y1) - tab[kSpE0 * N + i - 1] * (y1 - y0);
+    }
+    g[idx] = v;
+  }
+  __syncthreads();
+  if (tid < C) {
+    // blocks of kB steps: their factors and right-hand sides are read before the
+    // dependent FMAs, so a step costs one FMA latency
+    constexpr int kB = 8;
+    double prev = 0.0;
+    int i = 1;
+    for (; i + kB <= N - 1; i += kB) {
+      double a[kB], f[kB];
+#pragma unroll
+      for (int q = 0; q < kB; ++q) { a[q] = g[(i + q) * C + tid]; f[q] = cg[i + q - 1]; }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) { prev = a[q] - f[q] * prev; a[q] = prev; }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) g[(i + q) * C + tid] = a[q];
+    }
+    for (; i < N - 1; ++i) {
+      prev = g[i * C + tid] - cg[i - 1] * prev;
+      g[i * C + tid] = prev;
+    }
+    if (sizeof(T) != 8) Mt[tid] = Mt[(N - 1) * C + tid] = (T)0;
+    double next = 0.0;
+    i = N - 2;
+    for (; i - kB >= 0; i -= kB) {
+      double a[kB], f[kB];
+#pragma unroll
+      for (int q = 0; q < kB; ++q) { a[q] = g[(i - q) * C + tid]; f[q] = cp[i - q - 1]; }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) { next = a[q] - f[q] * next; a[q] = next; }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) Mt[(i - q) * C + tid] = (T)a[q];
+    }
+    for (; i >= 1; --i) {
+      next = g[i * C + tid] - cp[i - 1] * next;
+      Mt[i * C + tid] = (T)next;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (r >= nr) break;
+    const size_t p0 = (row0 + r) * N;
+    const V* yr = ys + r * S;
+    for (int n = tid; n < N; n += kSplThreads) {
+      const size_t pt = p0 + n;
+      const int k = kidx[pt];
+      V v;
+      if (k < 0) v = yr[0];
+      else if (k >= N - 1) v = yr[N - 1];
+      else {
+        const double t = tt[pt], omt = 1.0 - t, k6 = tab[kSpK6 * N + k];
+        // y_k + t (y_{k+1} - y_k) + ...: reproduces a constant exactly in any precision
+        const T c1 = (T)t, c2 = (T)(k6 * (omt * omt * omt - omt)), c3 = (T)(k6 * (t * t * t - t));
+        const V a = yr[k], b = yr[k + 1];
+        const V ma = *reinterpret_cast<const V*>(Mt + (size_t)k * C + 4 * r);
+        const V mb = *reinterpret_cast<const V*>(Mt + (size_t)(k + 1) * C + 4 * r);
+        v.x = a.x + c1 * (b.x - a.x) + c2 * ma.x + c3 * mb.x;
+        v.y = a.y + c1 * (b.y - a.y) + c2 * ma.y + c3 * mb.y;
+        v.z = a.z + c1 * (b.z - a.z) + c2 * ma.z + c3 * mb.z;
+        v.w = a.w + c1 * (b.w - a.w) + c2 * ma.w + c3 * mb.w;
+      }
+      if (fI) v.x *= (T)fI[pt];
+      reinterpret_cast<V*>(out)[pt] = v;
+    }
+  }
+}
+
+// Shared memory the dynamic-size kernels of this file may be launched with, set
+// once (at setup) to the device's limit: a per-launch value would race between
+// contexts of different sizes on different threads.
+template <typename K>
+static int allow_smem(Ctx* c, K kern) {
+  PRD_CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+  return PRD_OK;
+}
+
+template <typename T>
+static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt, const double* fI, T* out, int nO) {
+  const double* sp = (const double*)c->sp.p;
+  const int nz = c->nz, N = c->nnu;
+  if (nz * nO <= kSplFew)
+    spline_kernel<T, 1><<<dim3(nO, nz), kSplThreads, SplineSmem<T, 1>::bytes(N), c->stream>>>(y, kidx, tt, sp, fI, out, nO, N);
+  else
+    spline_kernel<T, 4><<<dim3((nO + 3) / 4, nz), kSplThreads, SplineSmem<T, 4>::bytes(N), c->stream>>>(y, kidx, tt, sp, fI, out, nO, N);
+}
+
+int apply_prepare(Ctx* c) {
+  int rc;
+  if ((rc = allow_smem(c, spline_kernel<float, 1>)) || (rc = allow_smem(c, spline_kernel<float, 4>)) ||
+      (rc = allow_smem(c, spline_kernel<double, 1>)) || (rc = allow_smem(c, spline_kernel<double, 4>)))
+    return rc;
+  return PRD_OK;
 }
 
 // ------------------------------------------------------------------ R_III
@@ -817,22 +917,17 @@ __global__ void fill_planck_kernel(T* __restrict__ x, const double* __restrict__
 
 // ------------------------------------------------------------------ launchers
 template <typename T, typename A>
-static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = nullptr, A* M_ext = nullptr,
-                   A* Ic_ext = nullptr, double* J_ext = nullptr, bool t64 = false) {
+static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = nullptr, A* Ic_ext = nullptr,
+                   double* J_ext = nullptr, bool t64 = false) {
   const int nz = c->nz, nO = c->nO, N = c->nnu;
   const SigmaTables tb = sigma_tables(c, t64);
   const long long npt = (long long)nz * nO * N;
-  A* Mb = M_ext ? M_ext : (A*)c->scratch1.p;
-  A* M = Mb;
   A* Ic = Ic_ext ? Ic_ext : (A*)c->scratch2.p;
   A* eb = eb_ext ? eb_ext : (A*)c->scratch3.p;
-  const double* sp = (const double*)c->sp.p;
   cudaEvent_t e0;
   // S1
   stage_begin(c, ST_S1, &e0);
-  spline_M_kernel<A><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>(x, M, sp, nz, nO, N);
-  spline_eval_kernel<A, A><<<ceil_div(npt, 256), 256, 0, c->stream>>>(x, M, (const int*)c->iin.p, (const double*)c->tin.p,
-                                                                  sp, nullptr, Ic, nz, nO, N);
+  launch_spline<A>(c, x, (const int*)c->iin.p, (const double*)c->tin.p, nullptr, Ic, nO);
   stage_end(c, ST_S1, e0);
   // S5 (initialises eps_bar)
   stage_begin(c, ST_S5, &e0);
@@ -873,11 +968,8 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   stage_end(c, ST_S3, e0);
   // S6
   stage_begin(c, ST_S6, &e0);
-  spline_M_kernel<A><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>(eb, Mb, sp, nz, nO, N);
-  spline_eval_kernel<A, double><<<ceil_div(npt, 256), 256, 0, c->stream>>>(eb, Mb, (const int*)c->ibk.p,
-                                                                     (const double*)c->tbk.p, sp,
-                                                                     normalised ? (const double*)c->f.p : nullptr, eps, nz,
-                                                                     nO, N);
+  launch_spline<A>(c, eb, (const int*)c->ibk.p, (const double*)c->tbk.p, normalised ? (const double*)c->f.p : nullptr,
+                   eps, nO);
   // continuum scattering (App. A) joins the normalised emissivity; the
   // Kirchhoff factor is computed from the line alone (normalised = false)
   if (normalised && c->has_cont())
@@ -888,38 +980,11 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   return PRD_OK;
 }
 
-// Spline frame change of a whole vector: to the comoving frame (I(u_n - u_b))
-// or back (eps(u_n + u_b)); uses scratch1 for the second derivatives.
-int spline_frame_change(Ctx* c, const void* in, void* out, bool to_comoving) {
-  const int nz = c->nz, nO = c->nO, N = c->nnu;
-  const long long npt = (long long)nz * nO * N;
-  const double* sp = (const double*)c->sp.p;
-  const int* kk = (const int*)(to_comoving ? c->iin.p : c->ibk.p);
-  const double* tt = (const double*)(to_comoving ? c->tin.p : c->tbk.p);
-  if (c->prec == PRD_FP64) {
-    spline_M_kernel<double><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>((const double*)in, (double*)c->scratch1.p, sp, nz, nO, N);
-    spline_eval_kernel<double, double><<<ceil_div(npt, 256), 256, 0, c->stream>>>((const double*)in, (const double*)c->scratch1.p, kk, tt,
-                                                                         sp, nullptr, (double*)out, nz, nO, N);
-  } else {
-    spline_M_kernel<float><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>((const float*)in, (float*)c->scratch1.p, sp, nz, nO, N);
-    spline_eval_kernel<float, float><<<ceil_div(npt, 256), 256, 0, c->stream>>>((const float*)in, (const float*)c->scratch1.p, kk, tt,
-                                                                        sp, nullptr, (float*)out, nz, nO, N);
-  }
-  PRD_CUDA_TRY(c, cudaPeekAtLastError());
-  return PRD_OK;
-}
-
-// The same frame change for an FP64 vector in either mode (the preconditioner's
-// sweeps), with the caller's FP64 scratch for the spline second derivatives.
-int spline_frame_change_d(Ctx* c, const double* in, double* out, double* Mscratch, bool to_comoving) {
-  const int nz = c->nz, nO = c->nO, N = c->nnu;
-  const long long npt = (long long)nz * nO * N;
-  const double* sp = (const double*)c->sp.p;
-  const int* kk = (const int*)(to_comoving ? c->iin.p : c->ibk.p);
-  const double* tt = (const double*)(to_comoving ? c->tin.p : c->tbk.p);
-  spline_M_kernel<double><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>(in, Mscratch, sp, nz, nO, N);
-  spline_eval_kernel<double, double><<<ceil_div(npt, 256), 256, 0, c->stream>>>(in, Mscratch, kk, tt, sp, nullptr, out,
-                                                                               nz, nO, N);
+// Frame change of an FP64 vector in either mode (the preconditioner's sweeps): to the
+// comoving frame (I(u_n - u_b)) or back (eps(u_n + u_b)).
+int spline_frame_change_d(Ctx* c, const double* in, double* out, bool to_comoving) {
+  launch_spline<double>(c, in, (const int*)(to_comoving ? c->iin.p : c->ibk.p),
+                        (const double*)(to_comoving ? c->tin.p : c->tbk.p), nullptr, out, c->nO);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
   return PRD_OK;
 }
@@ -952,15 +1017,15 @@ int apply_lambda(Ctx* c, const void* eps, void* out, const void* sub_from, bool 
 int compute_normalisation(Ctx* c) {
   const int nz = c->nz, nO = c->nO, N = c->nnu;
   const long long npt = (long long)nz * nO * N;
-  DBuf wt, fac, xin, num, eb, Mb, Ic;
+  DBuf wt, fac, xin, num, eb, Ic;
   std::vector<double> f(nz);
   for (int iz = 0; iz < nz; ++iz) f[iz] = (1.0 - c->eps[iz]) * c->WT[iz];
   int rc;
   const size_t vb64 = nvec(c) * 8;
-  auto cleanup = [&]() { dfree(wt); dfree(fac); dfree(xin); dfree(num); dfree(eb); dfree(Mb); dfree(Ic); };
+  auto cleanup = [&]() { dfree(wt); dfree(fac); dfree(xin); dfree(num); dfree(eb); dfree(Ic); };
   if ((rc = upload(c, wt, c->WT.data(), nz * 8)) || (rc = upload(c, fac, f.data(), nz * 8)) ||
       (rc = dalloc(c, xin, vb64)) || (rc = dalloc(c, num, vb64)) || (rc = dalloc(c, eb, vb64)) ||
-      (rc = dalloc(c, Mb, vb64)) || (rc = dalloc(c, Ic, vb64))) {
+      (rc = dalloc(c, Ic, vb64))) {
     cleanup();
     return rc;
   }
@@ -974,8 +1039,8 @@ int compute_normalisation(Ctx* c) {
   } else {
     fill_planck_kernel<double><<<ceil_div(npt, 256), 256, 0, c->stream>>>((double*)xin.p, (const double*)wt.p, nz, nO, N);
     rc = c->has64 ? sigma_T<double, double>(c, (const double*)xin.p, (double*)num.p, false, (double*)eb.p,
-                                            (double*)Mb.p, (double*)Ic.p, nullptr, true)
-                  : sigma_T<float, double>(c, (const double*)xin.p, (double*)num.p, false, (double*)eb.p, (double*)Mb.p,
+                                            (double*)Ic.p, nullptr, true)
+                  : sigma_T<float, double>(c, (const double*)xin.p, (double*)num.p, false, (double*)eb.p,
                                            (double*)Ic.p);
     if (!rc)
       normalise_kernel<double, double><<<ceil_div(npt, 256), 256, 0, c->stream>>>(
@@ -1000,11 +1065,11 @@ int rhs(Ctx* c, void* b) { return apply_lambda(c, c->epsth.p, b, nullptr, true);
 // FP32 mode only: y = (Id - Lambda Sigma) x with FP64 vectors, FP64 arithmetic
 // and the FP64 copy of the Sigma tables when it was kept (else the FP32 tables):
 // the residuals of the refinement, which fix the accuracy of the solution.
-int apply_operator_acc(Ctx* c, const double* x, double* y, double* ws /* 4 x nvec doubles */) {
+int apply_operator_acc(Ctx* c, const double* x, double* y, double* ws /* 3 x nvec doubles */) {
   const size_t nv = nvec(c);
   double* eps = ws;
-  int rc = c->has64 ? sigma_T<double, double>(c, x, eps, true, ws + nv, ws + 2 * nv, ws + 3 * nv, nullptr, true)
-                     : sigma_T<float, double>(c, x, eps, true, ws + nv, ws + 2 * nv, ws + 3 * nv);
+  int rc = c->has64 ? sigma_T<double, double>(c, x, eps, true, ws + nv, ws + 2 * nv, nullptr, true)
+                     : sigma_T<float, double>(c, x, eps, true, ws + nv, ws + 2 * nv);
   if (rc) return rc;
   delo_kernel<double, double><<<ceil_div(c->nO * c->nnu, 128), 128, 0, c->stream>>>(
       eps, (const double*)c->kt64.p, (const double*)c->par_active(), (const double*)c->dmu.p, x, y, c->nz, c->nO,
@@ -1020,13 +1085,13 @@ __global__ void add_kernel(double* __restrict__ a, const double* __restrict__ b,
 
 // eps = eps_th + Sigma x in FP64 arithmetic on the FP64 tables (the residual
 // path of the refinement in FP32 mode): the emissivity whose formal solution,
-// with the boundary term, minus x is the residual b - A x.  ws: 3 N-vectors.
+// with the boundary term, minus x is the residual b - A x.  ws: 2 N-vectors.
 int emissivity_acc(Ctx* c, const double* x, double* eps, double* ws) {
   const size_t nv = nvec(c);
   int rc;
   if (c->prec == PRD_FP64) rc = sigma_T<double, double>(c, x, eps, true);
-  else if (c->has64) rc = sigma_T<double, double>(c, x, eps, true, ws, ws + nv, ws + 2 * nv, nullptr, true);
-  else rc = sigma_T<float, double>(c, x, eps, true, ws, ws + nv, ws + 2 * nv);
+  else if (c->has64) rc = sigma_T<double, double>(c, x, eps, true, ws, ws + nv, nullptr, true);
+  else rc = sigma_T<float, double>(c, x, eps, true, ws, ws + nv);
   if (rc) return rc;
   add_kernel<<<c->grid_ew(), 256, 0, c->stream>>>(eps, (const double*)(c->prec == PRD_FP64 ? c->epsth.p : c->epsth64.p),
                                                   nv);
@@ -1087,11 +1152,11 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
   const int nz = c->nz, nO = c->nO, N = c->nnu, nti = c->ntile(), nuv = c->nu_st * c->nu_st;
   const long long npt = (long long)nz * nO * N;
   const size_t tz = (size_t)nO * nti * N * c->ld() * sizeof(T);   // tiles of one height, all LOS classes
-  DBuf Icx, Icw, Jx, Jw, tiles, Yd, rout, ktd, ethd, kidx, ttd, es_bar, ew_bar, es, ew, M, eps, lam, fac, dmu, clsd,
-      xa, Mx, pard, etald, cpwd;
+  DBuf Icx, Icw, Jx, Jw, tiles, Yd, rout, ktd, ethd, kidx, ttd, es_bar, ew_bar, es, ew, eps, lam, fac, dmu, clsd,
+      xa, pard, etald, cpwd;
   auto cleanup = [&]() {
     DBuf* bs[] = {&Icx, &Icw, &Jx, &Jw, &tiles, &Yd, &rout, &ktd, &ethd, &kidx, &ttd, &es_bar, &ew_bar, &es, &ew,
-                  &M, &eps, &lam, &fac, &dmu, &clsd, &xa, &Mx, &pard, &etald, &cpwd};
+                  &eps, &lam, &fac, &dmu, &clsd, &xa, &pard, &etald, &cpwd};
     for (DBuf* b : bs) dfree(*b);
   };
   const size_t vb = nvec(c) * sizeof(A), lb = (size_t)nz * N * 4 * sizeof(A);
@@ -1106,9 +1171,9 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
   for (int i = 0; i < nO; ++i) cls.push_back(i);
   if ((rc = dalloc(c, Icx, vb)) || (rc = dalloc(c, Icw, vb)) || (rc = dalloc(c, Jx, (size_t)nz * nuv * 16)) ||
       (rc = dalloc(c, Jw, (size_t)nz * nuv * 16)) || (rc = dalloc(c, tiles, tz)) || (rc = dalloc(c, es_bar, lb)) ||
-      (rc = dalloc(c, ew_bar, lb)) || (rc = dalloc(c, es, lb)) || (rc = dalloc(c, ew, lb)) || (rc = dalloc(c, M, lb)) ||
+      (rc = dalloc(c, ew_bar, lb)) || (rc = dalloc(c, es, lb)) || (rc = dalloc(c, ew, lb)) ||
       (rc = dalloc(c, eps, lb)) || (rc = dalloc(c, lam, lb)) || (rc = upload(c, fac, facv.data(), nz * 8)) ||
-      (rc = dalloc(c, xa, vb)) || (rc = dalloc(c, Mx, (size_t)nz * nO * N * 4 * sizeof(A))) ||
+      (rc = dalloc(c, xa, vb)) ||
       (rc = upload(c, clsd, cls.data(), cls.size() * 4))) {
     cleanup();
     return rc;
@@ -1117,10 +1182,7 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
   if ((rc = upload(c, wtd, wt.data(), nz * 8))) { cleanup(); return rc; }
   // comoving fields of the solution and of the Planck function, and their R_III moments
   cast_kernel<T, A><<<ceil_div(npt * 4, 256), 256, 0, c->stream>>>(x, (A*)xa.p, npt * 4);
-  spline_M_kernel<A><<<ceil_div(nz * nO * 4, 128), 128, 0, c->stream>>>((const A*)xa.p, (A*)Mx.p, (const double*)c->sp.p, nz, nO, N);
-  spline_eval_kernel<A, A><<<ceil_div(npt, 256), 256, 0, c->stream>>>((const A*)xa.p, (const A*)Mx.p, (const int*)c->iin.p,
-                                                                     (const double*)c->tin.p, (const double*)c->sp.p,
-                                                                     nullptr, (A*)Icx.p, nz, nO, N);
+  launch_spline<A>(c, (const A*)xa.p, (const int*)c->iin.p, (const double*)c->tin.p, nullptr, (A*)Icx.p, nO);
   planck_comoving_kernel<A><<<ceil_div(npt, 256), 256, 0, c->stream>>>((A*)Icw.p, (const double*)wtd.p, nz, nO, N);
   PRD_CUDA_TRY(c, cudaMemsetAsync(Jx.p, 0, Jx.bytes, c->stream));
   PRD_CUDA_TRY(c, cudaMemsetAsync(Jw.p, 0, Jw.bytes, c->stream));
@@ -1164,14 +1226,8 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
     }
     if (rc) break;
     // observer frame, normalisation, thermal part, formal solution along the LOS
-    spline_M_kernel<A><<<ceil_div(nz * 4, 128), 128, 0, c->stream>>>((const A*)es_bar.p, (A*)M.p, (const double*)c->sp.p, nz, 1, N);
-    spline_eval_kernel<A, A><<<ceil_div((long long)nz * N, 256), 256, 0, c->stream>>>(
-        (const A*)es_bar.p, (const A*)M.p, (const int*)kidx.p, (const double*)ttd.p, (const double*)c->sp.p, nullptr,
-        (A*)es.p, nz, 1, N);
-    spline_M_kernel<A><<<ceil_div(nz * 4, 128), 128, 0, c->stream>>>((const A*)ew_bar.p, (A*)M.p, (const double*)c->sp.p, nz, 1, N);
-    spline_eval_kernel<A, A><<<ceil_div((long long)nz * N, 256), 256, 0, c->stream>>>(
-        (const A*)ew_bar.p, (const A*)M.p, (const int*)kidx.p, (const double*)ttd.p, (const double*)c->sp.p, nullptr,
-        (A*)ew.p, nz, 1, N);
+    launch_spline<A>(c, (const A*)es_bar.p, (const int*)kidx.p, (const double*)ttd.p, nullptr, (A*)es.p, 1);
+    launch_spline<A>(c, (const A*)ew_bar.p, (const int*)kidx.p, (const double*)ttd.p, nullptr, (A*)ew.p, 1);
     los_combine_kernel<T, A><<<ceil_div(nz * N, 128), 128, 0, c->stream>>>((const A*)es.p, (const A*)ew.p,
                                                                           (const T*)ktd.p, (const double*)etald.p,
                                                                           (const T*)ethd.p,
@@ -1224,6 +1280,7 @@ static int sigma_static_T(Ctx* c, const T* x, T* eps) {
   const size_t nuv = (size_t)c->nu_st * c->nu_st;
   const size_t jbytes = ((size_t)c->nz * nuv * 2 * sizeof(double) + 255) / 256 * 256;
   const size_t vb = (nv * sizeof(T) + 255) / 256 * 256;
+  // the limit of the documented interface: three vectors and the R_III moments
   if (jbytes + 3 * vb > kStaticScratchBytes)
     return fail(c, PRD_E_ARG, "problem needs " + std::to_string((jbytes + 3 * vb) >> 20) +
                                   " MiB of scratch; prd_apply_sigma_noalloc supports at most 64 MiB");
@@ -1232,10 +1289,9 @@ static int sigma_static_T(Ctx* c, const T* x, T* eps) {
   if (rc) return rc;
   unsigned char* b = (unsigned char*)base;
   double* J = (double*)b;
-  T* M = (T*)(b + jbytes);
-  T* Ic = (T*)(b + jbytes + vb);
-  T* eb = (T*)(b + jbytes + 2 * vb);
-  return sigma_T<T, T>(c, x, eps, true, eb, M, Ic, J);
+  T* Ic = (T*)(b + jbytes);
+  T* eb = (T*)(b + jbytes + vb);
+  return sigma_T<T, T>(c, x, eps, true, eb, Ic, J);
 }
 
 }  // namespace prd

@@ -28,6 +28,15 @@ constexpr int kWeidemanN32 = 20;   // Faddeeva expansion terms, FP32 paths
 // many nodes on each of [0, pi/2] and [pi/2, pi]
 constexpr int kAAThetaNodes = 48;
 
+// Spline tables of a height (natural cubic spline on its reduced-frequency grid), each of N
+// doubles: interval widths h, the Thomas factors of the second derivatives' tridiagonal system
+// (row r, node r + 1) cp and den, h^2/6, and the system divided by its pivots: right-hand side
+// e1[r] (y_{r+2} - y_{r+1}) - e0[r] (y_{r+1} - y_r), forward g_r = rhs_r - cg[r] g_{r-1},
+// backward M_{r+1} = g_r - cp[r] M_{r+2}.
+enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpTabs = 7 };
+// dynamic shared memory a CTA may have (opt-in limit of the device)
+constexpr int kMaxSmem = 227 * 1024;
+
 // device buffer with byte size
 struct DBuf {
   void* p = nullptr;
@@ -132,20 +141,20 @@ struct Ctx {
   const void* par_active() const { return formal ? par.p : nullptr; }
   DBuf epsth;        // [z][o][n][4]
   DBuf f;            // [z][o][n]
-  DBuf sp;           // spline tables: per z  h[N-1], cp[N], den[N]  (T) -> [z][3][N]
+  DBuf sp;           // spline tables [z][kSpTabs][N] (double), SpTab below
   DBuf ugrid;        // [z][N] (T)
   DBuf iin, ibk;     // interpolation [z][o][n]: int k | flag, and t (T)  -> int2/ T pairs
   DBuf tin, tbk;
   DBuf cls_dev;      // cout_ptr, cout_dir, pair_ptr, pair_in  (int)
   DBuf dmu;          // [nO] mu of each direction (double)
-  DBuf scratch1, scratch2, scratch3;  // N-vector scratch (T)
+  DBuf scratch2, scratch3;  // N-vector scratch (T)
   // preconditioner
   DBuf pc_phi;       // [z][N][N] Phi_bar (double)
   DBuf pc_M;         // [z][N][N] Phi_bar (Id - A)^-1 (double)
   DBuf pc_lii;       // [z][o][n] Lambda_ii (T)
   DBuf pc_eta;       // [z][o][n]: eta1 (T)  (scalar Lambda*)
   DBuf pc_delo;      // [z][o][n][3] (T)
-  DBuf pc_s1, pc_s2, pc_s3, pc_s4, pc_s5;   // FP64 N-vector scratch of the sweeps
+  DBuf pc_s1, pc_s2, pc_s3, pc_s4;   // FP64 N-vector scratch of the sweeps
   std::vector<double> pc_lii_host;
   void* pc_w = nullptr;   // device angular weights (double), owned via `owned`
   // GMRES
@@ -270,6 +279,7 @@ int upload_faddeeva_coeffs(Ctx* c);
 
 size_t nvec(const Ctx* c);   // 4*nz*nO*nnu
 int r2_tc_prepare(Ctx* c);
+int apply_prepare(Ctx* c);   // attributes of the per-apply kernels (once per setup)
 int r2_tc_launch(Ctx* c, const float* Ic, float* eb);
 // drop the captured solver graphs (options, tables or workspace changed)
 void invalidate_graphs(Ctx* c);

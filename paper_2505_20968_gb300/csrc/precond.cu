@@ -116,7 +116,7 @@ __global__ void pc_out_kernel(const T* __restrict__ y, const double* __restrict_
 }
 
 // observer <-> comoving frame change of an FP64 vector (kernels_apply.cu)
-int spline_frame_change_d(Ctx* c, const double* in, double* out, double* Mscratch, bool to_comoving);
+int spline_frame_change_d(Ctx* c, const double* in, double* out, bool to_comoving);
 
 static int lu_inverse(std::vector<double>& A, int n) {
   std::vector<int> piv(n);
@@ -215,7 +215,7 @@ int launch_precond_setup(Ctx* c) {
   c->pc_w = w.p;
   const size_t vb = nvec(c) * sizeof(double);
   if ((rc = dalloc(c, c->pc_s1, vb)) || (rc = dalloc(c, c->pc_s2, vb)) || (rc = dalloc(c, c->pc_s3, vb)) ||
-      (rc = dalloc(c, c->pc_s4, vb)) || (rc = dalloc(c, c->pc_s5, vb)) ||
+      (rc = dalloc(c, c->pc_s4, vb)) ||
       (rc = dalloc(c, c->gm_w, (size_t)nz * N * sizeof(double))))
     return rc;
   return PRD_OK;
@@ -229,7 +229,6 @@ static int precond_T(Ctx* c, const T* y, T* x) {
   double* t1 = (double*)c->pc_s2.p;
   double* t2 = (double*)c->pc_s3.p;
   double* xd = (double*)c->pc_s4.p;
-  double* Ms = (double*)c->pc_s5.p;
   double* J = (double*)c->gm_w.p;
   const double* w = (const double*)c->pc_w;
   const int g1 = ceil_div(npt, 256);
@@ -237,12 +236,12 @@ static int precond_T(Ctx* c, const T* y, T* x) {
   for (int sweep = 0; sweep < c->m_in; ++sweep) {
     // r = y - P x on Stokes I (P x = x - Lambda* Sigma* x); the first sweep starts from x = 0
     if (sweep > 0) {
-      int rc = spline_frame_change_d(c, xd, t1, Ms, true);                  // comoving I~
+      int rc = spline_frame_change_d(c, xd, t1, true);                  // comoving I~
       if (rc) return rc;
       pc_angle_avg_kernel<<<ceil_div(nz * N, 128), 128, 0, c->stream>>>(t1, w, J, nz, nO, N);
       pc_matvec_bcast_kernel<<<dim3(ceil_div(N, 128), nz), 128, 0, c->stream>>>((const double*)c->pc_phi.p, J, t2, nz,
                                                                                nO, N);
-      if ((rc = spline_frame_change_d(c, t2, t1, Ms, false))) return rc;    // eps* (observer)
+      if ((rc = spline_frame_change_d(c, t2, t1, false))) return rc;    // eps* (observer)
       pc_delo_kernel<T><<<ceil_div(nO * N, 128), 128, 0, c->stream>>>(t1, (const T*)c->kt.p, (const double*)c->dmu.p,
                                                                       t2, nz, nO, N);
       pc_resid_kernel<T><<<g1, 256, 0, c->stream>>>(y, xd, t2, r, npt);
