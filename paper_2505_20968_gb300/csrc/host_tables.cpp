@@ -501,9 +501,11 @@ int build_device_tables(Ctx* c) {
       double* h = &sp[(size_t)iz * kSpTabs * N];
       double *cp = h + kSpCp * N, *den = h + kSpDen * N, *k6 = h + kSpK6 * N;
       double *e0 = h + kSpE0 * N, *e1 = h + kSpE1 * N, *cg = h + kSpCg * N;
+      double *iden = h + kSpIden * N, *s6 = h + kSp6h * N;
       for (int i = 0; i < N - 1; ++i) {
         h[i] = u[i + 1] - u[i];
         k6[i] = h[i] * h[i] / 6.0;
+        s6[i] = 6.0 / h[i];
       }
       const int m = N - 2;
       for (int r = 0; r < m; ++r) {
@@ -513,6 +515,7 @@ int build_device_tables(Ctx* c) {
         den[r] = dn;
         cp[r] = (r < m - 1) ? h[i] / dn : 0.0;
         cg[r] = sub / dn;
+        iden[r] = 1.0 / dn;
         e0[r] = 6.0 / (h[i - 1] * dn);
         e1[r] = 6.0 / (h[i] * dn);
       }

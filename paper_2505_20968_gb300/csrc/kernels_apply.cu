@@ -1143,6 +1143,61 @@ __global__ void cast_kernel(const S* __restrict__ in, D* __restrict__ out, long 
   if (i < n) out[i] = (D)in[i];
 }
 
+// R_II along one line of sight: es_bar[z][n][i] += sum over the incident directions o' (each
+// its own scattering angle) and tiles of Re(T[n][m] Z[m][i]), Z = Y I~, in FP64, and the same
+// for the Planck field (W_T, 0, 0, 0), which is flat in frequency: only the row sums of T and
+// Y_00 enter, into the intensity of ew_bar.  A thread takes a tile row n, a CTA the tiles
+// [tg * y, tg * (y + 1)) of one direction and height (grid.z = heights z0 ..): both fields share
+// one read of the tile, and small problems get a CTA per tile.  FP64-bound (six operations a
+// tile element); the generic contraction, a launch per height and field of one CTA per
+// direction, took 6.6 ms a height at 16 directions x 41 frequencies.
+template <typename T>
+__global__ void los_r2_kernel(const T* __restrict__ tiles, const T* __restrict__ Y, const double* __restrict__ Ic,
+                              const double* __restrict__ WT, double* __restrict__ es, double* __restrict__ ew, int z0,
+                              int ncls, int nO, int nti, int N, int ld, int tiled, int tg) {
+  extern __shared__ __align__(16) unsigned char lsm[];
+  double* Z = reinterpret_cast<double*>(lsm);              // [m][zr(4) | zi(4)]
+  const int op = blockIdx.x, zl = blockIdx.z, iz = z0 + zl, n = threadIdx.x;
+  const int c = ncls == 1 ? 0 : op;                        // angle-averaged: one class for all directions
+  const double4_16a* I = reinterpret_cast<const double4_16a*>(Ic) + ((size_t)iz * nO + op) * N;
+  double acc[4] = {0, 0, 0, 0}, accw = 0.0;
+  const double W = WT[iz];
+  for (int ti = blockIdx.y * tg; ti < min(nti, (int)(blockIdx.y + 1) * tg); ++ti) {
+    const T* y = Y + (((size_t)iz * nO + op) * nti + ti) * 32;
+    __syncthreads();
+    for (int m = threadIdx.x; m < N; m += blockDim.x) {
+      const double4_16a v = I[m];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const T* yi = y + i * 8;
+        Z[m * 8 + i] = (double)yi[0] * v.x + (double)yi[2] * v.y + (double)yi[4] * v.z + (double)yi[6] * v.w;
+        Z[m * 8 + 4 + i] = (double)yi[1] * v.x + (double)yi[3] * v.y + (double)yi[5] * v.z + (double)yi[7] * v.w;
+      }
+    }
+    __syncthreads();
+    if (n < N) {
+      const T* t = tiles + (((size_t)zl * ncls + c) * nti + ti) * N * ld;
+      double sr = 0.0, si = 0.0;
+#pragma unroll 4
+      for (int m = 0; m < N; ++m) {
+        const double ar = (double)t[tile_off(n, m, N, ld, tiled != 0)], ai = (double)t[tile_off(n, N + m, N, ld, tiled != 0)];
+        const double* z = Z + m * 8;
+        sr += ar;
+        si += ai;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] += ar * z[i] - ai * z[4 + i];
+      }
+      accw += W * ((double)y[0] * sr - (double)y[1] * si);
+    }
+  }
+  if (n < N) {
+    double* e = es + ((size_t)iz * N + n) * 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) atomicAdd(e + i, acc[i]);
+    atomicAdd(ew + ((size_t)iz * N + n) * 4, accw);
+  }
+}
+
 // T: precision of the stored tables and of x / out; A: precision of the fields
 // along the line of sight (double in FP32 mode, like the FP64-accumulated
 // residual path, so the emergent spectrum carries no FP32 cancellation).
@@ -1151,35 +1206,30 @@ template <typename T, typename A>
 static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const double* chis, T* out) {
   const int nz = c->nz, nO = c->nO, N = c->nnu, nti = c->ntile(), nuv = c->nu_st * c->nu_st;
   const long long npt = (long long)nz * nO * N;
-  const size_t tz = (size_t)nO * nti * N * c->ld() * sizeof(T);   // tiles of one height, all LOS classes
-  DBuf Icx, Icw, Jx, Jw, tiles, Yd, rout, ktd, ethd, kidx, ttd, es_bar, ew_bar, es, ew, eps, lam, fac, dmu, clsd,
+  const int ncl = c->mode == PRD_MODE_AA ? 1 : nO;               // scattering angles of a line of sight
+  const size_t tz = (size_t)ncl * nti * N * c->ld() * sizeof(T);   // tiles of one height
+  DBuf Icx, Icw, Jx, Jw, tiles, Yd, rout, ktd, ethd, kidx, ttd, es_bar, ew_bar, es, ew, eps, lam, fac, dmu, wtd,
       xa, pard, etald, cpwd;
+  int rc, zb = 1;
+  LosTiles* lt = los_tiles_create(c, ncl, &zb, &rc);
+  if (!lt) return rc;
   auto cleanup = [&]() {
     DBuf* bs[] = {&Icx, &Icw, &Jx, &Jw, &tiles, &Yd, &rout, &ktd, &ethd, &kidx, &ttd, &es_bar, &ew_bar, &es, &ew,
-                  &eps, &lam, &fac, &dmu, &clsd, &xa, &pard, &etald, &cpwd};
+                  &eps, &lam, &fac, &dmu, &wtd, &xa, &pard, &etald, &cpwd};
     for (DBuf* b : bs) dfree(*b);
+    los_tiles_destroy(lt);
   };
   const size_t vb = nvec(c) * sizeof(A), lb = (size_t)nz * N * 4 * sizeof(A);
-  int rc;
   std::vector<double> facv(nz), wt(c->WT);
   for (int iz = 0; iz < nz; ++iz) facv[iz] = (1.0 - c->eps[iz]) * c->WT[iz];
-  // class structure of one LOS: class o' has the single output entry 0 and the single pair (LOS, o')
-  std::vector<int> cls;
-  for (int i = 0; i <= nO; ++i) cls.push_back(i);
-  for (int i = 0; i < nO; ++i) cls.push_back(0);
-  for (int i = 0; i <= nO; ++i) cls.push_back(i);
-  for (int i = 0; i < nO; ++i) cls.push_back(i);
   if ((rc = dalloc(c, Icx, vb)) || (rc = dalloc(c, Icw, vb)) || (rc = dalloc(c, Jx, (size_t)nz * nuv * 16)) ||
-      (rc = dalloc(c, Jw, (size_t)nz * nuv * 16)) || (rc = dalloc(c, tiles, tz)) || (rc = dalloc(c, es_bar, lb)) ||
+      (rc = dalloc(c, Jw, (size_t)nz * nuv * 16)) || (rc = dalloc(c, tiles, tz * zb)) || (rc = dalloc(c, es_bar, lb)) ||
       (rc = dalloc(c, ew_bar, lb)) || (rc = dalloc(c, es, lb)) || (rc = dalloc(c, ew, lb)) ||
       (rc = dalloc(c, eps, lb)) || (rc = dalloc(c, lam, lb)) || (rc = upload(c, fac, facv.data(), nz * 8)) ||
-      (rc = dalloc(c, xa, vb)) ||
-      (rc = upload(c, clsd, cls.data(), cls.size() * 4))) {
+      (rc = dalloc(c, xa, vb)) || (rc = upload(c, wtd, wt.data(), nz * 8))) {
     cleanup();
     return rc;
   }
-  DBuf wtd;
-  if ((rc = upload(c, wtd, wt.data(), nz * 8))) { cleanup(); return rc; }
   // comoving fields of the solution and of the Planck function, and their R_III moments
   cast_kernel<T, A><<<ceil_div(npt * 4, 256), 256, 0, c->stream>>>(x, (A*)xa.p, npt * 4);
   launch_spline<A>(c, (const A*)xa.p, (const int*)c->iin.p, (const double*)c->tin.p, nullptr, (A*)Icx.p, nO);
@@ -1190,7 +1240,6 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
   launch_r3_J<T, A>(c, (const A*)Icx.p, (double*)Jx.p, nO, tb);
   launch_r3_J<T, A>(c, (const A*)Icw.p, (double*)Jw.p, nO, tb);
   PRD_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  const double mu1 = 1.0;
   for (int l = 0; l < nlos && !rc; ++l) {
     LosTables L;
     los_tables(c, mus[l], chis[l], L);
@@ -1205,26 +1254,21 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
         (rc = upload(c, kidx, L.kidx.data(), L.kidx.size() * 4)) || (rc = upload(c, ttd, L.tt.data(), L.tt.size() * 8)) ||
         (rc = upload(c, dmu, &mus[l], 8)))
       break;
-    (void)mu1;
     // R_III parts initialise the comoving rows
     launch_r3_out<T, A>(c, (const double*)Jx.p, (const T*)rout.p, (A*)es_bar.p, 1, tb);
     launch_r3_out<T, A>(c, (const double*)Jw.p, (const T*)rout.p, (A*)ew_bar.p, 1, tb);
-    // R_II: tiles of every height for the LOS classes, then the contraction
-    for (int iz = 0; iz < nz && !rc; ++iz) {
-      std::vector<double> th(L.theta);
-      if ((rc = gen_tiles_z(c, iz, th, tiles.p))) break;
-      const size_t smem = sizeof(A) * (size_t)kMB * 2 * kCW * 4 + sizeof(T) * (size_t)2 * N * (kMB + 1);
-      cudaFuncSetAttribute(r2_simt_kernel<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      const T* Yz = (const T*)Yd.p + (size_t)iz * nO * nti * 32;
-      r2_simt_kernel<T, A><<<dim3(1, nO, 1), 256, smem, c->stream>>>(
-          (const T*)tiles.p, Yz, (const A*)Icx.p + (size_t)iz * nO * N * 4, (const int*)clsd.p,
-          (A*)es_bar.p + (size_t)iz * N * 4, nO, nti, nO, N, nO, c->ld(), c->tiled());
-      r2_simt_kernel<T, A><<<dim3(1, nO, 1), 256, smem, c->stream>>>(
-          (const T*)tiles.p, Yz, (const A*)Icw.p + (size_t)iz * nO * N * 4, (const int*)clsd.p,
-          (A*)ew_bar.p + (size_t)iz * N * 4, nO, nti, nO, N, nO, c->ld(), c->tiled());
-      PRD_CUDA_TRY(c, cudaPeekAtLastError());
+    // R_II: tiles of the heights for the LOS classes, zb heights at a time, then the contraction
+    if (ncl > 1 && (rc = los_tiles_angles(c, lt, L.theta))) break;
+    const int tg = (size_t)nO * nz >= 608 ? nti : 1;
+    for (int z0 = 0; z0 < nz && !rc; z0 += zb) {
+      const int n = std::min(zb, nz - z0);
+      if ((rc = los_tiles_gen(c, lt, z0, n, tiles.p))) break;
+      los_r2_kernel<T><<<dim3(nO, (nti + tg - 1) / tg, n), (N + 31) / 32 * 32, (size_t)N * 64, c->stream>>>(
+          (const T*)tiles.p, (const T*)Yd.p, (const double*)Icx.p, (const double*)wtd.p, (double*)es_bar.p,
+          (double*)ew_bar.p, z0, ncl, nO, nti, N, c->ld(), c->tiled(), tg);
     }
     if (rc) break;
+    PRD_CUDA_TRY(c, cudaPeekAtLastError());
     // observer frame, normalisation, thermal part, formal solution along the LOS
     launch_spline<A>(c, (const A*)es_bar.p, (const int*)kidx.p, (const double*)ttd.p, nullptr, (A*)es.p, 1);
     launch_spline<A>(c, (const A*)ew_bar.p, (const int*)kidx.p, (const double*)ttd.p, nullptr, (A*)ew.p, 1);
@@ -1244,7 +1288,6 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
                                                                   out + (size_t)l * N * 4, (long long)N * 4);
     PRD_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   }
-  dfree(wtd);
   cleanup();
   return rc;
 }

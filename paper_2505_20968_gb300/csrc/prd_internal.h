@@ -23,7 +23,6 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr double kSqrtPi = 1.77245385090551602730;
 
 constexpr int kWeidemanN64 = 36;   // Faddeeva expansion terms, FP64 paths
-constexpr int kWeidemanN32 = 20;   // Faddeeva expansion terms, FP32 paths
 // Angle-averaged R_II (Eq. R_AA): composite Gauss-Legendre in Theta with this
 // many nodes on each of [0, pi/2] and [pi/2, pi]
 constexpr int kAAThetaNodes = 48;
@@ -32,8 +31,8 @@ constexpr int kAAThetaNodes = 48;
 // doubles: interval widths h, the Thomas factors of the second derivatives' tridiagonal system
 // (row r, node r + 1) cp and den, h^2/6, and the system divided by its pivots: right-hand side
 // e1[r] (y_{r+2} - y_{r+1}) - e0[r] (y_{r+1} - y_r), forward g_r = rhs_r - cg[r] g_{r-1},
-// backward M_{r+1} = g_r - cp[r] M_{r+2}.
-enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpTabs = 7 };
+// backward M_{r+1} = g_r - cp[r] M_{r+2}; the reciprocal pivots, and 6/h.
+enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpIden = 7, kSp6h = 8, kSpTabs = 9 };
 // dynamic shared memory a CTA may have (opt-in limit of the device)
 constexpr int kMaxSmem = 227 * 1024;
 
@@ -249,7 +248,12 @@ struct LosTables {
   std::vector<double> tt;      // [z][N]
 };
 void los_tables(const Ctx* c, double mu, double chi, LosTables& L);
-int gen_tiles_z(Ctx* c, int iz, const std::vector<double>& thetas, void* outT);
+// tiles of a line of sight's scattering angles, zb heights at a time (kernels_tiles.cu)
+struct LosTiles;
+LosTiles* los_tiles_create(Ctx* c, int ncl, int* zb, int* rc);
+void los_tiles_destroy(LosTiles* t);
+int los_tiles_angles(Ctx* c, LosTiles* t, const std::vector<double>& thetas);
+int los_tiles_gen(Ctx* c, LosTiles* t, int z0, int n, void* out);
 // DELOPAR source weights of a step of optical thickness dM followed downwind by dP
 void delopar_weights(double dM, double dP, double* psi);
 // dipole (Rayleigh) phase matrix P[4][4] from direction (mu_p, chi_p) into (mu_o, chi_o)
