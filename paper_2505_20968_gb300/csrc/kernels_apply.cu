@@ -7,7 +7,8 @@
 //   S6  frame change back (u_n + u_b(z,Omega)) and Kirchhoff factor f (App. E)
 //   S7+S8  DELO-linear sweep per ray, y = x - Lambda eps      (Sect. 3)
 #include <cstdio>
-#include <mutex>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <type_traits>
 #include "prd_internal.h"
 #include "device_common.cuh"
@@ -181,14 +182,6 @@ static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt,
     spline_kernel<T, 4><<<dim3((nO + 3) / 4, nz), kSplThreads, SplineSmem<T, 4>::bytes(N), c->stream>>>(y, kidx, tt, sp, fI, out, nO, N);
 }
 
-int apply_prepare(Ctx* c) {
-  int rc;
-  if ((rc = allow_smem(c, spline_kernel<float, 1>)) || (rc = allow_smem(c, spline_kernel<float, 4>)) ||
-      (rc = allow_smem(c, spline_kernel<double, 1>)) || (rc = allow_smem(c, spline_kernel<double, 4>)))
-    return rc;
-  return PRD_OK;
-}
-
 // ------------------------------------------------------------------ R_III
 // J[z][ku kv] += sum_{o', j} rin[z][o'][q][j] * sum_m r3w[z][q][m] I~[z][o'][m][j],  q = (ku kv, l')
 // One block per (o', z): the direction's comoving row I~[z][o'][.][.] is staged in
@@ -271,12 +264,15 @@ __global__ void r3_out_kernel(const double* __restrict__ J, const T* __restrict_
 // FP64 copies kept for the refinement residuals.
 struct SigmaTables {
   const void *tiles, *Y, *r3w, *r3in, *r3out, *r3prof, *r3ab;
-  int ld, tiled;
+  int ld, fmt;
+  const float* tsc;
 };
 static SigmaTables sigma_tables(const Ctx* c, bool t64) {
   if (t64)
-    return {c->tiles64.p, c->Y64.p, c->r3w64.p, c->r3in64.p, c->r3out64.p, c->r3prof64.p, c->r3ab64.p, c->ld64(), 0};
-  return {c->tiles.p, c->Y.p, c->r3w.p, c->r3in.p, c->r3out.p, c->r3prof.p, c->r3ab.p, c->ld(), c->tiled() ? 1 : 0};
+    return {c->tiles64.p, c->Y64.p, c->r3w64.p, c->r3in64.p, c->r3out64.p, c->r3prof64.p, c->r3ab64.p, c->ld64(), TILE_PLAIN,
+            nullptr};
+  return {c->tiles.p, c->Y.p, c->r3w.p, c->r3in.p, c->r3out.p, c->r3prof.p, c->r3ab.p, c->ld(), c->tile_fmt(),
+          (const float*)c->tile_scale.p};
 }
 
 // launchers (shared by the apply and the line-of-sight paths)
@@ -304,11 +300,24 @@ constexpr int kCW = 16;      // output directions per CTA
 constexpr int kMB = 16;      // incident-frequency block
 constexpr int kMaxRows = 16; // rows per thread (N <= 256)
 
+// element (n, k) of the stored tile at t (format fmt, row scale sc)
+template <typename T>
+__device__ __forceinline__ T tile_get(const unsigned char* t, int n, int k, int N, int ld, int fmt, float sc) {
+  if (sizeof(T) == 8 || fmt == TILE_PLAIN) return reinterpret_cast<const T*>(t)[(size_t)n * ld + k];
+  if (fmt == TILE_FP16) {
+    const __half* h = reinterpret_cast<const __half*>(t);
+    return (T)((__half2float(h[tile_off_split(n, k, N, ld, false)]) + __half2float(h[tile_off_split(n, k, N, ld, true)])) * sc);
+  }
+  const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(t);
+  if (fmt == TILE_BF16HI) return (T)__bfloat162float(b[tile_off_hi(n, k, N, ld)]);
+  return (T)(__bfloat162float(b[tile_off_split(n, k, N, ld, false)]) + __bfloat162float(b[tile_off_split(n, k, N, ld, true)]));
+}
+
 template <typename T, typename A>
-__global__ void __launch_bounds__(256) r2_simt_kernel(const T* __restrict__ tiles, const T* __restrict__ Y,
+__global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __restrict__ tiles, const float* __restrict__ tsc, const T* __restrict__ Y,
                                                       const A* __restrict__ Ic, const int* __restrict__ cls,
                                                       A* __restrict__ eb, int ncls, int ntrip, int nO, int N,
-                                                      int npairs, int ld, int tiled) {
+                                                      int npairs, int ld, int fmt) {
   const int chunk = blockIdx.x, c = blockIdx.y, iz = blockIdx.z;
   const int* cout_ptr = cls;
   const int* cout_dir = cls + ncls + 1;
@@ -331,13 +340,14 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const T* __restrict__ tile
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[r][i] = (A)0;
   const int nrows = (N + 15) / 16;
-  const size_t tile_sz = (size_t)N * ld;
-  const T* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
+  const size_t tile_sz = (size_t)N * ld * (fmt == TILE_BF16HI ? 2 : sizeof(T));
+  const unsigned char* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
+  const float* sc = fmt == TILE_FP16 ? tsc + ((size_t)iz * ncls + c) * N : nullptr;
   // Z-building role: thread -> (e = tid & 15, m = tid >> 4)
   const int ze = tid & 15, zm = tid >> 4;
   const int e_z = e0 + ze;
   for (int t = 0; t < ntrip; ++t) {
-    const T* tile = tbase + (size_t)t * tile_sz;
+    const unsigned char* tile = tbase + (size_t)t * tile_sz;
     for (int m0 = 0; m0 < N; m0 += kMB) {
       // ---- Z block
       {
@@ -369,7 +379,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const T* __restrict__ tile
         const int h = (idx / kMB) & 1;
         const int n = idx / (2 * kMB);
         const int m = m0 + mm;
-        Asb[(h * N + n) * (kMB + 1) + mm] = (m < N) ? tile[tile_off(n, h * N + m, N, ld, tiled != 0)] : (T)0;
+        Asb[(h * N + n) * (kMB + 1) + mm] = (m < N) ? tile_get<T>(tile, n, h * N + m, N, ld, fmt, sc ? sc[n] : 1.f) : (T)0;
       }
       __syncthreads();
 #pragma unroll 4
@@ -916,6 +926,16 @@ __global__ void fill_planck_kernel(T* __restrict__ x, const double* __restrict__
 }
 
 // ------------------------------------------------------------------ launchers
+int apply_prepare(Ctx* c) {
+  int rc;
+  if ((rc = allow_smem(c, spline_kernel<float, 1>)) || (rc = allow_smem(c, spline_kernel<float, 4>)) ||
+      (rc = allow_smem(c, spline_kernel<double, 1>)) || (rc = allow_smem(c, spline_kernel<double, 4>)) ||
+      (rc = allow_smem(c, r2_simt_kernel<float, float>)) || (rc = allow_smem(c, r2_simt_kernel<float, double>)) ||
+      (rc = allow_smem(c, r2_simt_kernel<double, double>)) || (rc = allow_smem(c, r2_dd_kernel)))
+    return rc;
+  return PRD_OK;
+}
+
 template <typename T, typename A>
 static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = nullptr, A* Ic_ext = nullptr,
                    double* J_ext = nullptr, bool t64 = false) {
@@ -951,7 +971,6 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   if constexpr (std::is_same<T, double>::value && std::is_same<A, double>::value) {
     if (t64) {
       const size_t smem = sizeof(float4) * (size_t)kMB * kCW * 4 + sizeof(float2) * (size_t)2 * N * (kMB + 1);
-      cudaFuncSetAttribute(r2_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       r2_dd_kernel<<<dim3(nchunk, c->ncls, nz), 256, smem, c->stream>>>(
           (const double*)tb.tiles, (const double*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(), nO, N,
           c->npairs, tb.ld);
@@ -960,10 +979,9 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   }
   if (!s3_done) {
     const size_t smem = sizeof(A) * (size_t)kMB * 2 * kCW * 4 + sizeof(T) * (size_t)2 * N * (kMB + 1);
-    cudaFuncSetAttribute(r2_simt_kernel<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     r2_simt_kernel<T, A><<<dim3(nchunk, c->ncls, nz), 256, smem, c->stream>>>(
-        (const T*)tb.tiles, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(), nO, N, c->npairs,
-        tb.ld, tb.tiled);
+        (const unsigned char*)tb.tiles, tb.tsc, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(),
+        nO, N, c->npairs, tb.ld, tb.fmt);
   }
   stage_end(c, ST_S3, e0);
   // S6

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include "prd_internal.h"
 #include "device_common.cuh"
 
@@ -521,63 +522,78 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) r3_kernel(R3Params p, floa
 //   tiles[c][ngrp + t][.] = G_t - mean of its group
 // so that the large dispersion parts that cancel between Zeeman components
 // of one J level are summed once, in FP64, before rounding to the storage type.
-// the FP32 value v of a tile entry stored as bf16 planes hi = rn(v), lo = rn(v - hi)
-__device__ __forceinline__ void store_split(__nv_bfloat16* t, int n, int k, int N, int ld, float v) {
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  t[tile_off_split(n, k, N, ld, false)] = hi;
-  t[tile_off_split(n, k, N, ld, true)] = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
+// One CTA per (row n, class, height); formats of the stored element (n, k):
+//   TILE_PLAIN  T, rows of ld (tiled: the FP32 K-step layout of tile_off)
+//   TILE_FP16   FP16 planes hi = rn(s v), lo = rn(s v - hi), s a power of two per (class, n) that
+//               brings the row's largest element over all tiles of the class to [2^13, 2^14);
+//               tsc[c][n] = 1/s
+//   TILE_BF16   bf16 planes (BF16x3), TILE_BF16HI the hi plane alone (BF16x2)
+constexpr int kSplitThreads = 128;
 
-// split: 0 the storage type T (plain or tiled), 1 the bf16 hi and lo planes of
-// BF16x3 contexts (the bytes of an FP32 tile), 2 the hi plane alone (BF16x2:
-// half the bytes; dst is then read as bf16 with tiles of N ld elements)
 template <typename T>
-__global__ void group_split_kernel(const double* __restrict__ src, T* __restrict__ dst, const int* __restrict__ grp,
-                                   int ncls, int ntrip, int ngrp, int N, int ld, int tiled, int split) {
-  const int rowlen = 2 * N * N;                 // one FP64 scratch tile: N rows of 2N
-  // one height per blockIdx.y
-  src += (size_t)blockIdx.y * ncls * ntrip * rowlen;
-  const size_t zt = (size_t)blockIdx.y * ncls * (ngrp + ntrip) * N * ld;
-  if (split == 2) dst = reinterpret_cast<T*>(reinterpret_cast<__nv_bfloat16*>(dst) + zt);
-  else dst += zt;
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // (c, n*2N + k)
-  if (idx >= (long long)ncls * rowlen) return;
-  const int c = (int)(idx / rowlen);
-  const int e = (int)(idx - (long long)c * rowlen);
-  const int n = e / (2 * N), kk = e - n * 2 * N;
-  const size_t o = tile_off(n, kk, N, ld, tiled != 0);
-  const size_t tsz = (size_t)N * ld;
-  double mean[2] = {0.0, 0.0};
-  int cnt[2] = {0, 0};
-  for (int t = 0; t < ntrip; ++t) {
-    const int g = grp[t];
-    mean[g] += src[((size_t)c * ntrip + t) * rowlen + e];
-    cnt[g] += 1;
+__global__ void __launch_bounds__(kSplitThreads) group_split_kernel(const double* __restrict__ src, T* __restrict__ dst,
+                                                                    float* __restrict__ tsc, const int* __restrict__ grp,
+                                                                    int ncls, int ntrip, int ngrp, int N, int ld,
+                                                                    int tiled, int fmt) {
+  const int n = blockIdx.x, c = blockIdx.y, z = blockIdx.z, nti = ngrp + ntrip;
+  const size_t rowlen = (size_t)2 * N * N;             // one FP64 scratch tile: N rows of 2N
+  src += ((size_t)z * ncls + c) * ntrip * rowlen + (size_t)n * 2 * N;
+  const size_t tsz = (size_t)N * ld;                   // elements of one stored tile
+  const size_t t0 = ((size_t)z * ncls + c) * nti;
+  auto means = [&](int k, double (&mean)[2]) {
+    int cnt[2] = {0, 0};
+    mean[0] = mean[1] = 0.0;
+    for (int t = 0; t < ntrip; ++t) {
+      const int g = grp[t];
+      mean[g] += src[t * rowlen + k];
+      cnt[g] += 1;
+    }
+    for (int g = 0; g < ngrp; ++g) mean[g] = cnt[g] ? mean[g] / cnt[g] : 0.0;
+  };
+  double scale = 1.0;
+  if (fmt == TILE_FP16) {
+    double m = 0.0, mean[2];
+    for (int k = threadIdx.x; k < 2 * N; k += kSplitThreads) {
+      means(k, mean);
+      for (int g = 0; g < ngrp; ++g) m = fmax(m, fabs(mean[g]));
+      for (int t = 0; t < ntrip; ++t) m = fmax(m, fabs(src[t * rowlen + k] - mean[grp[t]]));
+    }
+    __shared__ double red[kSplitThreads / 32];
+    for (int x = 16; x > 0; x >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, x));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = red[0];
+    for (int w = 1; w < kSplitThreads / 32; ++w) m = fmax(m, red[w]);
+    // exponent kept where the scale and its inverse are normal FP32 numbers
+    const int e = (m > 0.0 && m < 1e300) ? min(120, max(-120, 13 - ilogb(m))) : 0;
+    scale = ldexp(1.0, e);
+    if (threadIdx.x == 0) tsc[((size_t)z * ncls + c) * N + n] = (float)ldexp(1.0, -e);
   }
-  for (int g = 0; g < ngrp; ++g) mean[g] = cnt[g] ? mean[g] / cnt[g] : 0.0;
-  if (split == 2) {
-    __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(dst);
-    const size_t oh = tile_off_hi(n, kk, N, ld);
-    for (int g = 0; g < ngrp; ++g) h[((size_t)c * (ngrp + ntrip) + g) * tsz + oh] = __float2bfloat16_rn((float)mean[g]);
-    for (int t = 0; t < ntrip; ++t)
-      h[((size_t)c * (ngrp + ntrip) + ngrp + t) * tsz + oh] =
-          __float2bfloat16_rn((float)(src[((size_t)c * ntrip + t) * rowlen + e] - mean[grp[t]]));
-    return;
+  auto store = [&](int ti, int k, double v) {
+    if (fmt == TILE_PLAIN) {
+      dst[(t0 + ti) * tsz + tile_off(n, k, N, ld, tiled != 0)] = (T)v;
+    } else if (fmt == TILE_FP16) {
+      __half* t = reinterpret_cast<__half*>(dst) + (t0 + ti) * tsz * 2;
+      const double w = v * scale;
+      const __half hi = __float2half_rn((float)w);
+      t[tile_off_split(n, k, N, ld, false)] = hi;
+      t[tile_off_split(n, k, N, ld, true)] = __float2half_rn((float)(w - (double)__half2float(hi)));
+    } else if (fmt == TILE_BF16) {
+      __nv_bfloat16* t = reinterpret_cast<__nv_bfloat16*>(dst) + (t0 + ti) * tsz * 2;
+      const float w = (float)v;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+      t[tile_off_split(n, k, N, ld, false)] = hi;
+      t[tile_off_split(n, k, N, ld, true)] = __float2bfloat16_rn(w - __bfloat162float(hi));
+    } else {
+      reinterpret_cast<__nv_bfloat16*>(dst)[(t0 + ti) * tsz + tile_off_hi(n, k, N, ld)] = __float2bfloat16_rn((float)v);
+    }
+  };
+  for (int k = threadIdx.x; k < 2 * N; k += kSplitThreads) {
+    double mean[2];
+    means(k, mean);
+    for (int g = 0; g < ngrp; ++g) store(g, k, mean[g]);
+    for (int t = 0; t < ntrip; ++t) store(ngrp + t, k, src[t * rowlen + k] - mean[grp[t]]);
   }
-  if (split) {
-    // split layout (BF16x3 contexts): T is float, each tile's bytes hold the two bf16 planes
-    for (int g = 0; g < ngrp; ++g)
-      store_split(reinterpret_cast<__nv_bfloat16*>(dst + ((size_t)c * (ngrp + ntrip) + g) * tsz), n, kk, N, ld,
-                  (float)mean[g]);
-    for (int t = 0; t < ntrip; ++t)
-      store_split(reinterpret_cast<__nv_bfloat16*>(dst + ((size_t)c * (ngrp + ntrip) + ngrp + t) * tsz), n, kk, N, ld,
-                  (float)(src[((size_t)c * ntrip + t) * rowlen + e] - mean[grp[t]]));
-    return;
-  }
-  for (int g = 0; g < ngrp; ++g) dst[((size_t)c * (ngrp + ntrip) + g) * tsz + o] = (T)mean[g];
-  for (int t = 0; t < ntrip; ++t)
-    dst[((size_t)c * (ngrp + ntrip) + ngrp + t) * tsz + o] =
-        (T)(src[((size_t)c * ntrip + t) * rowlen + e] - mean[grp[t]]);
 }
 
 // -------------------------------------------------------------- launchers
@@ -640,9 +656,9 @@ struct TileGen {
   }
   // Stored tiles (group means, then deviations) of the heights z0 .. z0 + n - 1 from their rows in scr
   template <typename T>
-  int split(Ctx* c, int n, T* dst, int ld, int tiled, int how) {
-    group_split_kernel<T><<<dim3(ceil_div((long long)p.ncls * 2 * p.N * p.N, 256), n), 256, 0, c->stream>>>(
-        (const double*)scr.p, dst, (const int*)grp.p, p.ncls, p.ntrip, c->ngrp, p.N, ld, tiled, how);
+  int split(Ctx* c, int n, T* dst, int ld, int tiled, int fmt, float* tsc = nullptr) {
+    group_split_kernel<T><<<dim3(p.N, p.ncls, n), kSplitThreads, 0, c->stream>>>(
+        (const double*)scr.p, dst, tsc, (const int*)grp.p, p.ncls, p.ntrip, c->ngrp, p.N, ld, tiled, fmt);
     PRD_CUDA_TRY(c, cudaPeekAtLastError());
     return PRD_OK;
   }
@@ -677,13 +693,13 @@ int launch_tiles(Ctx* c) {
     // their group mean, so their errors must be far below the storage epsilon
     if ((rc = g.rows(c, z0, n, (double*)g.scr.p))) break;
     if (c->prec == PRD_FP64) {
-      rc = g.split<double>(c, n, (double*)c->tiles.p + z0 * ztile, c->ld(), c->tiled(), 0);
+      rc = g.split<double>(c, n, (double*)c->tiles.p + z0 * ztile, c->ld(), c->tiled(), TILE_PLAIN);
     } else {
-      rc = g.split<float>(c, n, (float*)((char*)c->tiles.p + z0 * ztile * c->tile_esz()), c->ld(), c->tiled(),
-                          c->hi_only ? 2 : (c->split_tiles ? 1 : 0));
+      rc = g.split<float>(c, n, (float*)((char*)c->tiles.p + z0 * ztile * c->tile_esz()), c->ld(), 1, c->tile_fmt(),
+                          c->tile_scale.p ? (float*)c->tile_scale.p + (size_t)z0 * c->ncls * N : nullptr);
       if (!rc && c->has64)
         rc = g.split<double>(c, n, (double*)c->tiles64.p + (size_t)z0 * c->ncls * c->ntile() * N * c->ld64(), c->ld64(),
-                             0, 0);
+                             0, TILE_PLAIN);
     }
   }
   if (!rc) {
@@ -730,8 +746,8 @@ int los_tiles_angles(Ctx* c, LosTiles* t, const std::vector<double>& thetas) {
 int los_tiles_gen(Ctx* c, LosTiles* t, int z0, int n, void* out) {
   int rc = t->g.rows(c, z0, n, (double*)t->g.scr.p);
   if (rc) return rc;
-  return c->prec == PRD_FP64 ? t->g.split<double>(c, n, (double*)out, c->ld(), c->tiled(), 0)
-                             : t->g.split<float>(c, n, (float*)out, c->ld(), c->tiled(), 0);
+  return c->prec == PRD_FP64 ? t->g.split<double>(c, n, (double*)out, c->ld(), c->tiled(), TILE_PLAIN)
+                             : t->g.split<float>(c, n, (float*)out, c->ld(), c->tiled(), TILE_PLAIN);
 }
 
 // Angle-averaged tiles and R_III incident weights of the unmagnetised J-level

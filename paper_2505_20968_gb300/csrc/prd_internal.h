@@ -33,6 +33,8 @@ constexpr int kAAThetaNodes = 48;
 // e1[r] (y_{r+2} - y_{r+1}) - e0[r] (y_{r+1} - y_r), forward g_r = rhs_r - cg[r] g_{r-1},
 // backward M_{r+1} = g_r - cp[r] M_{r+2}; the reciprocal pivots, and 6/h.
 enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpIden = 7, kSp6h = 8, kSpTabs = 9 };
+// Storage of the context's R_II tiles (kernels_tiles.cu, group_split_kernel)
+enum TileFmt { TILE_PLAIN = 0, TILE_FP16 = 1, TILE_BF16 = 2, TILE_BF16HI = 3 };
 // dynamic shared memory a CTA may have (opt-in limit of the device)
 constexpr int kMaxSmem = 227 * 1024;
 
@@ -118,7 +120,8 @@ struct Ctx {
   int test_zero_op = 0;        // GMRES iterates with the zero map (failure injection for tests)
   double refine_floor = 3e-5;  // FP32 refinement: floor of the inner GMRES relative tolerance
   int ld64() const { return (2 * nnu + 3) / 4 * 4; }
-  DBuf tiles;        // [z][c][t][n][2N]    (T)
+  DBuf tiles;        // [z][c][t][n][2N], format tile_fmt()
+  DBuf tile_scale;   // [z][c][n] power-of-two scale to undo (float; TILE_FP16 only)
   DBuf Y;            // [z][pair][t][16]    complex (T2)
   DBuf r3w;          // [z][q3][N] complex  (T2)  R_III incident weights
   DBuf r3in;         // [z][o'][q3][4] complex: w_o' * I_j(o'; ku, kv, kl)
@@ -182,14 +185,17 @@ struct Ctx {
   void* alloc_user = nullptr;
   // tensor-core contraction (r2_tc.cu)
   DBuf tc_err;
-  DBuf tc_work;      // tcgen05 contraction work items: (class, first output entry) pairs
+  DBuf tc_work;      // tcgen05 contraction work records (r2_tc.cu)
   int tc_nwork = 0;
   bool tc_ready = false;
   int use_tc = 0;
   long long tc_spin = 0;   // poll limit of the contraction's pipeline waits (0: the default)
-  int tc_bf16 = 0;         // contraction products: 0 3xTF32, 1 split-BF16 (BF16x3)
+  int tc_bf16 = 0;         // contraction products: 0 split-FP16, 1 split-BF16 (BF16x3)
   bool split_tiles = false;   // PRD_FP32_BF16X3/X2: R_II tiles stored as bf16 planes (tile_off_split)
   bool hi_only = false;       // PRD_FP32_BF16X2: the hi plane only (tile_off_hi), two products
+  int tile_fmt() const {
+    return prec == PRD_FP64 ? TILE_PLAIN : (hi_only ? TILE_BF16HI : (split_tiles ? TILE_BF16 : TILE_FP16));
+  }
   // bytes of one stored tile element (tile_bytes / elements of the padded layout)
   size_t tile_esz() const { return hi_only ? 2 : esz; }
   int tc_stages = 0;       // tile ring depth of the contraction (0: the deepest that fits)
