@@ -22,16 +22,22 @@
 // of that below, leaving <= 3 * 2^-24 a product.  TF32 products left 3 * 2^-22 at half the
 // rate.  BF16 contexts use bf16 planes, unscaled.
 //
-// Roles (320 threads): warp 0 streams the tile into a ring of K steps with two bulk
-// asynchronous copies each (the planes are stored pre-swizzled, step by step) and owns the
-// TMEM allocation; warp 1 issues tcgen05.mma; warps 2-9 stage I~ and Y and apply Y.  TMEM:
+// Roles (640 threads): warp 0 streams the tile into a ring of K step pairs with two bulk
+// asynchronous copies a step (the planes are stored pre-swizzled, step by step) and owns the
+// TMEM allocation; warp 1 issues tcgen05.mma; warps 4-19 stage I~ and Y and apply Y.  TMEM:
 // [half][row block of 128][128 columns (o', j)], so the products of one half run
 // while Y is applied to the other.  Every mbarrier wait is bounded; on expiry the CTA
 // records an error flag, drains what it issued and returns.
 //
-// Measured (operator apply, FP32): Mg II 8 heights x 64 directions x 200 frequencies
-// 2952 -> 1693 us, H I 4 x 96 x 150 2680 -> 1423 us, H I angle-averaged 8 x 64 x 91
-// 12480 -> 690 us, Mg II 10 x 16 x 27 201 -> 161 us; BF16x3, Mg II 4 x 64 x 163, 1313 -> 918 us.
+// What shaped it, in turn (contraction of Mg II 8 heights x 64 directions x 200 frequencies):
+// the products' order above 2795 -> 1515 us; products issued by an elected lane of a uniform
+// warp 1200; K steps in pairs and 16 Y warps of 8 entries each instead of 8 of 16 1100; bare
+// poll loops in the products' warp 967.  HBM alone takes 722, the copies without products
+// 804, the products without copies or Y about 800 (shared memory feeds them at 100 bytes a
+// clock); the rest is their overlap, the operand's build (7 us a CTA) and a last wave.
+// Measured (operator apply, FP32, start -> now): that problem 3394 -> 1132 us, H I 4 x 96 x 150
+// 2680 -> 938, H I angle-averaged 8 x 64 x 91 12722 -> 400, Mg II 10 x 16 x 27 263 -> 79;
+// BF16x3, Mg II 4 x 64 x 163, 1314 -> 552 us.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
@@ -46,26 +52,37 @@ namespace tc {
 
 constexpr int kStagesMax = 8;                 // tile ring depth: 2..8, the most that fit beside the rest
 constexpr int kKC = 16;                       // columns of a K step (32-byte rows per plane)
+constexpr int kSteps = 2;                     // K steps per stage: a stage's waits and commits cost the
+                                              // issuing warps some 300 clocks, a step's products 400
 constexpr int kMaxE = 32;                     // output entries per CTA
 constexpr int kMaxIn = 32;                    // incident directions per CTA (128 operand rows)
 constexpr int kPlane = 4 * kMaxIn * 32;       // bytes of one K step of one I~ plane
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;
+constexpr int kEV = kMaxE / (kEpiWarps / 4);   // entries of a Y warp (4 warps share a lane quarter)
 constexpr int kEpi = 32 * kEpiWarps;          // threads of the Y warps
-constexpr int kThreads = 64 + kEpi;
+constexpr int kThreads = 128 + kEpi;          // warps 0, 1: copies, products (2, 3 fill their warpgroup)
+// registers a thread: launched with 96, the first warpgroup gives up what the Y warps'
+// accumulators need (128 * 32 + 512 * 112 = 640 * 96)
+constexpr int kRegsFew = 32, kRegsMany = 112;
 constexpr int kYS = 36;                       // floats of a staged pair: Re [j][i], -Im [j][i], 4 of padding (banks)
 constexpr int kYBytes = 2 * kMaxE * kYS * 4;  // one tile's Y (two buffers)
 constexpr int kRec = 4 + 32 + 32 + 64 + 32;   // ints of a work record
 constexpr int kAuxBytes = 2048;               // work record, column scales, barriers, TMEM slot, abort flag
 __host__ __device__ constexpr int rows16(int N) { return (N + 15) / 16 * 16; }
-__host__ __device__ constexpr int stage_bytes(int N, bool hi) { return rows16(N) * (hi ? 32 : 64); }
+// Tiles per pass: up to 64 (32) rows, two (four) tiles share the 128 accumulator rows, each
+// with its own lane quarters and Y, so a small tile does not leave most of a product
+// and of the Y warps idle.
+__host__ __device__ constexpr int tiles_per_pass(int N) { return N <= 32 ? 4 : (N <= 64 ? 2 : 1); }
+__host__ __device__ constexpr int plane_bytes(int N) { return (N <= 64 ? 128 : rows16(N)) * 32; }
+__host__ __device__ constexpr int step_bytes(int N, bool hi) { return plane_bytes(N) * (hi ? 1 : 2); }
 // Shared memory of one CTA: the tile ring, the resident I~ operand (two planes), two Y
 // buffers, the auxiliary tables, 1 KB to align the base.  The second row block of a
 // tile plane reads past its rows (into what follows: rows nobody uses), so the
 // operand stands behind the ring.
 __host__ __device__ constexpr int smem_bytes(int N, int st, bool hi) {
-  return st * stage_bytes(N, hi) + rows16(N) / kKC * 2 * kPlane + 2 * kYBytes + kAuxBytes + 1024;
+  return st * kSteps * step_bytes(N, hi) + rows16(N) / kKC * 2 * kPlane + 2 * tiles_per_pass(N) * kYBytes + kAuxBytes + 1024;
 }
-constexpr long long kSpin = 1ll << 24;        // bounded waits (default limit of the pipeline waits; drains)
+constexpr int kSpin = 1 << 24;                // bounded waits (default limit of the pipeline waits; drains)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -89,15 +106,32 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// the same without the suspension of try_wait
+__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\tmbarrier.test_wait.parity.shared::cta.b64 P, [%1], %2;\n\tselp.b32 %0, 1, 0, P;\n\t}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // bounded pipeline wait of at most `limit` polls; returns false (and raises the
-// CTA abort flag) on expiry or when another role has aborted
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, long long limit) {
-  for (long long i = 0; i < limit; ++i) {
-    if (mbar_try(b, parity)) return true;
-    if (*abort_flag) return false;
+// CTA abort flag) on expiry or when another role has aborted, which it looks at
+// between bursts of polls
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, int limit) {
+  bool r = mbar_try(b, parity);
+  for (int n = 1; !r && n < limit && !*abort_flag;) {
+    const int m = min(n + 64, limit);
+    for (; n < m && !r; ++n) r = mbar_try(b, parity);
   }
-  *abort_flag = 1;
-  return false;
+  if (!r) *abort_flag = 1;
+  return r;
+}
+// the same by a converged warp
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag, int limit) {
+  const bool r = mbar_wait(b, parity, abort_flag, limit);
+  return __all_sync(0xffffffffu, r);
 }
 
 // bulk asynchronous copy global -> shared (16-byte aligned ends, size a multiple
@@ -160,6 +194,13 @@ __device__ __forceinline__ void split4(float4 v, uint2& hi, uint2& lo) {
   }
 }
 
+// one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+  return r != 0;
+}
+
 struct Params {
   const unsigned char* tiles;   // [z][class][tile] pre-swizzled K steps of [plane][N][16]
   const float* tsc;     // [z][class][N] power-of-two scale to undo per tile row (NULL: none)
@@ -171,7 +212,7 @@ struct Params {
   int* err;
   int ncls, ntile, nO, N, npairs, ld;
   int nst;              // tile stages
-  long long spin;       // poll limit of the pipeline waits (the drains keep kSpin)
+  int spin;             // poll limit of the pipeline waits (the drains keep kSpin)
 };
 
 // barrier over the Y warps only (named barrier 1), returning whether v holds on all of
@@ -194,29 +235,30 @@ __device__ __forceinline__ void tmem_ld4(float (&w)[4], uint32_t addr) {
 }
 template <int K>
 __device__ __forceinline__ void tmem_wait(float (&w)[K][4]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;");
   // the values pass through here, so that no use of them moves above the wait
 #pragma unroll
   for (int k = 0; k < K; ++k) asm volatile("" : "+f"(w[k][0]), "+f"(w[k][1]), "+f"(w[k][2]), "+f"(w[k][3]));
 }
 
-// NB: row blocks of 128 (N <= 128: 1, else 2).  BF: bf16 planes, else scaled FP16.  HI: the
+// NB: row blocks of 128 (N <= 128: 1, else 2).  G: tiles per pass (1, or 2 or 4 where N is
+// small).  BF: bf16 planes, else scaled FP16.  HI: the
 // tiles hold the hi plane alone (BF16x2: products hi hi + hi lo(I~)).  CONV: FP16 tiles
 // contracted with bf16 products (PRD_OPT_CONTRACTION): warp 1 re-splits each landed step
 // in place before its products.
-template <int NB, bool BF, bool HI, bool CONV>
+template <int NB, int G, bool BF, bool HI, bool CONV>
 __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   // 1024-byte aligned base, derived by offset so that the compiler keeps the
   // shared address space on every pointer below (plain LDS/STS, no generic access)
   unsigned char* sm = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);
   const int N = p.N, nst = p.nst;
-  const int SA = stage_bytes(N, HI);             // one K step of the tile
-  const int PA = rows16(N) * 32;                 // one plane of it
+  const int SA = step_bytes(N, HI);              // one K step of the tile
+  const int PA = plane_bytes(N);                 // one plane of it (of the pass's G tiles)
   const int KCH = p.ld / kKC, KH = KCH >> 1;     // K steps per tile and per half
-  unsigned char* Iop = sm + nst * SA;            // [K step][hi | lo][128 rows][32 bytes]
-  float* Ys = (float*)(Iop + KH * 2 * kPlane);   // [buffer][entry][pair][kYS]
-  int* rec = (int*)((unsigned char*)Ys + 2 * kYBytes);
+  unsigned char* Iop = sm + nst * kSteps * SA;   // [K step][hi | lo][128 rows][32 bytes]
+  float* Ys = (float*)(Iop + KH * 2 * kPlane);   // [buffer][tile of the pass][entry][pair][kYS]
+  int* rec = (int*)((unsigned char*)Ys + 2 * G * kYBytes);
   float* colinv = (float*)(rec + kRec);          // scale to undo per operand row (o', j)
   uint64_t* full = (uint64_t*)(((uintptr_t)(colinv + 4 * kMaxIn) + 7) & ~(uintptr_t)7);
   uint64_t* empty = full + kStagesMax;
@@ -228,8 +270,8 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int iz = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int et = threadIdx.x - 64;               // index among the Y threads
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // uniform
+  const int et = threadIdx.x - 128;              // index among the Y threads
   constexpr uint32_t tm_cols = NB * 256u;
   // tiles of this CTA (grid.z splits them where there are too few work items)
   const int t0 = p.ntile * (int)blockIdx.z / (int)gridDim.z, t1 = p.ntile * ((int)blockIdx.z + 1) / (int)gridDim.z;
@@ -242,9 +284,9 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
     }
     for (int h = 0; h < 2; ++h) {
       mbar_init(&accfull[h], 1);
-      mbar_init(&accfree[h], kEpi);
+      mbar_init(&accfree[h], kEpiWarps);   // one arrival a warp
     }
-    mbar_init(iready, kEpi);
+    mbar_init(iready, kEpiWarps);
     mbar_init(done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -263,111 +305,171 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   const int* vinfo = rec + 36;
   const int* vpair = rec + 68;
   const int* sdir = rec + 132;
-  const int iters = (t1 - t0) * KCH;
+  const int passes = (t1 - t0 + G - 1) / G, iters = passes * KH;   // stages of kSteps = 2 steps
 
-  if (warp == 0) {
-    // ---------------- producer: lane 0 waits for a free stage, arms its barrier with the
-    // bytes of the step and copies the planes, up to nst steps ahead of the products
-    if (lane == 0) {
-      int it = 0;
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
+    if (warp == 0) {
+      // ---------------- producer: the warp waits for a free stage and arms its barrier with the
+      // bytes of the copies, then each lane issues its one (plane, step, tile of the pass), up
+      // to nst stages ahead of the products
       const uint64_t pol_t = policy_evict_first();
-      const uint32_t pbytes = (uint32_t)N * 32;   // one plane of a step
+      const uint32_t pbytes = (uint32_t)N * 32;     // one plane of a step
       const size_t sbytes = (size_t)pbytes * (HI ? 1 : 2);
-      const unsigned char* src = p.tiles + (((size_t)iz * p.ncls + c) * p.ntile + t0) * KCH * sbytes;
-      int s = 0, ps = 0;                          // it % nst and (it / nst) & 1
-      for (; it < iters; ++it, src += sbytes, s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1) {
-        if (it >= nst && !mbar_wait(&empty[s], ps ^ 1, abort_flag, p.spin)) break;
-        // rows n >= N of the stage keep stale data: they only reach accumulator rows
-        // that nobody reads
-        mbar_expect_tx(&full[s], (uint32_t)sbytes);
-        bulk_load(sm + s * SA, src, pbytes, &full[s], pol_t);
-        if constexpr (!HI) bulk_load(sm + s * SA + PA, src + pbytes, pbytes, &full[s], pol_t);
+      const int pl = lane & 1, c2 = (lane >> 1) & 1, g = lane >> 2;
+      const unsigned char* src = p.tiles + (((size_t)iz * p.ncls + c) * p.ntile + t0 + g) * KCH * sbytes + c2 * sbytes + pl * pbytes;
+      unsigned char* dst = sm + c2 * SA + pl * PA + g * (4096 / G);
+      int it = 0, s = 0, ps = 0, j = 0, left = t1 - t0;   // it % nst and (it / nst) & 1; step pair; tiles left
+      for (; it < iters; ++it, s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1) {
+        if (it >= nst && !mbar_wait_warp(&empty[s], ps ^ 1, abort_flag, p.spin)) break;
+        // rows n >= N of the stage (and the places of a last pass's missing tiles) keep stale
+        // data: they only reach accumulator rows that nobody reads
+        const int g1 = min(G, left);
+        if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(kSteps * sbytes) * g1);
+        __syncwarp();
+        if (g < g1 && (!HI || pl == 0)) bulk_load(dst + s * kSteps * SA, src, pbytes, &full[s], pol_t);
+        src += kSteps * sbytes;
+        if (++j == KH) {
+          j = 0;
+          left -= G;
+          src += (size_t)(G - 1) * KCH * sbytes;
+        }
       }
+      __syncwarp();
       if (*abort_flag) {
         // drain copies that were issued and may not have been consumed
-        for (int j = max(0, it - nst); j < it; ++j)
-          for (long long i = 0; i < kSpin && !mbar_try(&full[j % nst], (j / nst) & 1); ++i) {
+        for (int k = max(0, it - nst); k < it; ++k)
+          for (int i = 0; i < kSpin && !mbar_try(&full[k % nst], (k / nst) & 1); ++i) {
           }
       }
-    }
-  } else if (warp == 1) {
-    // ---------------- products.  CONV: the whole warp re-splits a step first, so every lane
-    // takes part in the waits; otherwise lane 0 alone.
-    if (CONV || lane == 0) {
+    } else if (warp == 1) {
+      // ---------------- products: the warp runs uniformly (waits by all lanes, descriptors in
+      // uniform registers) and an elected lane issues; a loop of one lane issued a product
+      // every 160 clocks, three times what it takes to execute
       const uint32_t ty = BF ? 1u : 0u;
       const uint32_t idesc = (1u << 4) | (ty << 7) | (ty << 10) | ((uint32_t)(rows16(4 * ns) >> 3) << 17) | ((128u >> 4) << 24);
+      const uint64_t a0 = sdesc32(sm), b0 = sdesc32(Iop);    // the address field counts 16 bytes
+      // A stage's waits are kept to a bare poll loop, without a vote on their outcome or a look
+      // at the abort flag (either cost 100 to 200 clocks a stage in this warp of few
+      // registers): a wait that gives up raises the flag and makes the waits after it one poll
+      // each, so the products to the end of the tile go to an accumulator nobody reads any
+      // more; the flag ends the loop at the next tile.
+      int lim = p.spin;
       auto wait = [&](uint64_t* b, uint32_t par) {
-        const bool r = mbar_wait(b, par, abort_flag, p.spin);
-        return CONV ? (bool)__all_sync(0xffffffffu, r) : r;
+        bool r = false;
+        for (int i = 0; i < lim && !r; ++i) r = mbar_try(b, par);
+        if (!r) {
+          *abort_flag = 1;
+          lim = 1;
+        }
+        __syncwarp();
       };
-      bool ok = wait(iready, 0);
+      {
+        // I~ takes microseconds to build: plain polls, so that a short poll limit expires here
+        bool r = false;
+        for (int i = 0; i < lim && !r; ++i) r = mbar_test(iready, 0);
+        if (!r) {
+          *abort_flag = 1;
+          lim = 1;
+        }
+        __syncwarp();
+      }
       int s = 0, ps = 0;
       bool issued = false;
-      for (int t = 0; t < t1 - t0 && ok; ++t)
-        for (int h = 0; h < 2 && ok; ++h) {
-          if (t > 0) ok = wait(&accfree[h], (t - 1) & 1);
-          for (int kc = 0; kc < KH && ok; ++kc) {
-            ok = wait(&full[s], ps);
-            if (!ok) break;
-            unsigned char* A = sm + s * SA;
-            if constexpr (CONV) {
-              for (int i = lane; i < PA / 16; i += 32) {
-                uint4 h4 = reinterpret_cast<uint4*>(A)[i], l4 = reinterpret_cast<uint4*>(A + PA)[i];
-                uint32_t* hp = &h4.x;
-                uint32_t* lp = &l4.x;
+      for (int t = 0; t < passes; ++t) {
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+        int h = 0, kc = 0;                           // half and K step within it
+        for (int j = 0; j < KH; ++j) {
+          wait(&full[s], ps);
+          // a half's accumulators are free once Y has been applied to the pass before
+          if (t > 0 && kc == 0) wait(&accfree[h], (t - 1) & 1);
+          if (t > 0 && kc + 1 == KH && h == 0) wait(&accfree[1], (t - 1) & 1);
+          if constexpr (CONV) {
+            for (int i = lane; i < kSteps * (PA / 16); i += 32) {
+              unsigned char* A = sm + s * kSteps * SA + (i >= PA / 16 ? SA : 0);
+              const int e = i >= PA / 16 ? i - PA / 16 : i;
+              uint4 h4 = reinterpret_cast<uint4*>(A)[e], l4 = reinterpret_cast<uint4*>(A + PA)[e];
+              uint32_t* hp = &h4.x;
+              uint32_t* lp = &l4.x;
 #pragma unroll
-                for (int q = 0; q < 4; q += 2) {
-                  const float2 a = __half22float2(*reinterpret_cast<__half2*>(hp + q)), b = __half22float2(*reinterpret_cast<__half2*>(lp + q));
-                  const float2 e = __half22float2(*reinterpret_cast<__half2*>(hp + q + 1)), f = __half22float2(*reinterpret_cast<__half2*>(lp + q + 1));
-                  uint2 hi, lo;
-                  split4<true>(make_float4(a.x + b.x, a.y + b.y, e.x + f.x, e.y + f.y), hi, lo);
-                  hp[q] = hi.x; hp[q + 1] = hi.y;
-                  lp[q] = lo.x; lp[q + 1] = lo.y;
-                }
-                reinterpret_cast<uint4*>(A)[i] = h4;
-                reinterpret_cast<uint4*>(A + PA)[i] = l4;
+              for (int q = 0; q < 4; q += 2) {
+                const float2 a = __half22float2(*reinterpret_cast<__half2*>(hp + q)), b = __half22float2(*reinterpret_cast<__half2*>(lp + q));
+                const float2 x = __half22float2(*reinterpret_cast<__half2*>(hp + q + 1)), f = __half22float2(*reinterpret_cast<__half2*>(lp + q + 1));
+                uint2 hi, lo;
+                split4<true>(make_float4(a.x + b.x, a.y + b.y, x.x + f.x, x.y + f.y), hi, lo);
+                hp[q] = hi.x; hp[q + 1] = hi.y;
+                lp[q] = lo.x; lp[q + 1] = lo.y;
               }
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-              __syncwarp();
+              reinterpret_cast<uint4*>(A)[e] = h4;
+              reinterpret_cast<uint4*>(A + PA)[e] = l4;
             }
-            if (lane == 0) {
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              const uint64_t bh = sdesc32(Iop + kc * 2 * kPlane), bl = sdesc32(Iop + kc * 2 * kPlane + kPlane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+          }
+          if (kc == 0 || kc + 1 == KH)   // orders the products behind the Y warps' reads of the accumulators
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t as = a0 + (uint64_t)((uint32_t)(s * kSteps * SA) >> 4);
+          if (elect_one()) {
+            int h2 = h, k2 = kc;
+#pragma unroll
+            for (int u = 0; u < kSteps; ++u) {
+              const uint64_t ah = as + (uint64_t)((uint32_t)(u * SA) >> 4), al = ah + (uint64_t)((uint32_t)PA >> 4);
+              const uint64_t bh = b0 + (uint64_t)((uint32_t)(k2 * 2 * kPlane) >> 4), bl = bh + (kPlane >> 4);
 #pragma unroll
               for (int b = 0; b < NB; ++b) {
-                const uint32_t d = tmem + (uint32_t)(h * NB + b) * 128u;
-                const uint64_t ah = sdesc32(A + b * 4096);
-                mma_f16(d, ah, bh, idesc, kc > 0 ? 1u : 0u);
-                mma_f16(d, ah, bl, idesc, 1u);
-                if constexpr (!HI) mma_f16(d, sdesc32(A + PA + b * 4096), bh, idesc, 1u);
+                const uint32_t d = tmem + (uint32_t)(h2 * NB + b) * 128u;
+                mma_f16(d, ah + b * 256, bh, idesc, k2 > 0 ? 1u : 0u);
+                mma_f16(d, ah + b * 256, bl, idesc, 1u);
+                if constexpr (!HI) mma_f16(d, al + b * 256, bh, idesc, 1u);
               }
-              mma_commit(&empty[s]);
-              if (kc == KH - 1) mma_commit(&accfull[h]);
-              issued = true;
+              if (++k2 == KH) {
+                mma_commit(&accfull[h2]);
+                k2 = 0;
+                ++h2;
+              }
             }
-            s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1;
+            mma_commit(&empty[s]);
           }
+          kc += kSteps;
+          if (kc >= KH) { kc -= KH; ++h; }
+          issued = true;
+          s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1;
         }
+      }
       // every product issued completes before TMEM is released
-      if (lane == 0 && issued) {
-        mma_commit(done);
-        for (long long i = 0; i < kSpin && !mbar_try(done, 0); ++i) {
+      __syncwarp();
+      if (issued) {
+        if (elect_one()) mma_commit(done);
+        for (int i = 0; i < kSpin && !mbar_try(done, 0); ++i) {
         }
       }
     }
   } else {
     // ---------------- Y warps
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsMany));
     const int q = warp & 3;                        // TMEM lane quarter of this warp
-    const int og = (warp - 2) >> 2;                // entries of this warp: 2 i + og
+    const int og = (warp - 4) >> 2;                // entries of this warp: 4 i + og
     // Y of a tile: thread (pair slot, i) moves the 8 coefficients of output Stokes i
-    const int yp = et >> 2, yi = et & 3;           // pair slot 2 entry + pair, Stokes i
-    const int ypair = (yp >> 1) < E ? vpair[yp] : -1;
+    // (tiles of the pass are shared out between the two halves of the threads)
+    constexpr int GY = (G + 1) / 2;
+    const int yp = (et & 255) >> 2, yi = et & 3;   // pair slot 2 entry + pair, Stokes i
+    const int yg = et >> 8;                        // tiles yg, yg + 2 of the pass
+    const int ypair = (yp >> 1) < E && yg < G ? vpair[yp] : -1;
     const float4* ysrc = reinterpret_cast<const float4*>(p.Y + (((size_t)iz * p.npairs + max(ypair, 0)) * p.ntile + t0) * 32 + yi * 8);
-    float4 ya = make_float4(0.f, 0.f, 0.f, 0.f), yb = ya;
-    if (ypair >= 0) { ya = ysrc[0]; yb = ysrc[1]; }
+    float4 ya[GY], yb[GY];
+    auto load_y = [&](int t) {                     // Y of pass t's tiles
+#pragma unroll
+      for (int k = 0; k < GY; ++k) {
+        const int ti = t * G + yg + 2 * k;
+        if (ypair >= 0 && ti < t1 - t0) { ya[k] = ysrc[ti * 8]; yb[k] = ysrc[ti * 8 + 1]; }
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < GY; ++k) ya[k] = yb[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    load_y(0);
     // I~ operand: a warp per incident direction; the scale of each of its 4 rows brings
     // the largest element to [2^13, 2^14)
-    for (int sl = warp - 2; sl < ns; sl += kEpiWarps) {
+    for (int sl = warp - 4; sl < ns; sl += kEpiWarps) {
       const float4* src = reinterpret_cast<const float4*>(p.Ic) + ((size_t)iz * p.nO + sdir[sl]) * N;
       float sc[4] = {1.f, 1.f, 1.f, 1.f};
       if constexpr (!BF) {
@@ -408,7 +510,8 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive(iready);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(iready);
     bool ok = epi_all(true);                       // colinv is complete
 
     float ci[4] = {1.f, 1.f, 1.f, 1.f};            // column scales of this thread's Y
@@ -417,55 +520,51 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) ci[j] = colinv[sl * 4 + j];
     }
-    const bool live0 = q * 32 < N, live1 = NB > 1 && 128 + q * 32 < N;
-    float acc[16][NB][4];
+    // tile of the pass and row of this lane
+    const int gt = q * G / 4, n0 = (q % (4 / G)) * 32 + lane;
+    const bool live0 = (q % (4 / G)) * 32 < N, live1 = NB > 1 && 128 + q * 32 < N;
+    float acc[kEV][NB][4];
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
+    for (int i = 0; i < kEV; ++i)
 #pragma unroll
       for (int b = 0; b < NB; ++b)
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[i][b][k] = 0.f;
     const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-    for (int t = 0; t < t1 - t0; ++t) {
-      float* Yb = Ys + (t & 1) * (kYBytes / 4);
-      {
-        float* d = Yb + yp * kYS + yi;             // [half][j][i]
-        d[0] = ya.x * ci[0]; d[4] = ya.z * ci[1]; d[8] = yb.x * ci[2]; d[12] = yb.z * ci[3];
-        d[16] = -ya.y * ci[0]; d[20] = -ya.w * ci[1]; d[24] = -yb.y * ci[2]; d[28] = -yb.w * ci[3];
+    for (int t = 0; t < passes; ++t) {
+      float* Yb = Ys + (t & 1) * (G * kYBytes / 4);
+#pragma unroll
+      for (int k = 0; k < GY; ++k) {
+        const int g = yg + 2 * k;
+        if (g >= G) break;
+        float* d = Yb + g * (kYBytes / 4) + yp * kYS + yi;             // [half][j][i]
+        d[0] = ya[k].x * ci[0]; d[4] = ya[k].z * ci[1]; d[8] = yb[k].x * ci[2]; d[12] = yb[k].z * ci[3];
+        d[16] = -ya[k].y * ci[0]; d[20] = -ya[k].w * ci[1]; d[24] = -yb[k].y * ci[2]; d[28] = -yb[k].w * ci[3];
       }
       ok = epi_all(ok);
       if (!ok) break;
-      if (ypair >= 0 && t + 1 < t1 - t0) { ya = ysrc[(t + 1) * 8]; yb = ysrc[(t + 1) * 8 + 1]; }
+      if (t + 1 < passes) load_y(t + 1);
       for (int h = 0; h < 2 && ok; ++h) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&accfull[h], t & 1, abort_flag, p.spin));
+        ok = mbar_wait_warp(&accfull[h], t & 1, abort_flag, p.spin);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (live0) {
+        if (live0 && (G == 1 || t * G + gt < t1 - t0)) {
           const uint32_t ta = tq + (uint32_t)(h * NB) * 128u;
-          const float* Yh = Yb + h * 16;
-          // entry i + 1's columns are read while Y is applied to entry i's
-          float w[2][2 * NB][4];                   // [buffer][pair, row block]
-          auto load = [&](int i) {
-            const int v = 2 * i + og;
-            if (v >= E) return;
-            const int info = vinfo[v];
-            float(&x)[2 * NB][4] = w[i & 1];
-            tmem_ld4(x[0], ta + (uint32_t)(info & 255) * 4u);
-            if (NB > 1) tmem_ld4(x[NB - 1], ta + 128u + (uint32_t)(info & 255) * 4u);
-            if ((info >> 16) > 1) {
-              const uint32_t cb = (uint32_t)((info >> 8) & 255) * 4u;
-              tmem_ld4(x[NB], ta + cb);
-              if (NB > 1) tmem_ld4(x[2 * NB - 1], ta + 128u + cb);
-            }
-          };
-          load(0);
+          const float* Yh = Yb + gt * (kYBytes / 4) + h * 16;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int v = 2 * i + og;
+          for (int i = 0; i < kEV; ++i) {
+            const int v = 4 * i + og;
             if (v >= E) break;
-            tmem_wait<2 * NB>(w[i & 1]);
-            if (i + 1 < 16) load(i + 1);
-            const int np = vinfo[v] >> 16;
+            const int info = vinfo[v], np = info >> 16;
+            const uint32_t ca = ta + (uint32_t)(info & 255) * 4u, cb = ta + (uint32_t)((info >> 8) & 255) * 4u;
+            float w[2 * NB][4];                    // [pair, row block]
+#pragma unroll
+            for (int b = 0; b < NB; ++b) tmem_ld4(w[b], ca + b * 128u);
+            if (np > 1) {
+#pragma unroll
+              for (int b = 0; b < NB; ++b) tmem_ld4(w[NB + b], cb + b * 128u);
+            }
+            tmem_wait<2 * NB>(w);
 #pragma unroll
             for (int pr = 0; pr < 2; ++pr) {
               if (pr < np) {
@@ -475,8 +574,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
                   const float4 y = y4[j];
 #pragma unroll
                   for (int b = 0; b < NB; ++b) {
-                    if (b > 0 && !live1) continue;
-                    const float x = w[i & 1][pr * NB + b][j];
+                    const float x = w[pr * NB + b][j];
                     acc[i][b][0] += y.x * x;
                     acc[i][b][1] += y.y * x;
                     acc[i][b][2] += y.z * x;
@@ -488,18 +586,19 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(&accfree[h]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&accfree[h]);
       }
     }
     if (ok) {
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
-        const int n = b * 128 + q * 32 + lane;
-        if (n >= N) continue;
+        const int n = b * 128 + n0;
+        if (n >= N || (b > 0 && !live1)) continue;
         const float sc = p.tsc ? p.tsc[((size_t)iz * p.ncls + c) * N + n] : 1.f;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int v = 2 * i + og;
+        for (int i = 0; i < kEV; ++i) {
+          const int v = 4 * i + og;
           if (v < E) {
             float* dst = p.eb + (((size_t)iz * p.nO + vdir[v]) * N + n) * 4;
             asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(acc[i][b][0] * sc),
@@ -528,12 +627,21 @@ static int r2_tc_stages(int N, bool hi) {
   return 0;
 }
 
-template <int NB>
-static int r2_tc_attr(Ctx* c) {
-  for (auto k : {tc::r2_tc_kernel<NB, false, false, false>, tc::r2_tc_kernel<NB, true, false, false>,
-                 tc::r2_tc_kernel<NB, true, true, false>, tc::r2_tc_kernel<NB, true, false, true>})
-    PRD_CUDA_TRY(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-  return PRD_OK;
+// The kernel of a context's tile format and products for N rows.
+using R2Kernel = void (*)(tc::Params);
+template <int NB, int G>
+static R2Kernel r2_tc_pick(const Ctx* c) {
+  if (c->hi_only) return tc::r2_tc_kernel<NB, G, true, true, false>;
+  if (c->split_tiles) return tc::r2_tc_kernel<NB, G, true, false, false>;
+  if (c->tc_bf16) return tc::r2_tc_kernel<NB, G, true, false, true>;
+  return tc::r2_tc_kernel<NB, G, false, false, false>;
+}
+static R2Kernel r2_tc_pick(const Ctx* c) {
+  switch (tc::tiles_per_pass(c->nnu)) {
+    case 4: return r2_tc_pick<1, 4>(c);
+    case 2: return r2_tc_pick<1, 2>(c);
+    default: return c->nnu <= 128 ? r2_tc_pick<1, 1>(c) : r2_tc_pick<2, 1>(c);
+  }
 }
 
 // Work records of the contraction: every class's outputs cut into entries of at most two
@@ -614,7 +722,12 @@ int r2_tc_prepare(Ctx* c) {
   c->tc_nwork = (int)work.size() / tc::kRec;
   dfree(c->tc_work);
   int rc = dalloc(c, c->tc_work, work.size() * sizeof(int));
-  if (rc || (rc = r2_tc_attr<1>(c)) || (rc = r2_tc_attr<2>(c))) return rc;
+  if (rc) return rc;
+  const int bf16 = c->tc_bf16;
+  for (c->tc_bf16 = 0; c->tc_bf16 < 2; ++c->tc_bf16)   // the kernels PRD_OPT_CONTRACTION chooses from
+    if (cudaFuncSetAttribute(r2_tc_pick(c), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) rc = PRD_E_CUDA;
+  c->tc_bf16 = bf16;
+  if (rc) return fail(c, rc, "shared memory of the tensor-core contraction");
   PRD_CUDA_TRY(c, cudaMemcpy(c->tc_work.p, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice));
   PRD_CUDA_TRY(c, cudaMemset(c->tc_err.p, 0, sizeof(int)));
   c->tc_ready = true;
@@ -627,22 +740,14 @@ int r2_tc_launch(Ctx* c, const float* Ic, float* eb) {
   const int nst = c->tc_stages >= 2 ? std::min(c->tc_stages, nmax) : nmax;
   tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->tile_scale.p, (const float*)c->Y.p, Ic,
                (const int*)c->tc_work.p, eb, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu, c->npairs,
-               c->ld(), nst, c->tc_spin > 0 ? c->tc_spin : tc::kSpin};
+               c->ld(), nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
   const int smem = tc::smem_bytes(c->nnu, nst, c->hi_only);
   // fewer CTAs than SMs: split the tiles of a work item (at least 4 tiles each)
   const int items = c->tc_nwork * c->nz;
   const int zs = std::max(1, std::min(c->ntile() / 4, c->nsm / std::max(1, items)));
-  auto go = [&](auto k1, auto k2) -> int {
-    const dim3 g(c->tc_nwork, c->nz, zs);
-    if (c->nnu <= 128) k1<<<g, tc::kThreads, smem, c->stream>>>(p);
-    else k2<<<g, tc::kThreads, smem, c->stream>>>(p);
-    PRD_CUDA_TRY(c, cudaPeekAtLastError());
-    return PRD_OK;
-  };
-  if (c->hi_only) return go(tc::r2_tc_kernel<1, true, true, false>, tc::r2_tc_kernel<2, true, true, false>);
-  if (c->split_tiles) return go(tc::r2_tc_kernel<1, true, false, false>, tc::r2_tc_kernel<2, true, false, false>);
-  if (c->tc_bf16) return go(tc::r2_tc_kernel<1, true, false, true>, tc::r2_tc_kernel<2, true, false, true>);
-  return go(tc::r2_tc_kernel<1, false, false, false>, tc::r2_tc_kernel<2, false, false, false>);
+  r2_tc_pick(c)<<<dim3(c->tc_nwork, c->nz, zs), tc::kThreads, smem, c->stream>>>(p);
+  PRD_CUDA_TRY(c, cudaPeekAtLastError());
+  return PRD_OK;
 }
 
 int r2_tc_check_error(Ctx* c) {
