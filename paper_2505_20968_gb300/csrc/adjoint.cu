@@ -12,6 +12,7 @@
 // the forward Thomas solve.  In FP32 mode the adjoint reads the FP64 copy of the
 // Sigma tables, so it is the transpose of the operator whose solution
 // prd_solve returns.
+#include <algorithm>
 #include <cstdio>
 #include "prd_internal.h"
 #include "device_common.cuh"
@@ -101,70 +102,89 @@ __global__ void delo_t_kernel(const double* __restrict__ g, const T* __restrict_
 // Forward per row (z, Omega, s): M = T^-1 D y (natural spline, T symmetric
 // tridiagonal), then r(pt) = y_k + t (y_{k+1} - y_k) + c2 M_k + c3 M_{k+1}, with
 // constant extension outside the grid; the intensity row is scaled by fI.
-// Transpose: scatter gbar into ybar and Mbar, w = T^-1 Mbar, ybar += D^T w.
-// ybar and Mbar are per-row scratch rows in global memory.
-__global__ void spline_t_kernel(const double* __restrict__ gbar, const int* __restrict__ kidx,
-                                const double* __restrict__ tt, const double* __restrict__ sp,
-                                const double* __restrict__ fI, double* __restrict__ ybar, double* __restrict__ Mbar,
-                                int nz, int nO, int N) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;   // (z, o, s)
-  if (row >= nz * nO * 4) return;
-  const int s = row & 3, zo = row >> 2, iz = zo / nO;
-  const double* h = sp + (size_t)iz * kSpTabs * N;
-  const double* cp = h + kSpCp * N;
-  const double* den = h + kSpDen * N;
-  double* yb = ybar + (size_t)row * N;
-  double* mb = Mbar + (size_t)row * N;
-  for (int i = 0; i < N; ++i) { yb[i] = 0.0; mb[i] = 0.0; }
-  for (int n = 0; n < N; ++n) {
-    const size_t pt = (size_t)zo * N + n;
-    double gv = gbar[pt * 4 + s];
-    if (fI && s == 0) gv *= fI[pt];
-    const int k = kidx[pt];
-    if (k < 0) yb[0] += gv;
-    else if (k >= N - 1) yb[N - 1] += gv;
-    else {
-      const double t = tt[pt], omt = 1.0 - t;
-      const double hk = h[k], k6 = hk * hk / 6.0;
-      yb[k] += (1.0 - t) * gv;
-      yb[k + 1] += t * gv;
-      mb[k] += k6 * (omt * omt * omt - omt) * gv;
-      mb[k + 1] += k6 * (t * t * t - t) * gv;
+// Transpose: gather gbar into ybar and Mbar (the points of a row ascend, so the ones that
+// touch a node are a run of them), w = T^-1 Mbar, ybar += D^T w.
+// One (z, Omega) row per CTA, everything in shared memory, like the forward frame change and
+// for the same reason: the recurrence is one FP64 FMA a step, the rest is spread over the
+// CTA.  A thread per row walking global memory, dividing at each step, and a transposition of
+// its rows took 2 x 162 us for 6 x 16 rows of 48 points.
+constexpr int kStThreads = 128;
+static size_t spline_t_smem(int N) { return (size_t)N * (3 * 32 + 16 + 4) + 16; }
+__global__ void __launch_bounds__(kStThreads) spline_t_kernel(const double* __restrict__ gbar,
+                                                              const int* __restrict__ kidx,
+                                                              const double* __restrict__ tt,
+                                                              const double* __restrict__ sp,
+                                                              const double* __restrict__ fI, double* __restrict__ out,
+                                                              int nO, int N) {
+  extern __shared__ __align__(16) unsigned char stsm[];
+  double* gv = reinterpret_cast<double*>(stsm);        // [n][s] cotangents of the points
+  double* yb = gv + 4 * N;                             // [i][s]
+  double* mb = yb + 4 * N;                             // [i][s]
+  double* cm = mb + 4 * N;                             // [n][2] weights of M_k, M_{k+1}
+  int* ks = reinterpret_cast<int*>(cm + 2 * N);
+  const int zo = blockIdx.y * nO + blockIdx.x, tid = threadIdx.x;
+  const double* tab = sp + (size_t)blockIdx.y * kSpTabs * N;
+  const size_t p0 = (size_t)zo * N;
+  for (int i = tid; i < 4 * N; i += kStThreads) {
+    const double v = gbar[p0 * 4 + i];
+    gv[i] = (fI && (i & 3) == 0) ? v * fI[p0 + (i >> 2)] : v;
+  }
+  for (int n = tid; n < N; n += kStThreads) {
+    const int k = kidx[p0 + n];
+    ks[n] = k;
+    if (k >= 0 && k < N - 1) {
+      const double t = tt[p0 + n], omt = 1.0 - t, k6 = tab[kSpK6 * N + k];
+      cm[2 * n] = k6 * (omt * omt * omt - omt);
+      cm[2 * n + 1] = k6 * (t * t * t - t);
     }
   }
-  if (N <= 2) return;
-  // w = T^-1 Mbar on the interior nodes (M_0 = M_{N-1} = 0 are constants)
-  double gprev = 0.0;
-  for (int r = 0; r < N - 2; ++r) {
-    const int i = r + 1;
-    const double sub = (r > 0) ? h[i - 1] : 0.0;
-    const double gg = (mb[i] - sub * gprev) / den[r];
-    mb[i] = gg;
-    gprev = gg;
+  __syncthreads();
+  for (int q = tid; q < 4 * N; q += kStThreads) {
+    const int i = q >> 2, s = q & 3;
+    int lo = 0, hi = N;                                // first point with k >= i - 1
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (ks[mid] < i - 1) lo = mid + 1; else hi = mid;
+    }
+    double y = 0.0, m = 0.0;
+    for (int n = lo; n < N && ks[n] <= i; ++n) {
+      const int k = ks[n];
+      const double g = gv[n * 4 + s];
+      if (k < 0 || k >= N - 1) {                       // constant continuation: the end node alone
+        if (i == (k < 0 ? 0 : N - 1)) y += g;
+      } else {
+        const double t = tt[p0 + n];
+        y += (k == i ? 1.0 - t : t) * g;
+        m += (k == i ? cm[2 * n] : cm[2 * n + 1]) * g;
+      }
+    }
+    yb[q] = y;
+    mb[q] = (i > 0 && i < N - 1) ? m : 0.0;            // M_0 = M_{N-1} = 0 are constants
   }
-  double mnext = 0.0;
-  for (int r = N - 3; r >= 0; --r) {
-    const int i = r + 1;
-    const double m = mb[i] - cp[r] * mnext;
-    mb[i] = m;
-    mnext = m;
+  __syncthreads();
+  if (tid < 4) {
+    double prev = 0.0, next = 0.0;
+#pragma unroll 8
+    for (int i = 1; i < N - 1; ++i) {
+      prev = mb[i * 4 + tid] * tab[kSpIden * N + i - 1] - tab[kSpCg * N + i - 1] * prev;
+      mb[i * 4 + tid] = prev;
+    }
+#pragma unroll 8
+    for (int i = N - 2; i >= 1; --i) {
+      next = mb[i * 4 + tid] - tab[kSpCp * N + i - 1] * next;
+      mb[i * 4 + tid] = next;
+    }
   }
-  // ybar += D^T w,  (D y)_i = 6 [(y_{i+1} - y_i) / h_i - (y_i - y_{i-1}) / h_{i-1}]
-  for (int i = 1; i <= N - 2; ++i) {
-    const double w = 6.0 * mb[i];
-    yb[i + 1] += w / h[i];
-    yb[i] -= w * (1.0 / h[i] + 1.0 / h[i - 1]);
-    yb[i - 1] += w / h[i - 1];
+  __syncthreads();
+  // (D y)_i = 6 [(y_{i+1} - y_i) / h_i - (y_i - y_{i-1}) / h_{i-1}]
+  for (int q = tid; q < 4 * N; q += kStThreads) {
+    const int i = q >> 2;
+    const double sl = i > 0 ? tab[kSp6h * N + i - 1] : 0.0, sr = i < N - 1 ? tab[kSp6h * N + i] : 0.0;
+    double v = yb[q] - (sl + sr) * mb[q];
+    if (i > 0) v += sl * mb[q - 4];
+    if (i < N - 1) v += sr * mb[q + 4];
+    out[p0 * 4 + q] = v;
   }
-}
-
-// scratch rows [row][n] -> vector [z][o][n][s]
-__global__ void rows_to_vec_kernel(const double* __restrict__ rows, double* __restrict__ v, int nrows, int N) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // (row, n)
-  if (idx >= (long long)nrows * N) return;
-  const int row = (int)(idx / N), n = (int)(idx - (long long)row * N);
-  const int s = row & 3, zo = row >> 2;
-  v[((size_t)zo * N + n) * 4 + s] = rows[idx];
 }
 
 // ---------------------------------------------------------------- R_II^T
@@ -172,15 +192,18 @@ __global__ void rows_to_vec_kernel(const double* __restrict__ rows, double* __re
 //          Z[m][(e,i)] = sum_{pairs p of e} sum_j Y_p[i][j] I~[o'_p][m][j].
 // Transpose: Zr[m][(e,i)] = sum_n T_r[n][m] g[e][n][i],  Zi = -sum_n T_i[n][m] g[e][n][i],
 //            Ibar[o'][m][j] += sum_i (Y_r[i][j] Zr + Y_i[i][j] Zi).
-// Block per (chunk of kCE outputs, class, z); 16 incident frequencies m per pass.
+// Block per (part of the tiles, chunk of kCE outputs, class, z); 16 incident frequencies m per
+// pass.  FP64-bound; what cost more was uneven work: one block per chunk, most classes with
+// fewer outputs than a chunk, left SMs idle and lanes without a column.  Threads now take the
+// columns that exist, and the tiles are split between enough blocks to even the SMs out.
 constexpr int kCE = 8;
 constexpr int kMB2 = 16;
 
 __global__ void __launch_bounds__(256) r2_t_kernel(const double* __restrict__ tiles, const double* __restrict__ Y,
                                                    const double* __restrict__ g, const int* __restrict__ cls,
                                                    double* __restrict__ Ibar, int ncls, int ntile, int nO, int N,
-                                                   int npairs, int ld) {
-  const int chunk = blockIdx.x, c = blockIdx.y, iz = blockIdx.z;
+                                                   int npairs, int ld, int ts) {
+  const int chunk = blockIdx.x / ts, part = blockIdx.x - chunk * ts, c = blockIdx.y, iz = blockIdx.z;
   const int* cout_ptr = cls;
   const int* cout_dir = cls + ncls + 1;
   const int ne_tot = cout_ptr[ncls];
@@ -194,22 +217,22 @@ __global__ void __launch_bounds__(256) r2_t_kernel(const double* __restrict__ ti
   double* gs = reinterpret_cast<double*>(smraw);          // [e][n][i]
   double* zs = gs + (size_t)kCE * N * 4;                   // [m][e*4+i][2]
   const int tid = threadIdx.x;
-  for (int idx = tid; idx < kCE * N * 4; idx += blockDim.x) {
+  for (int idx = tid; idx < E * N * 4; idx += blockDim.x) {
     const int e = idx / (N * 4), rem = idx - e * N * 4;
-    gs[idx] = e < E ? g[((size_t)iz * nO + cout_dir[e0 + e]) * N * 4 + rem] : 0.0;
+    gs[idx] = g[((size_t)iz * nO + cout_dir[e0 + e]) * N * 4 + rem];
   }
+  const int NC = 4 * E;                                   // columns (e, i)
   __syncthreads();
   const size_t tsz = (size_t)N * ld;
   const double* tb = tiles + ((size_t)iz * ncls + c) * ntile * tsz;
-  for (int ti = 0; ti < ntile; ++ti) {
+  for (int ti = ntile * part / ts; ti < ntile * (part + 1) / ts; ++ti) {
     const double* T = tb + (size_t)ti * tsz;
     for (int m0 = 0; m0 < N; m0 += kMB2) {
-      // Zbar block: kMB2 m x (kCE * 4) columns, two entries per thread
-      for (int q = tid; q < kMB2 * kCE * 4; q += blockDim.x) {
-        const int mm = q / (kCE * 4), col = q - mm * (kCE * 4);
+      // Zbar block: kMB2 m x NC columns, at most two entries per thread
+      for (int q = tid; q < min(kMB2, N - m0) * NC; q += blockDim.x) {
+        const int mm = q / NC, col = q - mm * NC;
         const int m = m0 + mm, e = col >> 2, i = col & 3;
         double zr = 0.0, zi = 0.0;
-        if (m < N && e < E)
           for (int n = 0; n < N; ++n) {
             const double gv = gs[((size_t)e * N + n) * 4 + i];
             zr += T[(size_t)n * ld + m] * gv;
@@ -235,7 +258,7 @@ __global__ void __launch_bounds__(256) r2_t_kernel(const double* __restrict__ ti
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int col = e * 4 + i;
-          acc += y[(i * 4 + j) * 2] * zs[(mm * (kCE * 4) + col) * 2] + y[(i * 4 + j) * 2 + 1] * zs[(mm * (kCE * 4) + col) * 2 + 1];
+          acc += y[(i * 4 + j) * 2] * zs[(mm * NC + col) * 2] + y[(i * 4 + j) * 2 + 1] * zs[(mm * NC + col) * 2 + 1];
         }
         atomicAdd(&Ibar[(((size_t)iz * nO + pair_in[p]) * N + m) * 4 + j], acc);
       }
@@ -288,15 +311,19 @@ __global__ void r3_e_kernel(const double* __restrict__ g, const double* __restri
   }
 }
 
-__global__ void r3_ibar_kernel(const double* __restrict__ F, const double* __restrict__ rin,
-                               const double* __restrict__ r3w, double* __restrict__ Ibar, int nz, int nO, int N,
-                               int nq, int nl) {
-  const long long pt = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // (z, o', m)
-  if (pt >= (long long)nz * nO * N) return;
+// 32 points (lanes) per CTA, the terms q shared out between its warps and added in order
+// (the 72 terms of a two-term atom one after the other took 86 us for 6 x 16 x 48 points)
+__global__ void __launch_bounds__(256) r3_ibar_kernel(const double* __restrict__ F, const double* __restrict__ rin,
+                                                      const double* __restrict__ r3w, double* __restrict__ Ibar,
+                                                      int nz, int nO, int N, int nq, int nl) {
+  __shared__ double red[8][4][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long npt = (long long)nz * nO * N, pt0 = (long long)blockIdx.x * 32 + lane;   // (z, o', m)
+  const long long pt = pt0 < npt ? pt0 : npt - 1;
   const int m = (int)(pt % N);
   const int zo = (int)(pt / N), iz = zo / nO;
   double acc[4] = {0, 0, 0, 0};
-  for (int q = 0; q < nq; ++q) {
+  for (int q = warp; q < nq; q += 8) {
     const double* w = r3w + ((size_t)iz * nq + q) * 2 * N;
     const double* f = F + ((size_t)iz * (nq / nl) + q / nl) * 2;
     const double wr = w[m], wi = w[N + m];
@@ -305,7 +332,15 @@ __global__ void r3_ibar_kernel(const double* __restrict__ F, const double* __res
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j] += ri[2 * j] * cr - ri[2 * j + 1] * ci;
   }
-  for (int j = 0; j < 4; ++j) Ibar[pt * 4 + j] += acc[j];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) red[warp][j][lane] = acc[j];
+  __syncthreads();
+  if (warp < 4 && pt0 < npt) {
+    double v = red[0][warp][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) v += red[k][warp][lane];
+    Ibar[pt * 4 + warp] += v;
+  }
 }
 
 __global__ void to_f64_kernel(const float* __restrict__ a, double* __restrict__ b, size_t n) {
@@ -331,7 +366,6 @@ int apply_operator_t(Ctx* c, const void* x, void* y) {
     return fail(c, PRD_E_STATE, "adjoint needs the FP64 copy of the Sigma tables (not kept: too little memory)");
   const int nz = c->nz, nO = c->nO, N = c->nnu;
   const size_t nv = nvec(c);
-  const int nrows = nz * nO * 4;
   const double* tiles = (const double*)(fp32 ? c->tiles64.p : c->tiles.p);
   const double* Y = (const double*)(fp32 ? c->Y64.p : c->Y.p);
   const double* r3w = (const double*)(fp32 ? c->r3w64.p : c->r3w.p);
@@ -347,13 +381,10 @@ int apply_operator_t(Ctx* c, const void* x, void* y) {
   DBuf& g1 = c->adj[1];
   DBuf& g2 = c->adj[2];
   DBuf& ib = c->adj[3];
-  DBuf& ybr = c->adj[4];
-  DBuf& mbr = c->adj[5];
-  DBuf& F = c->adj[6];
+  DBuf& F = c->adj[4];
   int rc;
   if (!F.p && ((rc = dalloc(c, x64, nv * 8)) || (rc = dalloc(c, g1, nv * 8)) || (rc = dalloc(c, g2, nv * 8)) ||
-               (rc = dalloc(c, ib, nv * 8)) || (rc = dalloc(c, ybr, (size_t)nrows * N * 8)) ||
-               (rc = dalloc(c, mbr, (size_t)nrows * N * 8)) || (rc = dalloc(c, F, (size_t)nz * nuv * 2 * 8)))) {
+               (rc = dalloc(c, ib, nv * 8)) || (rc = dalloc(c, F, (size_t)nz * nuv * 2 * 8)))) {
     for (auto& b : c->adj) dfree(b);
     return rc;
   }
@@ -366,34 +397,36 @@ int apply_operator_t(Ctx* c, const void* x, void* y) {
   delo_t_kernel<double><<<cdiv((long long)nO * N, 128), 128, 0, c->stream>>>(
       xd, (const double*)(fp32 ? c->kt64.p : c->kt.p), (const double*)c->dmu.p, (double*)g1.p, nz, nO, N);
   // S6^T (with f): cotangent of the comoving emissivity
-  spline_t_kernel<<<cdiv(nrows, 64), 64, 0, c->stream>>>((const double*)g1.p, (const int*)c->ibk.p,
-                                                         (const double*)c->tbk.p, (const double*)c->sp.p,
-                                                         (const double*)c->f.p, (double*)ybr.p, (double*)mbr.p, nz,
-                                                         nO, N);
-  rows_to_vec_kernel<<<cdiv((long long)nrows * N, 256), 256, 0, c->stream>>>((const double*)ybr.p, (double*)g2.p,
-                                                                              nrows, N);
+  const size_t st_smem = spline_t_smem(N);
+  spline_t_kernel<<<dim3(nO, nz), kStThreads, st_smem, c->stream>>>(
+      (const double*)g1.p, (const int*)c->ibk.p, (const double*)c->tbk.p, (const double*)c->sp.p,
+      (const double*)c->f.p, (double*)g2.p, nO, N);
   // S3^T + S5^T: cotangent of the comoving field
   PRD_CUDA_TRY(c, cudaMemsetAsync(ib.p, 0, nv * 8, c->stream));
   {
     const size_t smem = sizeof(double) * ((size_t)kCE * N * 4 + (size_t)kMB2 * kCE * 4 * 2);
-    PRD_CUDA_TRY(c, cudaFuncSetAttribute(r2_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int nchunk = (c->max_cout + kCE - 1) / kCE;
-    r2_t_kernel<<<dim3(nchunk, c->ncls, nz), 256, smem, c->stream>>>(tiles, Y, (const double*)g2.p,
-                                                                     (const int*)c->cls_dev.p, (double*)ib.p, c->ncls,
-                                                                     c->ntile(), nO, N, c->npairs, ld);
+    const int ts = std::max(1, std::min(c->ntile(), 16 * c->nsm / (nchunk * c->ncls * nz)));
+    r2_t_kernel<<<dim3(nchunk * ts, c->ncls, nz), 256, smem, c->stream>>>(tiles, Y, (const double*)g2.p,
+                                                                          (const int*)c->cls_dev.p, (double*)ib.p,
+                                                                          c->ncls, c->ntile(), nO, N, c->npairs, ld, ts);
   }
   r3_e_kernel<<<dim3(nuv, nz), kTB, 0, c->stream>>>((const double*)g2.p, r3out, r3prof, r3ab, (double*)F.p, nO, N,
                                                     nuv, c->nl_st);
-  r3_ibar_kernel<<<cdiv((long long)nz * nO * N, 128), 128, 0, c->stream>>>((const double*)F.p, r3in, r3w,
+  r3_ibar_kernel<<<cdiv((long long)nz * nO * N, 32), 256, 0, c->stream>>>((const double*)F.p, r3in, r3w,
                                                                             (double*)ib.p, nz, nO, N, nq, c->nl_st);
   // S1^T
-  spline_t_kernel<<<cdiv(nrows, 64), 64, 0, c->stream>>>((const double*)ib.p, (const int*)c->iin.p,
-                                                         (const double*)c->tin.p, (const double*)c->sp.p, nullptr,
-                                                         (double*)ybr.p, (double*)mbr.p, nz, nO, N);
-  rows_to_vec_kernel<<<cdiv((long long)nrows * N, 256), 256, 0, c->stream>>>((const double*)ybr.p, (double*)g1.p,
-                                                                              nrows, N);
+  spline_t_kernel<<<dim3(nO, nz), kStThreads, st_smem, c->stream>>>(
+      (const double*)ib.p, (const int*)c->iin.p, (const double*)c->tin.p, (const double*)c->sp.p, nullptr,
+      (double*)g1.p, nO, N);
   sub_out_kernel<<<c->grid_ew(), 256, 0, c->stream>>>(xd, (const double*)g1.p, y, nv, fp32 ? 1 : 0);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
+  return PRD_OK;
+}
+
+// attribute of the transposed contraction (once per setup, like apply_prepare)
+int adjoint_prepare(Ctx* c) {
+  PRD_CUDA_TRY(c, cudaFuncSetAttribute(r2_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   return PRD_OK;
 }
 

@@ -65,8 +65,8 @@ static void free_all(Ctx* c) {
   DBuf* bufs[] = {&c->tiles, &c->tile_scale, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab, &c->kt,
                   &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk, &c->tin, &c->tbk, &c->cls_dev, &c->dmu,
                   &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M, &c->pc_lii, &c->pc_eta,
-                  &c->pc_delo, &c->pc_s1, &c->pc_s2, &c->pc_s3, &c->pc_s4, &c->gm_w, &c->gm_r, &c->gm_t, &c->gm_dots,
-                  &c->tc_err, &c->tc_work, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64, &c->r3out64,
+                  &c->pc_delo, &c->pc_qphi, &c->pc_x, &c->pc_r, &c->pc_v, &c->gm_t,
+                  &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64, &c->r3out64,
                   &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw, &c->cont_sig,
                   &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S, &c->kt64, &c->epsth64};
   invalidate_graphs(c);
@@ -125,7 +125,7 @@ static int setup(Ctx* c) {
   c->ready = false;
   free_all(c);
   int rc = build_host_tables(c);
-  if (rc || (rc = apply_prepare(c))) return rc;
+  if (rc || (rc = apply_prepare(c)) || (rc = adjoint_prepare(c))) return rc;
   if (c->lambda_only) {
     // the field gradient's perturbed formal solver: K, DELO weights, thermal emissivity
     if ((rc = upload(c, c->dmu, c->mu.data(), c->mu.size() * 8)) || (rc = build_device_tables(c)) ||
@@ -382,10 +382,10 @@ int prd_workspace_bytes(const prd_ctx* ctx, int64_t* bytes) {
                              &c->kt, &c->kt64, &c->epsth64, &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk,
                              &c->tin, &c->tbk,
                              &c->cls_dev, &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M,
-                             &c->pc_lii, &c->pc_eta, &c->pc_delo, &c->gm_t, &c->dmu, &c->pc_s1, &c->pc_s2,
-                             &c->pc_s3, &c->pc_s4, &c->tc_err, &c->tc_work, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64,
+                             &c->pc_lii, &c->pc_eta, &c->pc_delo, &c->gm_t, &c->dmu, &c->pc_qphi, &c->pc_x,
+                             &c->pc_r, &c->pc_v, &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64,
                              &c->r3out64, &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw,
-                             &c->cont_sig, &c->gm_w, &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S};
+                             &c->cont_sig, &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S};
   int64_t s = 0;
   for (auto* b : bufs) s += (int64_t)b->bytes;
   for (const auto& b : c->adj) s += (int64_t)b.bytes;   // scratch of the transposed operator, once used

@@ -6,6 +6,7 @@
 //   S5  R_III, separable in incident and outgoing frequency  (Eq. RIIIQKKp)
 //   S6  frame change back (u_n + u_b(z,Omega)) and Kirchhoff factor f (App. E)
 //   S7+S8  DELO-linear sweep per ray, y = x - Lambda eps      (Sect. 3)
+#include <algorithm>
 #include <cstdio>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -54,8 +55,17 @@ struct SplineSmem {
   static __host__ __device__ size_t bytes(int N) { return tab_off(N) + (size_t)2 * N * 8; }
 };
 
+// Contributions of the tensor-core contraction to a row, added to it as it is read: those of
+// the entries list[ptr[o]] .. of every part, ent [part][z][entry][N][4] (ent NULL: none).
+struct RowAdds {
+  const float4* ent = nullptr;
+  const int *ptr = nullptr, *list = nullptr;
+  int nent = 0, parts = 0;
+};
+
 template <typename T, int R>
-__global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict__ y, const int* __restrict__ kidx,
+__global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict__ y, RowAdds add,
+                                                             const int* __restrict__ kidx,
                                                              const double* __restrict__ tt,
                                                              const double* __restrict__ sp,
                                                              const double* __restrict__ fI, T* __restrict__ out,
@@ -78,7 +88,31 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
 #pragma unroll
     for (int r = 0; r < R; ++r)
       if (r < nr)
-        for (int i = tid; i < N; i += kSplThreads) ys[r * S + i] = src[(size_t)r * N + i];
+        for (int i = tid; i < N; i += kSplThreads) {
+          V v = src[(size_t)r * N + i];
+          if constexpr (sizeof(T) == 4) {
+            if (add.ent) {
+              // eight loads at a time, added in order
+              const int e1 = add.ptr[o0 + r + 1];
+              const size_t ps = (size_t)gridDim.y * add.nent * N;    // one part
+              const float4* base = add.ent + (size_t)iz * add.nent * N + i;
+              for (int e = add.ptr[o0 + r], p = 0; e < e1;) {
+                float4 w[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                  w[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                  if (e < e1) {
+                    w[q] = __ldcs(base + (size_t)add.list[e] * N + p * ps);
+                    if (++p == add.parts) { p = 0; ++e; }
+                  }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) { v.x += w[q].x; v.y += w[q].y; v.z += w[q].z; v.w += w[q].w; }
+              }
+            }
+          }
+          ys[r * S + i] = v;
+        }
   }
   for (int i = tid; i < N; i += kSplThreads) {
     cg[i] = tab[kSpCg * N + i];
@@ -173,13 +207,14 @@ static int allow_smem(Ctx* c, K kern) {
 }
 
 template <typename T>
-static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt, const double* fI, T* out, int nO) {
+static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt, const double* fI, T* out, int nO,
+                          const RowAdds& add = RowAdds()) {
   const double* sp = (const double*)c->sp.p;
   const int nz = c->nz, N = c->nnu;
   if (nz * nO <= kSplFew)
-    spline_kernel<T, 1><<<dim3(nO, nz), kSplThreads, SplineSmem<T, 1>::bytes(N), c->stream>>>(y, kidx, tt, sp, fI, out, nO, N);
+    spline_kernel<T, 1><<<dim3(nO, nz), kSplThreads, SplineSmem<T, 1>::bytes(N), c->stream>>>(y, add, kidx, tt, sp, fI, out, nO, N);
   else
-    spline_kernel<T, 4><<<dim3((nO + 3) / 4, nz), kSplThreads, SplineSmem<T, 4>::bytes(N), c->stream>>>(y, kidx, tt, sp, fI, out, nO, N);
+    spline_kernel<T, 4><<<dim3((nO + 3) / 4, nz), kSplThreads, SplineSmem<T, 4>::bytes(N), c->stream>>>(y, add, kidx, tt, sp, fI, out, nO, N);
 }
 
 // ------------------------------------------------------------------ R_III
@@ -221,42 +256,60 @@ __global__ void r3_J_kernel(const A* __restrict__ Ic, const T* __restrict__ r3w,
 }
 
 // eps_bar[z][o][n][i] = Re sum_uv ab[uv] J[uv] sum_l' O_i(o; uv, l') prof[uv][l'][n]
-// One block per (o, z), one thread per n: C = ab J per uv and the direction's
-// O_i coefficients are staged in shared memory; the profile rows are read
-// coalesced along n.  Arithmetic in A.
+// One block per (o, z): C = ab J per uv and the direction's O_i coefficients are
+// staged in shared memory; the profile rows are read coalesced along n.  The sum over
+// (uv, l') is a chain of loads, so where N is small its terms are shared out between `parts`
+// threads per n and added in order (72 terms one after the other took 27 us for 27
+// frequencies, shared out 9).  Arithmetic in A.
+constexpr int kR3Threads = 256;
 template <typename T, typename A>
-__global__ void r3_out_kernel(const double* __restrict__ J, const T* __restrict__ ab, const T* __restrict__ rout,
-                              const T* __restrict__ prof, A* __restrict__ eb, int nz, int nO, int N, int nuv,
-                              int nl) {
+__global__ void __launch_bounds__(kR3Threads) r3_out_kernel(const double* __restrict__ J, const T* __restrict__ ab,
+                                                            const T* __restrict__ rout, const T* __restrict__ prof,
+                                                            A* __restrict__ eb, int nO, int N, int nuv, int nl,
+                                                            int parts) {
+  using V = typename V4<A>::type;
   const int o = blockIdx.x, iz = blockIdx.y;
   const int zo = iz * nO + o;
   extern __shared__ __align__(16) unsigned char r3smem[];
-  A* C = reinterpret_cast<A*>(r3smem);                 // [uv][2]
+  V* P = reinterpret_cast<V*>(r3smem);                 // [part][n] partial sums (parts > 1)
+  A* C = reinterpret_cast<A*>(P + (parts > 1 ? parts * N : 0));   // [uv][2]
   A* R = C + 2 * nuv;                                  // [uv][l'][8]
-  for (int uv = threadIdx.x; uv < nuv; uv += blockDim.x) {
+  for (int uv = threadIdx.x; uv < nuv; uv += kR3Threads) {
     const double jr = J[((size_t)iz * nuv + uv) * 2], ji = J[((size_t)iz * nuv + uv) * 2 + 1];
     const double ar = (double)ab[((size_t)iz * nuv + uv) * 2], ai = (double)ab[((size_t)iz * nuv + uv) * 2 + 1];
     C[2 * uv] = (A)(ar * jr - ai * ji);
     C[2 * uv + 1] = (A)(ar * ji + ai * jr);
   }
-  for (int k = threadIdx.x; k < nuv * nl * 8; k += blockDim.x) R[k] = (A)rout[(size_t)zo * nuv * nl * 8 + k];
+  for (int k = threadIdx.x; k < nuv * nl * 8; k += kR3Threads) R[k] = (A)rout[(size_t)zo * nuv * nl * 8 + k];
   __syncthreads();
-  for (int n = threadIdx.x; n < N; n += blockDim.x) {
-    A acc[4] = {0, 0, 0, 0};
-    for (int uv = 0; uv < nuv; ++uv) {
+  const int part = threadIdx.x / N, n = threadIdx.x - part * N, nq = nuv * nl;
+  A acc[4] = {0, 0, 0, 0};
+  if (part < parts) {
+#pragma unroll 4
+    for (int q = part; q < nq; q += parts) {
+      const int uv = nl == 2 ? q >> 1 : q;             // 1 or 2 lower states
       const A cr = C[2 * uv], ci = C[2 * uv + 1];
-      for (int lp = 0; lp < nl; ++lp) {
-        const T* pp = prof + ((((size_t)iz * nuv + uv) * nl + lp) * N + n) * 2;
-        const A pr = (A)pp[0], pi = (A)pp[1];
-        const A dr = cr * pr - ci * pi, di = cr * pi + ci * pr;
-        const A* ro = R + (uv * nl + lp) * 8;
+      const T* pp = prof + (((size_t)iz * nq + q) * N + n) * 2;
+      const A pr = (A)pp[0], pi = (A)pp[1];
+      const A dr = cr * pr - ci * pi, di = cr * pi + ci * pr;
+      const A* ro = R + q * 8;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] += ro[2 * i] * dr - ro[2 * i + 1] * di;
-      }
+      for (int i = 0; i < 4; ++i) acc[i] += ro[2 * i] * dr - ro[2 * i + 1] * di;
     }
-    A* out = eb + ((size_t)zo * N + n) * 4;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) out[i] = acc[i];
+  }
+  if (parts > 1) {
+    if (part < parts) { V v; v.x = acc[0]; v.y = acc[1]; v.z = acc[2]; v.w = acc[3]; P[part * N + n] = v; }
+    __syncthreads();
+    if (part == 0)
+      for (int k = 1; k < parts; ++k) {
+        const V v = P[k * N + n];
+        acc[0] += v.x; acc[1] += v.y; acc[2] += v.z; acc[3] += v.w;
+      }
+  }
+  if (part == 0) {
+    V v;
+    v.x = acc[0]; v.y = acc[1]; v.z = acc[2]; v.w = acc[3];
+    reinterpret_cast<V*>(eb)[(size_t)zo * N + n] = v;
   }
 }
 
@@ -285,9 +338,10 @@ static void launch_r3_J(Ctx* c, const A* Ic, double* J, int nO, const SigmaTable
 template <typename T, typename A>
 static void launch_r3_out(Ctx* c, const double* J, const T* rout, A* eb, int nO, const SigmaTables& tb) {
   const int nuv = c->nu_st * c->nu_st, N = c->nnu;
-  const size_t smem = sizeof(A) * ((size_t)2 * nuv + (size_t)nuv * c->nl_st * 8);
-  r3_out_kernel<T, A><<<dim3(nO, c->nz), N <= 128 ? 128 : 256, smem, c->stream>>>(
-      J, (const T*)tb.r3ab, rout, (const T*)tb.r3prof, eb, c->nz, nO, N, nuv, c->nl_st);
+  const int parts = kR3Threads / N;                    // N <= 256
+  const size_t smem = sizeof(A) * ((parts > 1 ? (size_t)4 * parts * N : 0) + (size_t)2 * nuv + (size_t)nuv * c->nl_st * 8);
+  r3_out_kernel<T, A><<<dim3(nO, c->nz), kR3Threads, smem, c->stream>>>(
+      J, (const T*)tb.r3ab, rout, (const T*)tb.r3prof, eb, nO, N, nuv, c->nl_st, parts);
 }
 
 // ------------------------------------------------------------------ R_II (SIMT)
@@ -317,8 +371,8 @@ template <typename T, typename A>
 __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __restrict__ tiles, const float* __restrict__ tsc, const T* __restrict__ Y,
                                                       const A* __restrict__ Ic, const int* __restrict__ cls,
                                                       A* __restrict__ eb, int ncls, int ntrip, int nO, int N,
-                                                      int npairs, int ld, int fmt) {
-  const int chunk = blockIdx.x, c = blockIdx.y, iz = blockIdx.z;
+                                                      int npairs, int ld, int fmt, int ts) {
+  const int chunk = blockIdx.x / ts, part = blockIdx.x - chunk * ts, c = blockIdx.y, iz = blockIdx.z;
   const int* cout_ptr = cls;
   const int* cout_dir = cls + ncls + 1;
   const int ne_tot = cout_ptr[ncls];
@@ -346,7 +400,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
   // Z-building role: thread -> (e = tid & 15, m = tid >> 4)
   const int ze = tid & 15, zm = tid >> 4;
   const int e_z = e0 + ze;
-  for (int t = 0; t < ntrip; ++t) {
+  for (int t = ntrip * part / ts; t < ntrip * (part + 1) / ts; ++t) {
     const unsigned char* tile = tbase + (size_t)t * tile_sz;
     for (int m0 = 0; m0 < N; m0 += kMB) {
       // ---- Z block
@@ -444,8 +498,8 @@ __device__ __forceinline__ void dd_add(float& s, float& c, float x) {
 __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ tiles, const double* __restrict__ Y,
                                                     const double* __restrict__ Ic, const int* __restrict__ cls,
                                                     double* __restrict__ eb, int ncls, int ntrip, int nO, int N,
-                                                    int npairs, int ld) {
-  const int chunk = blockIdx.x, c = blockIdx.y, iz = blockIdx.z;
+                                                    int npairs, int ld, int ts) {
+  const int chunk = blockIdx.x / ts, part = blockIdx.x - chunk * ts, c = blockIdx.y, iz = blockIdx.z;
   const int* cout_ptr = cls;
   const int* cout_dir = cls + ncls + 1;
   const int ne_tot = cout_ptr[ncls];
@@ -470,7 +524,7 @@ __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ t
   const double* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
   const int ze = tid & 15, zm = tid >> 4;
   const int e_z = e0 + ze;
-  for (int t = 0; t < ntrip; ++t) {
+  for (int t = ntrip * part / ts; t < ntrip * (part + 1) / ts; ++t) {
     const double* tile = tbase + (size_t)t * tile_sz;
     for (int m0 = 0; m0 < N; m0 += kMB) {
       {
@@ -866,7 +920,6 @@ static int launch_delo(Ctx* c, const A* eps, const T* kt, const double* par, con
   if (allow_staged && c->staged_sweep && N % 2 == 0 && c->tc_err.p) {
     using L = DeloStage<T, A>;
     const int smem = kDStages * L::kBytes + 2 * kDStages * 8 + 16;
-    PRD_CUDA_TRY(c, cudaFuncSetAttribute(delo_staged_kernel<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     delo_staged_kernel<T, A><<<dim3(ceil_div(N, kDR), nO), 32 + kDR, smem, c->stream>>>(
         eps, kt, par, mu, x_sub, out, nz, nO, N, boundary, c->WT[0], (int*)c->tc_err.p);
   } else {
@@ -931,7 +984,8 @@ int apply_prepare(Ctx* c) {
   if ((rc = allow_smem(c, spline_kernel<float, 1>)) || (rc = allow_smem(c, spline_kernel<float, 4>)) ||
       (rc = allow_smem(c, spline_kernel<double, 1>)) || (rc = allow_smem(c, spline_kernel<double, 4>)) ||
       (rc = allow_smem(c, r2_simt_kernel<float, float>)) || (rc = allow_smem(c, r2_simt_kernel<float, double>)) ||
-      (rc = allow_smem(c, r2_simt_kernel<double, double>)) || (rc = allow_smem(c, r2_dd_kernel)))
+      (rc = allow_smem(c, r2_simt_kernel<double, double>)) || (rc = allow_smem(c, r2_dd_kernel)) ||
+      (rc = allow_smem(c, delo_staged_kernel<float, float>)) || (rc = allow_smem(c, delo_staged_kernel<double, double>)))
     return rc;
   return PRD_OK;
 }
@@ -960,49 +1014,48 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   // S3 + S4
   stage_begin(c, ST_S3, &e0);
   const int nchunk = (c->max_cout + kCW - 1) / kCW;
+  // CUDA-core contractions in FP64: with few work items their tiles are split between CTAs (the
+  // outputs are added up with atomics either way), up to about four CTAs per SM: 80 items of 4 tiles, 21 rows, FP64
+  // 292 -> 196 us; 96 items of 20 tiles, 26 rows, double-float 1120 -> 690 us
+  const int ts = std::is_same<A, double>::value
+                     ? std::max(1, std::min(c->ntile(), 4 * c->nsm / (nchunk * c->ncls * nz))) : 1;
   bool s3_done = false;   // the tensor-core or double-float contraction ran
+  RowAdds add;            // what the tensor cores contribute to eps_bar
   if constexpr (std::is_same<T, float>::value && std::is_same<A, float>::value) {
     if (c->use_tc && c->tc_ready && !t64) {
-      int rc = r2_tc_launch(c, Ic, eb);
+      int rc = r2_tc_launch(c, Ic);
       if (rc) return rc;
+      const int* lists = (const int*)c->tc_lists.p;
+      add = RowAdds{(const float4*)c->tc_ent.p, lists, lists + nO + 1, c->tc_nent, c->tc_parts};
       s3_done = true;
     }
   }
   if constexpr (std::is_same<T, double>::value && std::is_same<A, double>::value) {
     if (t64) {
       const size_t smem = sizeof(float4) * (size_t)kMB * kCW * 4 + sizeof(float2) * (size_t)2 * N * (kMB + 1);
-      r2_dd_kernel<<<dim3(nchunk, c->ncls, nz), 256, smem, c->stream>>>(
+      r2_dd_kernel<<<dim3(nchunk * ts, c->ncls, nz), 256, smem, c->stream>>>(
           (const double*)tb.tiles, (const double*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(), nO, N,
-          c->npairs, tb.ld);
+          c->npairs, tb.ld, ts);
       s3_done = true;
     }
   }
   if (!s3_done) {
     const size_t smem = sizeof(A) * (size_t)kMB * 2 * kCW * 4 + sizeof(T) * (size_t)2 * N * (kMB + 1);
-    r2_simt_kernel<T, A><<<dim3(nchunk, c->ncls, nz), 256, smem, c->stream>>>(
+    r2_simt_kernel<T, A><<<dim3(nchunk * ts, c->ncls, nz), 256, smem, c->stream>>>(
         (const unsigned char*)tb.tiles, tb.tsc, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(),
-        nO, N, c->npairs, tb.ld, tb.fmt);
+        nO, N, c->npairs, tb.ld, tb.fmt, ts);
   }
   stage_end(c, ST_S3, e0);
   // S6
   stage_begin(c, ST_S6, &e0);
   launch_spline<A>(c, eb, (const int*)c->ibk.p, (const double*)c->tbk.p, normalised ? (const double*)c->f.p : nullptr,
-                   eps, nO);
+                   eps, nO, add);
   // continuum scattering (App. A) joins the normalised emissivity; the
   // Kirchhoff factor is computed from the line alone (normalised = false)
   if (normalised && c->has_cont())
     continuum_kernel<A><<<ceil_div(npt, 256), 256, 0, c->stream>>>(x, (const double*)c->cont_pw.p,
                                                                  (const double*)c->cont_sig.p, eps, nz, nO, nO, N);
   stage_end(c, ST_S6, e0);
-  PRD_CUDA_TRY(c, cudaPeekAtLastError());
-  return PRD_OK;
-}
-
-// Frame change of an FP64 vector in either mode (the preconditioner's sweeps): to the
-// comoving frame (I(u_n - u_b)) or back (eps(u_n + u_b)).
-int spline_frame_change_d(Ctx* c, const double* in, double* out, bool to_comoving) {
-  launch_spline<double>(c, in, (const int*)(to_comoving ? c->iin.p : c->ibk.p),
-                        (const double*)(to_comoving ? c->tin.p : c->tbk.p), nullptr, out, c->nO);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
   return PRD_OK;
 }

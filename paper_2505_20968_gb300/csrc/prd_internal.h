@@ -134,7 +134,7 @@ struct Ctx {
   // the right-hand side and f (the formal solution of the residual operator
   // then carries no FP32 table rounding)
   DBuf kt64, epsth64;
-  DBuf adj[7];       // scratch of the transposed operator (allocated on first use)
+  DBuf adj[5];       // scratch of the transposed operator (allocated on first use)
   DBuf par;          // [z][o][n][3] DELOPAR source weights psi_M, psi_O, psi_P of the step arriving there (double)
   DBuf eta_line;     // [z][o][n] the line's share eta_line/eta_total of eta_I (double): f normalises the line only
   DBuf cont_pw;      // [o][o'][4][4] w_o' P(o, o') dipole phase matrix of continuum scattering (double)
@@ -156,12 +156,14 @@ struct Ctx {
   DBuf pc_lii;       // [z][o][n] Lambda_ii (T)
   DBuf pc_eta;       // [z][o][n]: eta1 (T)  (scalar Lambda*)
   DBuf pc_delo;      // [z][o][n][3] (T)
-  DBuf pc_s1, pc_s2, pc_s3, pc_s4;   // FP64 N-vector scratch of the sweeps
+  DBuf pc_qphi;      // [z][N][N] spline second derivatives of Phi_bar's columns (double)
+  DBuf pc_x, pc_r;   // [z][o][n] iterate and residual of the sweeps (double)
+  DBuf pc_v;         // [2][z][N] eps* before the frame change back: values, spline second derivatives (double)
   std::vector<double> pc_lii_host;
   void* pc_w = nullptr;   // device angular weights (double), owned via `owned`
   // GMRES
   std::vector<DBuf> krylov;
-  DBuf gm_w, gm_r, gm_t, gm_dots;
+  DBuf gm_t;
   // GMRES workspace kept across solves (basis V[m+1], residual r, operator
   // output w, current basis vector, device state), and the Arnoldi step
   // captured once as a CUDA graph over it: [0] A, [1] A^T
@@ -187,6 +189,9 @@ struct Ctx {
   DBuf tc_err;
   DBuf tc_work;      // tcgen05 contraction work records (r2_tc.cu)
   int tc_nwork = 0;
+  DBuf tc_ent;       // [tc_parts][z][entry][N][4] contributions of the records' entries (float)
+  DBuf tc_lists;     // entries of each output direction: [nO + 1] starts, then indices
+  int tc_nent = 0, tc_zs = 1, tc_parts = 1;
   bool tc_ready = false;
   int use_tc = 0;
   long long tc_spin = 0;   // poll limit of the contraction's pipeline waits (0: the default)
@@ -290,7 +295,8 @@ int upload_faddeeva_coeffs(Ctx* c);
 size_t nvec(const Ctx* c);   // 4*nz*nO*nnu
 int r2_tc_prepare(Ctx* c);
 int apply_prepare(Ctx* c);   // attributes of the per-apply kernels (once per setup)
-int r2_tc_launch(Ctx* c, const float* Ic, float* eb);
+int adjoint_prepare(Ctx* c);
+int r2_tc_launch(Ctx* c, const float* Ic);   // contributions to c->tc_ent, added up by the frame change back
 // drop the captured solver graphs (options, tables or workspace changed)
 void invalidate_graphs(Ctx* c);
 // Lockstep rounds of a batched solve (solver.cu): every context of the batch

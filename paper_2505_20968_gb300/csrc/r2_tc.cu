@@ -22,6 +22,11 @@
 // of that below, leaving <= 3 * 2^-24 a product.  TF32 products left 3 * 2^-22 at half the
 // rate.  BF16 contexts use bf16 planes, unscaled.
 //
+// The entries' contributions go to a buffer of their own and are added per output, in a fixed
+// order, where the frame change back reads its rows: repeated applies agree to the bit
+// (added with atomics they differed by the order the classes finished in, which far-wing
+// optical depths amplify a thousandfold), and 20 us of atomics an apply (8 heights) go.
+//
 // Roles (640 threads): warp 0 streams the tile into a ring of K step pairs with two bulk
 // asynchronous copies a step (the planes are stored pre-swizzled, step by step) and owns the
 // TMEM allocation; warp 1 issues tcgen05.mma; warps 4-19 stage I~ and Y and apply Y.  TMEM:
@@ -66,7 +71,7 @@ constexpr int kThreads = 128 + kEpi;          // warps 0, 1: copies, products (2
 constexpr int kRegsFew = 32, kRegsMany = 112;
 constexpr int kYS = 36;                       // floats of a staged pair: Re [j][i], -Im [j][i], 4 of padding (banks)
 constexpr int kYBytes = 2 * kMaxE * kYS * 4;  // one tile's Y (two buffers)
-constexpr int kRec = 4 + 32 + 32 + 64 + 32;   // ints of a work record
+constexpr int kRec = 4 + 32 + 64 + 32;        // ints of a work record
 constexpr int kAuxBytes = 2048;               // work record, column scales, barriers, TMEM slot, abort flag
 __host__ __device__ constexpr int rows16(int N) { return (N + 15) / 16 * 16; }
 // Tiles per pass: up to 64 (32) rows, two (four) tiles share the 128 accumulator rows, each
@@ -206,11 +211,11 @@ struct Params {
   const float* tsc;     // [z][class][N] power-of-two scale to undo per tile row (NULL: none)
   const float* Y;       // [z][pair][ntile][16][2]
   const float* Ic;      // [z][o][N][4]
-  const int* work;      // [item][kRec]: class, entries, incident directions, -, output direction of each entry,
-                        // its slots (a | b << 8 | pairs << 16), its pairs' indices, direction of each slot
-  float* eb;            // [z][o][N][4]
+  const int* work;      // [item][kRec]: class, entries, incident directions, first entry, then of each entry its
+                        // slots (a | b << 8 | pairs << 16) and its pairs' indices, and the direction of each slot
+  float* ent;           // [tile split * G][z][entry][N][4] contributions of the entries
   int* err;
-  int ncls, ntile, nO, N, npairs, ld;
+  int ncls, ntile, nO, N, npairs, ld, nent;
   int nst;              // tile stages
   int spin;             // poll limit of the pipeline waits (the drains keep kSpin)
 };
@@ -301,10 +306,9 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   const int c = rec[0], E = rec[1], ns = rec[2];
-  const int* vdir = rec + 4;
-  const int* vinfo = rec + 36;
-  const int* vpair = rec + 68;
-  const int* sdir = rec + 132;
+  const int* vinfo = rec + 4;
+  const int* vpair = rec + 36;
+  const int* sdir = rec + 100;
   const int passes = (t1 - t0 + G - 1) / G, iters = passes * KH;   // stages of kSteps = 2 steps
 
   if (warp < 4) {
@@ -600,10 +604,8 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
         for (int i = 0; i < kEV; ++i) {
           const int v = 4 * i + og;
           if (v < E) {
-            float* dst = p.eb + (((size_t)iz * p.nO + vdir[v]) * N + n) * 4;
-            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(acc[i][b][0] * sc),
-                         "f"(acc[i][b][1] * sc), "f"(acc[i][b][2] * sc), "f"(acc[i][b][3] * sc)
-                         : "memory");
+            float4* dst = reinterpret_cast<float4*>(p.ent) + (((size_t)(blockIdx.z * G + gt) * gridDim.y + iz) * p.nent + rec[3] + v) * N + n;
+            *dst = make_float4(acc[i][b][0] * sc, acc[i][b][1] * sc, acc[i][b][2] * sc, acc[i][b][3] * sc);
           }
         }
       }
@@ -649,7 +651,8 @@ static R2Kernel r2_tc_pick(const Ctx* c) {
 // takes several entries, which add up in eps_bar) and the entries packed into records of
 // at most 32 entries and 32 incident directions.  Where entries are many they are
 // taken by blocks of 32 incident directions, so that a record's entries share them.
-void r2_tc_records(const Ctx* c, std::vector<int>& out) {
+// entry_out: the output direction of every entry.
+static void r2_tc_records(const Ctx* c, std::vector<int>& out, std::vector<int>& entry_out) {
   using namespace tc;
   struct Entry { int o, p[2], n; };
   out.clear();
@@ -681,6 +684,7 @@ void r2_tc_records(const Ctx* c, std::vector<int>& out) {
         rec = (int)out.size();
         out.resize(out.size() + kRec, 0);
         out[rec] = k;
+        out[rec + 3] = (int)entry_out.size();
         slots.clear();
         add.clear();
         for (int i = 0; i < x.n; ++i) {
@@ -689,7 +693,7 @@ void r2_tc_records(const Ctx* c, std::vector<int>& out) {
         }
       }
       for (int d : add) {
-        out[rec + 132 + (int)slots.size()] = d;
+        out[rec + 100 + (int)slots.size()] = d;
         slots.push_back(d);
       }
       out[rec + 2] = (int)slots.size();
@@ -697,10 +701,10 @@ void r2_tc_records(const Ctx* c, std::vector<int>& out) {
       int sl[2] = {0, 0};
       for (int i = 0; i < x.n; ++i)
         sl[i] = (int)(std::find(slots.begin(), slots.end(), c->pair_in[x.p[i]]) - slots.begin());
-      out[rec + 4 + v] = x.o;
-      out[rec + 36 + v] = sl[0] | (sl[1] << 8) | (x.n << 16);
-      out[rec + 68 + 2 * v] = x.p[0];
-      out[rec + 68 + 2 * v + 1] = x.n > 1 ? x.p[1] : -1;
+      entry_out.push_back(x.o);
+      out[rec + 4 + v] = sl[0] | (sl[1] << 8) | (x.n << 16);
+      out[rec + 36 + 2 * v] = x.p[0];
+      out[rec + 36 + 2 * v + 1] = x.n > 1 ? x.p[1] : -1;
     }
   }
 }
@@ -717,35 +721,45 @@ int r2_tc_prepare(Ctx* c) {
   if (!c->tiled() || c->nnu > 224 || r2_tc_stages(c->nnu, c->hi_only) < 2)
     return fail(c, PRD_E_ARG, "tensor-core contraction needs FP32 tiles and N small enough for two tile stages "
                               "beside the resident I~ (N <= 224)");
-  std::vector<int> work;
-  r2_tc_records(c, work);
+  std::vector<int> work, eo;
+  r2_tc_records(c, work, eo);
   c->tc_nwork = (int)work.size() / tc::kRec;
-  dfree(c->tc_work);
-  int rc = dalloc(c, c->tc_work, work.size() * sizeof(int));
-  if (rc) return rc;
+  c->tc_nent = (int)eo.size();
+  // entries of each output direction, in order: [nO + 1] starts, then their indices
+  std::vector<int> lists(c->nO + 1, 0);
+  for (int o : eo) ++lists[o + 1];
+  for (int o = 0; o < c->nO; ++o) lists[o + 1] += lists[o];
+  std::vector<int> at(lists.begin(), lists.end() - 1);
+  lists.resize(c->nO + 1 + eo.size());
+  for (int e = 0; e < c->tc_nent; ++e) lists[c->nO + 1 + at[eo[e]]++] = e;
+  // fewer CTAs than SMs: split the tiles of a work item (at least 4 tiles each)
+  const int items = c->tc_nwork * c->nz;
+  c->tc_zs = std::max(1, std::min(c->ntile() / 4, c->nsm / std::max(1, items)));
+  c->tc_parts = c->tc_zs * tc::tiles_per_pass(c->nnu);
+  int rc;
+  if ((rc = upload(c, c->tc_work, work.data(), work.size() * sizeof(int))) ||
+      (rc = upload(c, c->tc_lists, lists.data(), lists.size() * sizeof(int))) ||
+      (rc = dalloc(c, c->tc_ent, (size_t)c->tc_parts * c->nz * c->tc_nent * c->nnu * 4 * sizeof(float))))
+    return rc;
   const int bf16 = c->tc_bf16;
   for (c->tc_bf16 = 0; c->tc_bf16 < 2; ++c->tc_bf16)   // the kernels PRD_OPT_CONTRACTION chooses from
     if (cudaFuncSetAttribute(r2_tc_pick(c), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) rc = PRD_E_CUDA;
   c->tc_bf16 = bf16;
   if (rc) return fail(c, rc, "shared memory of the tensor-core contraction");
-  PRD_CUDA_TRY(c, cudaMemcpy(c->tc_work.p, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice));
   PRD_CUDA_TRY(c, cudaMemset(c->tc_err.p, 0, sizeof(int)));
   c->tc_ready = true;
   return PRD_OK;
 }
 
-int r2_tc_launch(Ctx* c, const float* Ic, float* eb) {
+int r2_tc_launch(Ctx* c, const float* Ic) {
   // the deepest ring that fits, or the caller's (autotuned) depth if smaller
   const int nmax = r2_tc_stages(c->nnu, c->hi_only);
   const int nst = c->tc_stages >= 2 ? std::min(c->tc_stages, nmax) : nmax;
   tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->tile_scale.p, (const float*)c->Y.p, Ic,
-               (const int*)c->tc_work.p, eb, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu, c->npairs,
-               c->ld(), nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
+               (const int*)c->tc_work.p, (float*)c->tc_ent.p, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu,
+               c->npairs, c->ld(), c->tc_nent, nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
   const int smem = tc::smem_bytes(c->nnu, nst, c->hi_only);
-  // fewer CTAs than SMs: split the tiles of a work item (at least 4 tiles each)
-  const int items = c->tc_nwork * c->nz;
-  const int zs = std::max(1, std::min(c->ntile() / 4, c->nsm / std::max(1, items)));
-  r2_tc_pick(c)<<<dim3(c->tc_nwork, c->nz, zs), tc::kThreads, smem, c->stream>>>(p);
+  r2_tc_pick(c)<<<dim3(c->tc_nwork, c->nz, c->tc_zs), tc::kThreads, smem, c->stream>>>(p);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
   return PRD_OK;
 }
