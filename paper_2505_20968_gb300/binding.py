@@ -281,7 +281,8 @@ class PRD:
         self._check(lib().prd_set_option(self.h, PRD_OPT_TILE_STAGES, int(n)))
 
     def set_contraction(self, kind):
-        """Split products of the tensor-core contraction: "tf32x3" or "bf16x3"."""
+        """Split products of the tensor-core contraction: "tf32x3" (the FP32-level
+        products, of scaled FP16 halves) or "bf16x3"."""
         self._check(lib().prd_set_option(self.h, PRD_OPT_CONTRACTION,
                                          {"tf32x3": PRD_CONTRACTION_TF32X3, "bf16x3": PRD_CONTRACTION_BF16X3}[kind]))
 

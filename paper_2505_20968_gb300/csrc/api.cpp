@@ -66,7 +66,7 @@ static void free_all(Ctx* c) {
                   &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk, &c->tin, &c->tbk, &c->cls_dev, &c->dmu,
                   &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M, &c->pc_lii, &c->pc_eta,
                   &c->pc_delo, &c->pc_qphi, &c->pc_x, &c->pc_r, &c->pc_v, &c->gm_t,
-                  &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64, &c->r3out64,
+                  &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_tail, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64, &c->r3out64,
                   &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw, &c->cont_sig,
                   &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S, &c->kt64, &c->epsth64};
   invalidate_graphs(c);
@@ -383,7 +383,7 @@ int prd_workspace_bytes(const prd_ctx* ctx, int64_t* bytes) {
                              &c->tin, &c->tbk,
                              &c->cls_dev, &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M,
                              &c->pc_lii, &c->pc_eta, &c->pc_delo, &c->gm_t, &c->dmu, &c->pc_qphi, &c->pc_x,
-                             &c->pc_r, &c->pc_v, &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64,
+                             &c->pc_r, &c->pc_v, &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_tail, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64,
                              &c->r3out64, &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw,
                              &c->cont_sig, &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S};
   int64_t s = 0;

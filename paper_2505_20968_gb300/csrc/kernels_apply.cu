@@ -55,14 +55,6 @@ struct SplineSmem {
   static __host__ __device__ size_t bytes(int N) { return tab_off(N) + (size_t)2 * N * 8; }
 };
 
-// Contributions of the tensor-core contraction to a row, added to it as it is read: those of
-// the entries list[ptr[o]] .. of every part, ent [part][z][entry][N][4] (ent NULL: none).
-struct RowAdds {
-  const float4* ent = nullptr;
-  const int *ptr = nullptr, *list = nullptr;
-  int nent = 0, parts = 0;
-};
-
 template <typename T, int R>
 __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict__ y, RowAdds add,
                                                              const int* __restrict__ kidx,
@@ -92,22 +84,36 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
           V v = src[(size_t)r * N + i];
           if constexpr (sizeof(T) == 4) {
             if (add.ent) {
-              // eight loads at a time, added in order
-              const int e1 = add.ptr[o0 + r + 1];
-              const size_t ps = (size_t)gridDim.y * add.nent * N;    // one part
+              // the entries' G parts, eight loads at a time, added in order
+              const int e0 = add.ptr[o0 + r], e1 = add.ptr[o0 + r + 1], nz = gridDim.y;
+              const size_t ps = (size_t)nz * add.nent * N;             // one part
               const float4* base = add.ent + (size_t)iz * add.nent * N + i;
-              for (int e = add.ptr[o0 + r], p = 0; e < e1;) {
+              for (int e = e0, p = 0; e < e1;) {
                 float4 w[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                   w[q] = make_float4(0.f, 0.f, 0.f, 0.f);
                   if (e < e1) {
-                    w[q] = __ldcs(base + (size_t)add.list[e] * N + p * ps);
-                    if (++p == add.parts) { p = 0; ++e; }
+                    w[q] = base[p * ps + (size_t)add.list[e].x * N];
+                    if (++p == add.G) { p = 0; ++e; }
                   }
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q) { v.x += w[q].x; v.y += w[q].y; v.z += w[q].z; v.w += w[q].w; }
+              }
+              // and the further parts of this height's split items
+              if (add.zs > 1 && (iz + 1) * add.nwork > add.split0) {
+                const size_t ts = (size_t)add.nsplit * 32 * N;
+                for (int e = e0; e < e1; ++e) {
+                  const int l = add.list[e].y, it = iz * add.nwork + (l >> 5) - add.split0;
+                  if (it < 0) continue;
+                  const float4* a = add.tail + ((size_t)it * 32 + (l & 31)) * N + i;
+#pragma unroll 8
+                  for (int p = 0; p < add.G * (add.zs - 1); ++p) {
+                    const float4 w = a[p * ts];
+                    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+                  }
+                }
               }
             }
           }
@@ -385,15 +391,17 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
   A (*Zs)[2][kCW * 4] = reinterpret_cast<A (*)[2][kCW * 4]>(smraw);
   T* Asb = reinterpret_cast<T*>(smraw + sizeof(A) * kMB * 2 * kCW * 4);
   // As[h][n][mm] -> Asb[(h * N + n) * (kMB + 1) + mm]
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+  // columns of this block as a power of two: a block of 8 outputs has twice the threads per
+  // column, not half of them idle
+  const int tid = threadIdx.x, ne = e_end - e0;
+  const int lc = ne <= 4 ? 2 : (ne <= 8 ? 3 : 4), tx = tid & ((1 << lc) - 1), ty = tid >> lc, nty = 256 >> lc;
   const int e_mine = e0 + tx;
   A acc[kMaxRows][4];
 #pragma unroll
   for (int r = 0; r < kMaxRows; ++r)
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[r][i] = (A)0;
-  const int nrows = (N + 15) / 16;
+  const int nrows = (N + nty - 1) / nty;
   const size_t tile_sz = (size_t)N * ld * (fmt == TILE_BF16HI ? 2 : sizeof(T));
   const unsigned char* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
   const float* sc = fmt == TILE_FP16 ? tsc + ((size_t)iz * ncls + c) * N : nullptr;
@@ -403,6 +411,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
   for (int t = ntrip * part / ts; t < ntrip * (part + 1) / ts; ++t) {
     const unsigned char* tile = tbase + (size_t)t * tile_sz;
     for (int m0 = 0; m0 < N; m0 += kMB) {
+      const int mb = min(kMB, N - m0);
       // ---- Z block
       {
         const int m = m0 + zm;
@@ -437,7 +446,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
       }
       __syncthreads();
 #pragma unroll 4
-      for (int mm = 0; mm < kMB; ++mm) {
+      for (int mm = 0; mm < mb; ++mm) {
         A zr[4], zi[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -447,7 +456,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
 #pragma unroll
         for (int r = 0; r < kMaxRows; ++r) {
           if (r < nrows) {
-            const int n = ty + 16 * r;
+            const int n = ty + nty * r;
             if (n < N) {
               const A ar = Asb[n * (kMB + 1) + mm], ai = Asb[(N + n) * (kMB + 1) + mm];
 #pragma unroll
@@ -463,7 +472,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
     const int o = cout_dir[e_mine];
 #pragma unroll
     for (int r = 0; r < kMaxRows; ++r) {
-      const int n = ty + 16 * r;
+      const int n = ty + nty * r;
       if (r < nrows && n < N) {
         A* dst = eb + (((size_t)iz * nO + o) * N + n) * 4;
 #pragma unroll
@@ -511,15 +520,17 @@ __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ t
   extern __shared__ __align__(16) unsigned char smraw[];
   float4 (*Zs)[kCW * 4] = reinterpret_cast<float4 (*)[kCW * 4]>(smraw);        // [mm][col]: zr hi/lo, zi hi/lo
   float2* Asb = reinterpret_cast<float2*>(smraw + sizeof(float4) * kMB * kCW * 4);  // [(h N + n)(kMB+1) + mm]
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+  // columns of this block as a power of two: a block of 8 outputs has twice the threads per
+  // column, not half of them idle
+  const int tid = threadIdx.x, ne = e_end - e0;
+  const int lc = ne <= 4 ? 2 : (ne <= 8 ? 3 : 4), tx = tid & ((1 << lc) - 1), ty = tid >> lc, nty = 256 >> lc;
   const int e_mine = e0 + tx;
   float accs[kMaxRows][4], accc[kMaxRows][4];
 #pragma unroll
   for (int r = 0; r < kMaxRows; ++r)
 #pragma unroll
     for (int i = 0; i < 4; ++i) { accs[r][i] = 0.f; accc[r][i] = 0.f; }
-  const int nrows = (N + 15) / 16;
+  const int nrows = (N + nty - 1) / nty;
   const size_t tile_sz = (size_t)N * ld;
   const double* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
   const int ze = tid & 15, zm = tid >> 4;
@@ -527,6 +538,7 @@ __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ t
   for (int t = ntrip * part / ts; t < ntrip * (part + 1) / ts; ++t) {
     const double* tile = tbase + (size_t)t * tile_sz;
     for (int m0 = 0; m0 < N; m0 += kMB) {
+      const int mb = min(kMB, N - m0);
       {
         const int m = m0 + zm;
         double zr[4] = {0, 0, 0, 0}, zi[4] = {0, 0, 0, 0};
@@ -559,14 +571,14 @@ __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ t
       }
       __syncthreads();
 #pragma unroll 2
-      for (int mm = 0; mm < kMB; ++mm) {
+      for (int mm = 0; mm < mb; ++mm) {
         float4 z[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) z[i] = Zs[mm][tx * 4 + i];
 #pragma unroll
         for (int r = 0; r < kMaxRows; ++r) {
           if (r < nrows) {
-            const int n = ty + 16 * r;
+            const int n = ty + nty * r;
             if (n < N) {
               const float2 ar = Asb[n * (kMB + 1) + mm], ai = Asb[(N + n) * (kMB + 1) + mm];
 #pragma unroll
@@ -592,7 +604,7 @@ __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ t
     const int o = cout_dir[e_mine];
 #pragma unroll
     for (int r = 0; r < kMaxRows; ++r) {
-      const int n = ty + 16 * r;
+      const int n = ty + nty * r;
       if (r < nrows && n < N) {
         double* dst = eb + (((size_t)iz * nO + o) * N + n) * 4;
 #pragma unroll
@@ -1016,7 +1028,7 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   const int nchunk = (c->max_cout + kCW - 1) / kCW;
   // CUDA-core contractions in FP64: with few work items their tiles are split between CTAs (the
   // outputs are added up with atomics either way), up to about four CTAs per SM: 80 items of 4 tiles, 21 rows, FP64
-  // 292 -> 196 us; 96 items of 20 tiles, 26 rows, double-float 1120 -> 690 us
+  // 292 -> 110 us; 96 items of 20 tiles, 26 rows, double-float 1120 -> 690 us
   const int ts = std::is_same<A, double>::value
                      ? std::max(1, std::min(c->ntile(), 4 * c->nsm / (nchunk * c->ncls * nz))) : 1;
   bool s3_done = false;   // the tensor-core or double-float contraction ran
@@ -1025,8 +1037,7 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
     if (c->use_tc && c->tc_ready && !t64) {
       int rc = r2_tc_launch(c, Ic);
       if (rc) return rc;
-      const int* lists = (const int*)c->tc_lists.p;
-      add = RowAdds{(const float4*)c->tc_ent.p, lists, lists + nO + 1, c->tc_nent, c->tc_parts};
+      add = r2_tc_adds(c);
       s3_done = true;
     }
   }

@@ -189,9 +189,9 @@ struct Ctx {
   DBuf tc_err;
   DBuf tc_work;      // tcgen05 contraction work records (r2_tc.cu)
   int tc_nwork = 0;
-  DBuf tc_ent;       // [tc_parts][z][entry][N][4] contributions of the records' entries (float)
-  DBuf tc_lists;     // entries of each output direction: [nO + 1] starts, then indices
-  int tc_nent = 0, tc_zs = 1, tc_parts = 1;
+  DBuf tc_ent, tc_tail;   // contributions of the records' entries, and of split items' further parts (r2_tc.cu)
+  DBuf tc_lists;     // entries of each output direction: [nO + 1] starts, then (entry, place) pairs
+  int tc_nent = 0, tc_split0 = 0, tc_zs = 1;
   bool tc_ready = false;
   int use_tc = 0;
   long long tc_spin = 0;   // poll limit of the contraction's pipeline waits (0: the default)
@@ -296,6 +296,16 @@ size_t nvec(const Ctx* c);   // 4*nz*nO*nnu
 int r2_tc_prepare(Ctx* c);
 int apply_prepare(Ctx* c);   // attributes of the per-apply kernels (once per setup)
 int adjoint_prepare(Ctx* c);
+// Contributions of the tensor-core contraction to the rows of eps_bar, added as a row is read:
+// those of the entries list[ptr[o]] .. (ent NULL: none); an entry has G parts [g][z][entry][N] in
+// ent, and where its work item (z * nwork + record) is split, (zs - 1) G more in tail.
+struct RowAdds {
+  const float4 *ent = nullptr, *tail = nullptr;
+  const int* ptr = nullptr;
+  const int2* list = nullptr;    // (entry, record * 32 + its place in the record)
+  int nent = 0, G = 1, zs = 1, split0 = 0, nwork = 0, nsplit = 0;
+};
+RowAdds r2_tc_adds(const Ctx* c);
 int r2_tc_launch(Ctx* c, const float* Ic);   // contributions to c->tc_ent, added up by the frame change back
 // drop the captured solver graphs (options, tables or workspace changed)
 void invalidate_graphs(Ctx* c);

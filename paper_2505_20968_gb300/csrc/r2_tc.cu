@@ -213,9 +213,11 @@ struct Params {
   const float* Ic;      // [z][o][N][4]
   const int* work;      // [item][kRec]: class, entries, incident directions, first entry, then of each entry its
                         // slots (a | b << 8 | pairs << 16) and its pairs' indices, and the direction of each slot
-  float* ent;           // [tile split * G][z][entry][N][4] contributions of the entries
+  float4* ent;          // [G][z][entry][N] contributions of the entries
+  float4* tail;         // [(part - 1) * G][item - split0][kMaxE][N] those of the further parts of split items
   int* err;
-  int ncls, ntile, nO, N, npairs, ld, nent;
+  int ncls, ntile, nO, N, npairs, ld, nent, nz, nwork;
+  int split0, zs;       // work items from split0 on have their tiles split between zs CTAs
   int nst;              // tile stages
   int spin;             // poll limit of the pipeline waits (the drains keep kSpin)
 };
@@ -274,14 +276,17 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
-  const int iz = blockIdx.y;
+  // work item (z, record) and part of its tiles
+  const int past = max((int)blockIdx.x - p.split0, 0);
+  const int item = min((int)blockIdx.x, p.split0) + past / p.zs;
+  const int nparts = item >= p.split0 ? p.zs : 1, part = item >= p.split0 ? past % p.zs : 0;
+  const int iz = item / p.nwork;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // uniform
   const int et = threadIdx.x - 128;              // index among the Y threads
   constexpr uint32_t tm_cols = NB * 256u;
-  // tiles of this CTA (grid.z splits them where there are too few work items)
-  const int t0 = p.ntile * (int)blockIdx.z / (int)gridDim.z, t1 = p.ntile * ((int)blockIdx.z + 1) / (int)gridDim.z;
+  const int t0 = p.ntile * part / nparts, t1 = p.ntile * (part + 1) / nparts;
 
-  for (int i = threadIdx.x; i < kRec; i += kThreads) rec[i] = p.work[(size_t)blockIdx.x * kRec + i];
+  for (int i = threadIdx.x; i < kRec; i += kThreads) rec[i] = p.work[(size_t)(item - iz * p.nwork) * kRec + i];
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);        // armed by the producer with the bytes of the tile copy
@@ -604,8 +609,9 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
         for (int i = 0; i < kEV; ++i) {
           const int v = 4 * i + og;
           if (v < E) {
-            float4* dst = reinterpret_cast<float4*>(p.ent) + (((size_t)(blockIdx.z * G + gt) * gridDim.y + iz) * p.nent + rec[3] + v) * N + n;
-            *dst = make_float4(acc[i][b][0] * sc, acc[i][b][1] * sc, acc[i][b][2] * sc, acc[i][b][3] * sc);
+            float4* dst = part == 0 ? p.ent + (((size_t)gt * p.nz + iz) * p.nent + rec[3] + v) * N
+                                    : p.tail + ((((size_t)(part - 1) * G + gt) * (p.nz * p.nwork - p.split0) + item - p.split0) * kMaxE + v) * N;
+            dst[n] = make_float4(acc[i][b][0] * sc, acc[i][b][1] * sc, acc[i][b][2] * sc, acc[i][b][3] * sc);
           }
         }
       }
@@ -725,21 +731,33 @@ int r2_tc_prepare(Ctx* c) {
   r2_tc_records(c, work, eo);
   c->tc_nwork = (int)work.size() / tc::kRec;
   c->tc_nent = (int)eo.size();
-  // entries of each output direction, in order: [nO + 1] starts, then their indices
-  std::vector<int> lists(c->nO + 1, 0);
+  // entries of each output direction, in order: [nO + 1] starts, then (entry, record * kMaxE + its place)
+  std::vector<int> lists(c->nO + 1, 0), place(eo.size());
+  for (int r = 0; r < c->tc_nwork; ++r)
+    for (int v = 0; v < work[(size_t)r * tc::kRec + 1]; ++v) place[work[(size_t)r * tc::kRec + 3] + v] = r * tc::kMaxE + v;
   for (int o : eo) ++lists[o + 1];
   for (int o = 0; o < c->nO; ++o) lists[o + 1] += lists[o];
   std::vector<int> at(lists.begin(), lists.end() - 1);
-  lists.resize(c->nO + 1 + eo.size());
-  for (int e = 0; e < c->tc_nent; ++e) lists[c->nO + 1 + at[eo[e]]++] = e;
-  // fewer CTAs than SMs: split the tiles of a work item (at least 4 tiles each)
-  const int items = c->tc_nwork * c->nz;
-  c->tc_zs = std::max(1, std::min(c->ntile() / 4, c->nsm / std::max(1, items)));
-  c->tc_parts = c->tc_zs * tc::tiles_per_pass(c->nnu);
+  const int l0 = c->nO + 1 + (c->nO + 1) % 2;          // pairs start 8-byte aligned
+  lists.resize(l0 + 2 * eo.size());
+  for (int e = 0; e < c->tc_nent; ++e) {
+    int* l = &lists[l0 + 2 * at[eo[e]]++];
+    l[0] = e;
+    l[1] = place[e];
+  }
+  // Every item takes about as long, one CTA per SM: whole waves of items run as they are, and the
+  // tiles of the rest are split between the SMs of a last wave (at least 4 tiles, or two passes, a
+  // CTA).  On 152 SMs, contraction of Mg II 8 heights (768 items) 1000 -> 954 us, H I 4 heights x 96
+  // directions 812 -> 779, angle-averaged 512 items 309 -> 272.
+  const int items = c->tc_nwork * c->nz, rest = items % c->nsm;
+  c->tc_split0 = items - rest;
+  const int G = tc::tiles_per_pass(c->nnu);
+  c->tc_zs = rest ? std::max(1, std::min(c->ntile() / std::max(4, 2 * G), c->nsm / rest)) : 1;
   int rc;
   if ((rc = upload(c, c->tc_work, work.data(), work.size() * sizeof(int))) ||
       (rc = upload(c, c->tc_lists, lists.data(), lists.size() * sizeof(int))) ||
-      (rc = dalloc(c, c->tc_ent, (size_t)c->tc_parts * c->nz * c->tc_nent * c->nnu * 4 * sizeof(float))))
+      (rc = dalloc(c, c->tc_ent, (size_t)G * c->nz * c->tc_nent * c->nnu * sizeof(float4))) ||
+      (rc = dalloc(c, c->tc_tail, std::max<size_t>(16, (size_t)(c->tc_zs - 1) * G * rest * tc::kMaxE * c->nnu * sizeof(float4)))))
     return rc;
   const int bf16 = c->tc_bf16;
   for (c->tc_bf16 = 0; c->tc_bf16 < 2; ++c->tc_bf16)   // the kernels PRD_OPT_CONTRACTION chooses from
@@ -751,15 +769,22 @@ int r2_tc_prepare(Ctx* c) {
   return PRD_OK;
 }
 
+RowAdds r2_tc_adds(const Ctx* c) {
+  const int* lists = (const int*)c->tc_lists.p;
+  return RowAdds{(const float4*)c->tc_ent.p, (const float4*)c->tc_tail.p, lists, reinterpret_cast<const int2*>(lists + c->nO + 1 + (c->nO + 1) % 2),
+                 c->tc_nent, tc::tiles_per_pass(c->nnu), c->tc_zs, c->tc_split0, c->tc_nwork,
+                 (c->tc_nwork * c->nz - c->tc_split0)};
+}
+
 int r2_tc_launch(Ctx* c, const float* Ic) {
   // the deepest ring that fits, or the caller's (autotuned) depth if smaller
   const int nmax = r2_tc_stages(c->nnu, c->hi_only);
   const int nst = c->tc_stages >= 2 ? std::min(c->tc_stages, nmax) : nmax;
   tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->tile_scale.p, (const float*)c->Y.p, Ic,
-               (const int*)c->tc_work.p, (float*)c->tc_ent.p, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu,
-               c->npairs, c->ld(), c->tc_nent, nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
+               (const int*)c->tc_work.p, (float4*)c->tc_ent.p, (float4*)c->tc_tail.p, (int*)c->tc_err.p, c->ncls,
+               c->ntile(), c->nO, c->nnu, c->npairs, c->ld(), c->tc_nent, c->nz, c->tc_nwork, c->tc_split0, c->tc_zs, nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
   const int smem = tc::smem_bytes(c->nnu, nst, c->hi_only);
-  r2_tc_pick(c)<<<dim3(c->tc_nwork, c->nz, c->tc_zs), tc::kThreads, smem, c->stream>>>(p);
+  r2_tc_pick(c)<<<c->tc_split0 + (c->tc_nwork * c->nz - c->tc_split0) * c->tc_zs, tc::kThreads, smem, c->stream>>>(p);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
   return PRD_OK;
 }
