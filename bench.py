@@ -33,7 +33,9 @@ UNIT = "applies/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # layout tag of the contraction whose DRAM traffic profiles/traffic.json records;
 # the traffic figure is reported only while it matches the kernel that runs
-KERNEL_LAYOUT = "padded-v5"
+KERNEL_LAYOUT = "planes-v6"
+# what each value of --contraction multiplies on the tensor cores
+PRODUCTS = {"tf32x3": "scaled FP16 halves x3, FP32 level", "bf16x3": "bf16 halves x3", "bf16x2": "bf16 hi plane x2"}
 
 
 def _peaks():
@@ -402,13 +404,11 @@ def main():
     n_t = 18 if cfg["atom"]["twoS"] == 1 else 3
     useful, n_theta_omega = useful_contraction_flops(P, n_t=n_t)
     peaks, src = _peaks()
-    # The contraction runs 3 TF32 products per FP32-accurate product (hi*hi + hi*lo +
-    # lo*hi); its tensor time at peak exceeds the HBM time of streaming the tiles, so
-    # the tensor pipe at the TF32 rate bounds it.  TF32 peak = measured bf16 peak x
-    # the nominal dense TF32 / bf16 ratio (1.1 / 2.25 PFLOP/s).  `achieved` counts the
-    # useful work F3; `issued` the three TF32 products over the library's stored tiles
-    # (J-level means plus per-triple deviations, 20 per angle class).
-    tf32_peak = peaks["bf16_tflops"] * (1.1 / 2.25)
+    # The contraction runs 3 products of FP16 halves per FP32-accurate product (hi*hi + hi*lo +
+    # lo*hi); streaming the tiles once takes longer at the measured HBM rate than those products
+    # at the measured bf16 (= fp16) rate, so HBM bounds it.  `achieved` counts the tile bytes;
+    # `useful_tflops` the useful work F3 and `issued_frac` the three products over the stored
+    # tiles (J-level means plus per-triple deviations, 20 per angle class) against the tensor peak.
     achieved_tf = useful / (r2_ms * 1e-3) / 1e12
     issued_tf = 3.0 * flops / (r2_ms * 1e-3) / 1e12
     achieved_gbs = tile_bytes / (r2_ms * 1e-3) / 1e9
@@ -420,11 +420,12 @@ def main():
             traffic = tr.get("dram_bytes_per_launch")
     except (OSError, ValueError):
         pass
-    roofline = {"bound": "tensor", "kernel": f"r2_tc_kernel (S3+S4 R_II contraction, tcgen05 {args.contraction})",
-                "achieved": achieved_tf, "peak": tf32_peak, "unit": "TFLOP/s", "frac": achieved_tf / tf32_peak,
-                "useful_frac": achieved_tf / tf32_peak, "issued_frac": issued_tf / tf32_peak,
-                "issued": issued_tf,
-                "peak_source": src + " bf16 x nominal tf32/bf16 ratio", "traffic": traffic,
+    roofline = {"bound": "hbm", "kernel": f"r2_tc_kernel (S3+S4 R_II contraction, tcgen05, {PRODUCTS[args.contraction]})",
+                "achieved": achieved_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": achieved_gbs / peaks["hbm_gbs"],
+                "useful_tflops": achieved_tf, "useful_frac": achieved_tf / peaks["bf16_tflops"],
+                "issued": issued_tf, "issued_frac": issued_tf / peaks["bf16_tflops"],
+                "peak_source": src, "traffic": traffic,
                 "algorithmic_flops_per_launch": useful, "issued_flops_per_launch": 3.0 * flops,
                 "useful_flops_formula": f"16 N_r n_t N_nu^2 C = 16 x {P.nz} x {n_t} x {P.nN}^2 x {n_theta_omega}",
                 "algorithmic_bytes_per_launch": tile_bytes,
@@ -525,7 +526,7 @@ def main():
                 "clocks": clk,
                 "e2e": {"value": job_value(world, ms_e2e), "unit": UNIT, "h2d_bytes_per_step": nbytes,
                         "d2h_bytes_per_step": nbytes},
-                "gpu_launches": 8 * args.steps, "roofline": roofline, "cpu_baseline": cpu, "solve": solve,
+                "gpu_launches": 6 * args.steps, "roofline": roofline, "cpu_baseline": cpu, "solve": solve,
                 "contraction_modes": modes, "autotune": autotune, "batch": batch}
         print(json.dumps(line), flush=True)
     if dist:

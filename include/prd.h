@@ -54,18 +54,22 @@ enum {
 /* Precision of a context.  PRD_FP64: every table, vector and product in
  * FP64.  PRD_FP32: FP32 tables and vectors with FP64 reductions and an FP64
  * residual refinement in prd_solve; the R_II contraction runs on the tcgen05
- * tensor cores as 3xTF32 split products (<= 3 * 2^-22 per product).
+ * tensor cores as split products of scaled FP16 hi and lo parts, FP32 level
+ * (hi*hi + hi*lo + lo*hi, <= 3 * 2^-24 per product; the powers of two are one
+ * per tile row, and one per incident direction and Stokes parameter of the
+ * input, whose elements keep FP32 accuracy down to 2^-17 of the largest in that
+ * row over frequency, and 2^-40 of it in absolute terms below).
  * PRD_FP32_BF16X3: the same, with split-BF16 products (hi*hi + hi*lo + lo*hi
- * of bf16 halves, <= 3 * 2^-18 per product, twice the TF32 tensor rate); the
+ * of bf16 halves, <= 3 * 2^-18 per product, with FP32's range); the
  * context is a PRD_FP32 context (vectors are float) whose R_II tiles are
  * stored split into bf16 hi and lo planes in the operand layout of the MMA
  * (the same bytes as FP32), so its contraction is BF16x3 on the tensor cores
  * only: PRD_OPT_CONTRACTION = TF32X3 and PRD_OPT_TENSOR_CORES = 0 return
  * PRD_E_ARG.  A PRD_FP32 context can also run BF16x3 (PRD_OPT_CONTRACTION),
- * splitting its FP32 tiles on the fly.
+ * splitting its tiles again on the fly.
  * PRD_FP32_BF16X2: the same with the tiles stored as the bf16 hi plane alone
- * (half the bytes of FP32) and two products per element, hi(B)*hi(A) +
- * lo(B)*hi(A): the tile's rounding to bf16 (<= 2^-9 relative) is kept, so the
+ * (half the bytes of FP32) and two products per element, hi(I)*hi(A) +
+ * lo(I)*hi(A): the tile's rounding to bf16 (<= 2^-9 relative) is kept, so the
  * contraction is a ~1e-3-accurate inner operator; prd_solve's FP64 residuals
  * (FP64 table copy) still check the solution, and where the scattering
  * amplifies that error by more than its inverse (the Mg II case) the
@@ -239,7 +243,7 @@ int prd_apply_preconditioner(prd_ctx* ctx, const void* y_dev, void* x_dev);
 int prd_set_precond_sweeps(prd_ctx* ctx, int m_in);
 
 /* Options.  PRD_OPT_TENSOR_CORES (FP32 only): 1 runs the R_II contraction on
- * the tcgen05 tensor cores (TMA-fed tiles, TMEM accumulators, 3xTF32 split
+ * the tcgen05 tensor cores (TMA-fed tiles, TMEM accumulators, split
  * products), 0 on the CUDA cores.  PRD_OPT_PRECOND_SWEEPS: m_in as above.
  * PRD_OPT_WAIT_POLLS: poll limit of the tensor-core contraction's pipeline
  * waits (0: the default, 2^24 polls, about a second).  A wait that runs out
@@ -265,7 +269,8 @@ int prd_set_precond_sweeps(prd_ctx* ctx, int m_in);
  * The transposed operator, the adjoint solve and prd_grad_B are built for
  * DELO-linear and return PRD_E_STATE under PRD_DELOPAR.
  * PRD_OPT_CONTRACTION (FP32 contexts): the split products of the tensor-core
- * R_II contraction, PRD_CONTRACTION_TF32X3 (the PRD_FP32 default) or
+ * R_II contraction, PRD_CONTRACTION_TF32X3 (the PRD_FP32 default: the FP32-level
+ * products, three of 11-bit halves as in TF32, now taken in FP16) or
  * PRD_CONTRACTION_BF16X3 (the PRD_FP32_BF16X3 default).  prd_solve's FP64
  * residuals do not use the contraction, so the solution's accuracy is the
  * same with either; the inner iterations count changes.
@@ -342,10 +347,11 @@ int prd_narrowband(prd_ctx* ctx, const void* x_dev, int nlos, const double* mu, 
  * allocator, inside allocation-free real-time or replay loops, or in
  * environments where cudaMalloc is not permitted after initialisation.  This
  * call allocates nothing (no cudaMalloc/cudaFree, no allocating library call):
- * its intermediates (comoving field, spline second derivatives, comoving
- * emissivity, R_III moments) live in one static device array of 64 MiB that
- * every GPU which loads the library holds until the process exits.  A problem
- * whose intermediates need more than 64 MiB is rejected with PRD_E_ARG.  Each
+ * its intermediates (comoving field, comoving emissivity, R_III moments) live
+ * in one static device array of 64 MiB that every GPU which loads the library
+ * holds until the process exits, the tensor-core contraction's sums in the
+ * workspace of prd_setup.  A problem of which three vectors and the moments
+ * need more than 64 MiB is rejected with PRD_E_ARG.  Each
  * call looks up the array's device address in the current context (no
  * allocation; it stays valid if the device is reset in between); the first
  * call on a device may load the library's device code, so make it before any

@@ -40,9 +40,10 @@
 // poll loops in the products' warp 967.  HBM alone takes 722, the copies without products
 // 804, the products without copies or Y about 800 (shared memory feeds them at 100 bytes a
 // clock); the rest is their overlap, the operand's build (7 us a CTA) and a last wave.
-// Measured (operator apply, FP32, start -> now): that problem 3394 -> 1132 us, H I 4 x 96 x 150
-// 2680 -> 938, H I angle-averaged 8 x 64 x 91 12722 -> 400, Mg II 10 x 16 x 27 263 -> 79;
-// BF16x3, Mg II 4 x 64 x 163, 1314 -> 552 us.
+// Measured (operator apply, FP32; before: the operand formed per K step by builder warps, TF32 x3;
+// the frame changes and R_III of the apply also got faster): that problem 3398 -> 1152 us (its
+// contraction 954), H I 4 x 96 x 150 2681 -> 949, H I angle-averaged 8 x 64 x 91 12476 -> 382,
+// Mg II 10 x 16 x 27 262 -> 79; BF16x3, Mg II 4 x 64 x 163, 1316 -> 591 us.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
