@@ -51,6 +51,7 @@
 #include <cuda_fp16.h>
 #include "prd_internal.h"
 #include "device_common.cuh"
+#include "ring.h"
 
 namespace prd {
 
@@ -316,6 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   const int* vpair = rec + 36;
   const int* sdir = rec + 100;
   const int passes = (t1 - t0 + G - 1) / G, iters = passes * KH;   // stages of kSteps = 2 steps
+  int filled = 0;                                // stages warp 0 has filled
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
@@ -329,29 +331,24 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       const int pl = lane & 1, c2 = (lane >> 1) & 1, g = lane >> 2;
       const unsigned char* src = p.tiles + (((size_t)iz * p.ncls + c) * p.ntile + t0 + g) * KCH * sbytes + c2 * sbytes + pl * pbytes;
       unsigned char* dst = sm + c2 * SA + pl * PA + g * (4096 / G);
-      int it = 0, s = 0, ps = 0, j = 0, left = t1 - t0;   // it % nst and (it / nst) & 1; step pair; tiles left
-      for (; it < iters; ++it, s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1) {
-        if (it >= nst && !mbar_wait_warp(&empty[s], ps ^ 1, abort_flag, p.spin)) break;
-        // rows n >= N of the stage (and the places of a last pass's missing tiles) keep stale
-        // data: they only reach accumulator rows that nobody reads
-        const int g1 = min(G, left);
-        if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(kSteps * sbytes) * g1);
-        __syncwarp();
-        if (g < g1 && (!HI || pl == 0)) bulk_load(dst + s * kSteps * SA, src, pbytes, &full[s], pol_t);
-        src += kSteps * sbytes;
-        if (++j == KH) {
-          j = 0;
-          left -= G;
-          src += (size_t)(G - 1) * KCH * sbytes;
-        }
-      }
+      int j = 0, left = t1 - t0;                     // step pair of the pass; tiles left
+      filled = ring_produce(
+          iters, nst, [&](int s, uint32_t par) { return mbar_wait_warp(&empty[s], par, abort_flag, p.spin); },
+          [&](int s) {
+            // rows n >= N of the stage (and the places of a last pass's missing tiles) keep stale
+            // data: they only reach accumulator rows that nobody reads
+            const int g1 = min(G, left);
+            if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(kSteps * sbytes) * g1);
+            __syncwarp();
+            if (g < g1 && (!HI || pl == 0)) bulk_load(dst + s * kSteps * SA, src, pbytes, &full[s], pol_t);
+            src += kSteps * sbytes;
+            if (++j == KH) {
+              j = 0;
+              left -= G;
+              src += (size_t)(G - 1) * KCH * sbytes;
+            }
+          });
       __syncwarp();
-      if (*abort_flag) {
-        // drain copies that were issued and may not have been consumed
-        for (int k = max(0, it - nst); k < it; ++k)
-          for (int i = 0; i < kSpin && !mbar_try(&full[k % nst], (k / nst) & 1); ++i) {
-          }
-      }
     } else if (warp == 1) {
       // ---------------- products: the warp runs uniformly (waits by all lanes, descriptors in
       // uniform registers) and an elected lane issues; a loop of one lane issued a product
@@ -361,16 +358,17 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       const uint64_t a0 = sdesc32(sm), b0 = sdesc32(Iop);    // the address field counts 16 bytes
       // A stage's waits are kept to a bare poll loop, without a vote on their outcome or a look
       // at the abort flag (either cost 100 to 200 clocks a stage in this warp of few
-      // registers): a wait that gives up raises the flag and makes the waits after it one poll
-      // each, so the products to the end of the tile go to an accumulator nobody reads any
-      // more; the flag ends the loop at the next tile.
+      // registers).  A lane whose wait gives up raises the flag and polls no more (lim = 0).
+      // The products, their commits and with them a stage's return to the producer are the
+      // elected lane's, which leaves them out from then on: no stage goes back whose copies
+      // may be in flight.  The flag ends the loop at the next pass.
       int lim = p.spin;
       auto wait = [&](uint64_t* b, uint32_t par) {
         bool r = false;
         for (int i = 0; i < lim && !r; ++i) r = mbar_try(b, par);
         if (!r) {
           *abort_flag = 1;
-          lim = 1;
+          lim = 0;
         }
         __syncwarp();
       };
@@ -380,70 +378,76 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
         for (int i = 0; i < lim && !r; ++i) r = mbar_test(iready, 0);
         if (!r) {
           *abort_flag = 1;
-          lim = 1;
+          lim = 0;
         }
         __syncwarp();
       }
-      int s = 0, ps = 0;
+      RingPos pos;
       bool issued = false;
       for (int t = 0; t < passes; ++t) {
         if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
         int h = 0, kc = 0;                           // half and K step within it
         for (int j = 0; j < KH; ++j) {
-          wait(&full[s], ps);
-          // a half's accumulators are free once Y has been applied to the pass before
-          if (t > 0 && kc == 0) wait(&accfree[h], (t - 1) & 1);
-          if (t > 0 && kc + 1 == KH && h == 0) wait(&accfree[1], (t - 1) & 1);
-          if constexpr (CONV) {
-            for (int i = lane; i < kSteps * (PA / 16); i += 32) {
-              unsigned char* A = sm + s * kSteps * SA + (i >= PA / 16 ? SA : 0);
-              const int e = i >= PA / 16 ? i - PA / 16 : i;
-              uint4 h4 = reinterpret_cast<uint4*>(A)[e], l4 = reinterpret_cast<uint4*>(A + PA)[e];
-              uint32_t* hp = &h4.x;
-              uint32_t* lp = &l4.x;
+          ring_take(
+              pos, nst, lim,
+              [&](int s, uint32_t par, int& limit) {
+                wait(&full[s], par);
+                // a half's accumulators are free once Y has been applied to the pass before
+                if (t > 0 && kc == 0) wait(&accfree[h], (t - 1) & 1);
+                if (t > 0 && kc + 1 == KH && h == 0) wait(&accfree[1], (t - 1) & 1);
+                return limit > 0;
+              },
+              [&](int s, bool landed) {
+                if constexpr (CONV) {
+                  for (int i = landed ? lane : kSteps * (PA / 16); i < kSteps * (PA / 16); i += 32) {
+                    unsigned char* A = sm + s * kSteps * SA + (i >= PA / 16 ? SA : 0);
+                    const int e = i >= PA / 16 ? i - PA / 16 : i;
+                    uint4 h4 = reinterpret_cast<uint4*>(A)[e], l4 = reinterpret_cast<uint4*>(A + PA)[e];
+                    uint32_t* hp = &h4.x;
+                    uint32_t* lp = &l4.x;
 #pragma unroll
-              for (int q = 0; q < 4; q += 2) {
-                const float2 a = __half22float2(*reinterpret_cast<__half2*>(hp + q)), b = __half22float2(*reinterpret_cast<__half2*>(lp + q));
-                const float2 x = __half22float2(*reinterpret_cast<__half2*>(hp + q + 1)), f = __half22float2(*reinterpret_cast<__half2*>(lp + q + 1));
-                uint2 hi, lo;
-                split4<true>(make_float4(a.x + b.x, a.y + b.y, x.x + f.x, x.y + f.y), hi, lo);
-                hp[q] = hi.x; hp[q + 1] = hi.y;
-                lp[q] = lo.x; lp[q + 1] = lo.y;
-              }
-              reinterpret_cast<uint4*>(A)[e] = h4;
-              reinterpret_cast<uint4*>(A + PA)[e] = l4;
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-          }
-          if (kc == 0 || kc + 1 == KH)   // orders the products behind the Y warps' reads of the accumulators
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t as = a0 + (uint64_t)((uint32_t)(s * kSteps * SA) >> 4);
-          if (elect_one()) {
-            int h2 = h, k2 = kc;
+                    for (int q = 0; q < 4; q += 2) {
+                      const float2 a = __half22float2(*reinterpret_cast<__half2*>(hp + q)), b = __half22float2(*reinterpret_cast<__half2*>(lp + q));
+                      const float2 x = __half22float2(*reinterpret_cast<__half2*>(hp + q + 1)), f = __half22float2(*reinterpret_cast<__half2*>(lp + q + 1));
+                      uint2 hi, lo;
+                      split4<true>(make_float4(a.x + b.x, a.y + b.y, x.x + f.x, x.y + f.y), hi, lo);
+                      hp[q] = hi.x; hp[q + 1] = hi.y;
+                      lp[q] = lo.x; lp[q + 1] = lo.y;
+                    }
+                    reinterpret_cast<uint4*>(A)[e] = h4;
+                    reinterpret_cast<uint4*>(A + PA)[e] = l4;
+                  }
+                  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                  __syncwarp();
+                }
+                if (kc == 0 || kc + 1 == KH)   // orders the products behind the Y warps' reads of the accumulators
+                  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t as = a0 + (uint64_t)((uint32_t)(s * kSteps * SA) >> 4);
+                if (elect_one() && landed) {
+                  int h2 = h, k2 = kc;
 #pragma unroll
-            for (int u = 0; u < kSteps; ++u) {
-              const uint64_t ah = as + (uint64_t)((uint32_t)(u * SA) >> 4), al = ah + (uint64_t)((uint32_t)PA >> 4);
-              const uint64_t bh = b0 + (uint64_t)((uint32_t)(k2 * 2 * kPlane) >> 4), bl = bh + (kPlane >> 4);
+                  for (int u = 0; u < kSteps; ++u) {
+                    const uint64_t ah = as + (uint64_t)((uint32_t)(u * SA) >> 4), al = ah + (uint64_t)((uint32_t)PA >> 4);
+                    const uint64_t bh = b0 + (uint64_t)((uint32_t)(k2 * 2 * kPlane) >> 4), bl = bh + (kPlane >> 4);
 #pragma unroll
-              for (int b = 0; b < NB; ++b) {
-                const uint32_t d = tmem + (uint32_t)(h2 * NB + b) * 128u;
-                mma_f16(d, ah + b * 256, bh, idesc, k2 > 0 ? 1u : 0u);
-                mma_f16(d, ah + b * 256, bl, idesc, 1u);
-                if constexpr (!HI) mma_f16(d, al + b * 256, bh, idesc, 1u);
-              }
-              if (++k2 == KH) {
-                mma_commit(&accfull[h2]);
-                k2 = 0;
-                ++h2;
-              }
-            }
-            mma_commit(&empty[s]);
-          }
+                    for (int b = 0; b < NB; ++b) {
+                      const uint32_t d = tmem + (uint32_t)(h2 * NB + b) * 128u;
+                      mma_f16(d, ah + b * 256, bh, idesc, k2 > 0 ? 1u : 0u);
+                      mma_f16(d, ah + b * 256, bl, idesc, 1u);
+                      if constexpr (!HI) mma_f16(d, al + b * 256, bh, idesc, 1u);
+                    }
+                    if (++k2 == KH) {
+                      mma_commit(&accfull[h2]);
+                      k2 = 0;
+                      ++h2;
+                    }
+                  }
+                  mma_commit(&empty[s]);
+                }
+              });
           kc += kSteps;
           if (kc >= KH) { kc -= KH; ++h; }
           issued = true;
-          s = (s + 1 == nst) ? (ps ^= 1, 0) : s + 1;
         }
       }
       // every product issued completes before TMEM is released
@@ -622,6 +626,13 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   __syncthreads();
   if (*abort_flag && threadIdx.x == 0) atomicExch(p.err, 1);
   if (warp == 0) {
+    // a wait gave up: copies that nobody has waited for may be in flight (with every wait met
+    // all stages have been used)
+    if (*abort_flag)
+      ring_drain(filled, nst, [&](int s, uint32_t par) {
+        for (int i = 0; i < kSpin && !mbar_try(&full[s], par); ++i) {
+        }
+      });
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tm_cols));
   }
