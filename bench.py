@@ -35,7 +35,8 @@ PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # the traffic figure is reported only while it matches the kernel that runs
 KERNEL_LAYOUT = "planes-v6"
 # what each value of --contraction multiplies on the tensor cores
-PRODUCTS = {"tf32x3": "scaled FP16 halves x3, FP32 level", "bf16x3": "bf16 halves x3", "bf16x2": "bf16 hi plane x2"}
+PRODUCTS = {"tf32x3": "bf16 planes x6, FP32 level", "bf16x3": "bf16 planes x3", "bf16x2": "bf16 hi plane x2"}
+N_PRODUCTS = {"tf32x3": 6.0, "bf16x3": 3.0, "bf16x2": 2.0}
 
 
 def _peaks():
@@ -404,13 +405,13 @@ def main():
     n_t = 18 if cfg["atom"]["twoS"] == 1 else 3
     useful, n_theta_omega = useful_contraction_flops(P, n_t=n_t)
     peaks, src = _peaks()
-    # The contraction runs 3 products of FP16 halves per FP32-accurate product (hi*hi + hi*lo +
-    # lo*hi); streaming the tiles once takes longer at the measured HBM rate than those products
-    # at the measured bf16 (= fp16) rate, so HBM bounds it.  `achieved` counts the tile bytes;
-    # `useful_tflops` the useful work F3 and `issued_frac` the three products over the stored
+    # The contraction runs six products of bf16 planes per FP32-level product (three or two for
+    # the bf16 precisions); streaming the tiles once still takes longer at the measured HBM rate
+    # than those products at the measured bf16 rate, so HBM bounds it.  `achieved` counts the tile
+    # bytes; `useful_tflops` the useful work F3 and `issued_frac` the products over the stored
     # tiles (J-level means plus per-triple deviations, 20 per angle class) against the tensor peak.
     achieved_tf = useful / (r2_ms * 1e-3) / 1e12
-    issued_tf = 3.0 * flops / (r2_ms * 1e-3) / 1e12
+    issued_tf = N_PRODUCTS[args.contraction] * flops / (r2_ms * 1e-3) / 1e12
     achieved_gbs = tile_bytes / (r2_ms * 1e-3) / 1e9
     traffic = None
     try:
@@ -426,7 +427,7 @@ def main():
                 "useful_tflops": achieved_tf, "useful_frac": achieved_tf / peaks["bf16_tflops"],
                 "issued": issued_tf, "issued_frac": issued_tf / peaks["bf16_tflops"],
                 "peak_source": src, "traffic": traffic,
-                "algorithmic_flops_per_launch": useful, "issued_flops_per_launch": 3.0 * flops,
+                "algorithmic_flops_per_launch": useful, "issued_flops_per_launch": N_PRODUCTS[args.contraction] * flops,
                 "useful_flops_formula": f"16 N_r n_t N_nu^2 C = 16 x {P.nz} x {n_t} x {P.nN}^2 x {n_theta_omega}",
                 "algorithmic_bytes_per_launch": tile_bytes,
                 "hbm": {"achieved": achieved_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -480,7 +481,7 @@ def main():
         sol16, info16 = Pb.solve(tol=args.solve_tol, max_iter=900, restart=200, check=False)
         torch.cuda.synchronize()
         modes["bf16x3"] = {"contraction_ms": b16_ms, "useful_tflops": useful / (b16_ms * 1e-3) / 1e12,
-                           "issued_frac_of_bf16_peak": 3.0 * flops / (b16_ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
+                           "issued_frac_of_bf16_peak": N_PRODUCTS[args.contraction] * flops / (b16_ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
                            "hbm_frac": tile_bytes / (b16_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                            "solve_seconds": time.time() - t0, "solve_applies": info16["iters"],
                            "solve_true_rel_res": info16["true_rel_res"], "rc": info16["rc"],

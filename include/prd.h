@@ -54,13 +54,11 @@ enum {
 /* Precision of a context.  PRD_FP64: every table, vector and product in
  * FP64.  PRD_FP32: FP32 tables and vectors with FP64 reductions and an FP64
  * residual refinement in prd_solve; the R_II contraction runs on the tcgen05
- * tensor cores as split products of scaled FP16 hi and lo parts, FP32 level
- * (hi*hi + hi*lo + lo*hi, <= 3 * 2^-24 per product; the powers of two are one
- * per tile row, and one per incident direction and Stokes parameter of the
- * input, whose elements keep FP32 accuracy down to 2^-17 of the largest in that
- * row over frequency, and 2^-40 of it in absolute terms below).
+ * tensor cores with products at FP32 level: an FP32 value is three bf16 planes
+ * exactly, and six of the nine products of two values' planes are kept, which
+ * leaves <= 2^-24 of a product (1.004 times that), at any exponent.
  * PRD_FP32_BF16X3: the same, with split-BF16 products (hi*hi + hi*lo + lo*hi
- * of bf16 halves, <= 3 * 2^-18 per product, with FP32's range); the
+ * of bf16 planes, <= 2^-15 per product, with FP32's range); the
  * context is a PRD_FP32 context (vectors are float) whose R_II tiles are
  * stored split into bf16 hi and lo planes in the operand layout of the MMA
  * (the same bytes as FP32), so its contraction is BF16x3 on the tensor cores
@@ -69,7 +67,7 @@ enum {
  * splitting its tiles again on the fly.
  * PRD_FP32_BF16X2: the same with the tiles stored as the bf16 hi plane alone
  * (half the bytes of FP32) and two products per element, hi(I)*hi(A) +
- * lo(I)*hi(A): the tile's rounding to bf16 (<= 2^-9 relative) is kept, so the
+ * lo(I)*hi(A): the tile's rounding to bf16 (<= 2^-8 relative) is kept, so the
  * contraction is a ~1e-3-accurate inner operator; prd_solve's FP64 residuals
  * (FP64 table copy) still check the solution, and where the scattering
  * amplifies that error by more than its inverse (the Mg II case) the
@@ -270,7 +268,8 @@ int prd_set_precond_sweeps(prd_ctx* ctx, int m_in);
  * DELO-linear and return PRD_E_STATE under PRD_DELOPAR.
  * PRD_OPT_CONTRACTION (FP32 contexts): the split products of the tensor-core
  * R_II contraction, PRD_CONTRACTION_TF32X3 (the PRD_FP32 default: the FP32-level
- * products, three of 11-bit halves as in TF32, now taken in FP16) or
+ * products, six of bf16 planes; the name is that of the three TF32 products which first
+ * gave them) or
  * PRD_CONTRACTION_BF16X3 (the PRD_FP32_BF16X3 default).  prd_solve's FP64
  * residuals do not use the contraction, so the solution's accuracy is the
  * same with either; the inner iterations count changes.

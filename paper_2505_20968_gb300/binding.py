@@ -282,7 +282,7 @@ class PRD:
 
     def set_contraction(self, kind):
         """Split products of the tensor-core contraction: "tf32x3" (the FP32-level
-        products, of scaled FP16 halves) or "bf16x3"."""
+        products, six of bf16 planes) or "bf16x3"."""
         self._check(lib().prd_set_option(self.h, PRD_OPT_CONTRACTION,
                                          {"tf32x3": PRD_CONTRACTION_TF32X3, "bf16x3": PRD_CONTRACTION_BF16X3}[kind]))
 

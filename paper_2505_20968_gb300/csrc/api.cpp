@@ -62,7 +62,7 @@ int upload(Ctx* c, DBuf& b, const void* host, size_t bytes) {
 }
 
 static void free_all(Ctx* c) {
-  DBuf* bufs[] = {&c->tiles, &c->tile_scale, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab, &c->kt,
+  DBuf* bufs[] = {&c->tiles, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab, &c->kt,
                   &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk, &c->tin, &c->tbk, &c->cls_dev, &c->dmu,
                   &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M, &c->pc_lii, &c->pc_eta,
                   &c->pc_delo, &c->pc_qphi, &c->pc_x, &c->pc_r, &c->pc_v, &c->gm_t,
@@ -144,7 +144,6 @@ static int setup(Ctx* c) {
                                     std::to_string(fr >> 20) + " MiB free");
   if ((rc = dalloc(c, c->tiles, tile_bytes))) return rc;
   PRD_CUDA_TRY(c, cudaMemset(c->tiles.p, 0, tile_bytes));   // row padding (ld > 2N) stays zero
-  if (c->tile_fmt() == TILE_FP16 && (rc = dalloc(c, c->tile_scale, (size_t)c->nz * c->ncls * c->nnu * sizeof(float)))) return rc;
   const int nq = c->nu_st * c->nu_st * c->nl_st;
   if ((rc = dalloc(c, c->r3w, (size_t)c->nz * nq * 2 * c->nnu * c->esz))) return rc;
   // FP64 Sigma tables for the refinement residuals (FP32 mode), if they fit with room to spare
@@ -378,7 +377,7 @@ int prd_directions(const prd_ctx* ctx, double* mu, double* chi, double* w) {
 int prd_workspace_bytes(const prd_ctx* ctx, int64_t* bytes) {
   if (!ctx || !bytes) return PRD_E_ARG;
   const Ctx* c = &ctx->c;
-  const prd::DBuf* bufs[] = {&c->tiles, &c->tile_scale, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab,
+  const prd::DBuf* bufs[] = {&c->tiles, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab,
                              &c->kt, &c->kt64, &c->epsth64, &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk,
                              &c->tin, &c->tbk,
                              &c->cls_dev, &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M,

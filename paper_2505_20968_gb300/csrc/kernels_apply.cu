@@ -9,7 +9,6 @@
 #include <algorithm>
 #include <cstdio>
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <type_traits>
 #include "prd_internal.h"
 #include "device_common.cuh"
@@ -84,18 +83,17 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
           V v = src[(size_t)r * N + i];
           if constexpr (sizeof(T) == 4) {
             if (add.ent) {
-              // the entries' G parts, eight loads at a time, added in order
-              const int e0 = add.ptr[o0 + r], e1 = add.ptr[o0 + r + 1], nz = gridDim.y;
-              const size_t ps = (size_t)nz * add.nent * N;             // one part
-              const float4* base = add.ent + (size_t)iz * add.nent * N + i;
+              // the entries' parts, eight loads at a time, added in order
+              const int e0 = add.ptr[o0 + r], e1 = add.ptr[o0 + r + 1], cnt = gridDim.y * add.nent;
+              const int G = i >= add.n0 ? add.G : 1;
               for (int e = e0, p = 0; e < e1;) {
                 float4 w[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                   w[q] = make_float4(0.f, 0.f, 0.f, 0.f);
                   if (e < e1) {
-                    w[q] = base[p * ps + (size_t)add.list[e].x * N];
-                    if (++p == add.G) { p = 0; ++e; }
+                    w[q] = add.ent[add_off(p, iz * add.nent + add.list[e].x, cnt, N, add.n0, i)];
+                    if (++p == G) { p = 0; ++e; }
                   }
                 }
 #pragma unroll
@@ -103,15 +101,17 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
               }
               // and the further parts of this height's split items
               if (add.zs > 1 && (iz + 1) * add.nwork > add.split0) {
-                const size_t ts = (size_t)add.nsplit * 32 * N;
+                const size_t ps = (size_t)add.nsplit * 32 * (N + (add.G - 1) * (N - add.n0));
                 for (int e = e0; e < e1; ++e) {
                   const int l = add.list[e].y, it = iz * add.nwork + (l >> 5) - add.split0;
                   if (it < 0) continue;
-                  const float4* a = add.tail + ((size_t)it * 32 + (l & 31)) * N + i;
+                  for (int g = 0; g < G; ++g) {
+                    const float4* a = add.tail + add_off(g, it * 32 + (l & 31), add.nsplit * 32, N, add.n0, i);
 #pragma unroll 8
-                  for (int p = 0; p < add.G * (add.zs - 1); ++p) {
-                    const float4 w = a[p * ts];
-                    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+                    for (int p = 0; p < add.zs - 1; ++p) {
+                      const float4 w = a[p * ps];
+                      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+                    }
                   }
                 }
               }
@@ -324,14 +324,11 @@ __global__ void __launch_bounds__(kR3Threads) r3_out_kernel(const double* __rest
 struct SigmaTables {
   const void *tiles, *Y, *r3w, *r3in, *r3out, *r3prof, *r3ab;
   int ld, fmt;
-  const float* tsc;
 };
 static SigmaTables sigma_tables(const Ctx* c, bool t64) {
   if (t64)
-    return {c->tiles64.p, c->Y64.p, c->r3w64.p, c->r3in64.p, c->r3out64.p, c->r3prof64.p, c->r3ab64.p, c->ld64(), TILE_PLAIN,
-            nullptr};
-  return {c->tiles.p, c->Y.p, c->r3w.p, c->r3in.p, c->r3out.p, c->r3prof.p, c->r3ab.p, c->ld(), c->tile_fmt(),
-          (const float*)c->tile_scale.p};
+    return {c->tiles64.p, c->Y64.p, c->r3w64.p, c->r3in64.p, c->r3out64.p, c->r3prof64.p, c->r3ab64.p, c->ld64(), TILE_PLAIN};
+  return {c->tiles.p, c->Y.p, c->r3w.p, c->r3in.p, c->r3out.p, c->r3prof.p, c->r3ab.p, c->ld(), c->tile_fmt()};
 }
 
 // launchers (shared by the apply and the line-of-sight paths)
@@ -360,21 +357,18 @@ constexpr int kCW = 16;      // output directions per CTA
 constexpr int kMB = 16;      // incident-frequency block
 constexpr int kMaxRows = 16; // rows per thread (N <= 256)
 
-// element (n, k) of the stored tile at t (format fmt, row scale sc)
+// element (n, k) of the stored tile at t (format fmt)
 template <typename T>
-__device__ __forceinline__ T tile_get(const unsigned char* t, int n, int k, int N, int ld, int fmt, float sc) {
+__device__ __forceinline__ T tile_get(const unsigned char* t, int n, int k, int N, int ld, int fmt) {
   if (sizeof(T) == 8 || fmt == TILE_PLAIN) return reinterpret_cast<const T*>(t)[(size_t)n * ld + k];
-  if (fmt == TILE_FP16) {
-    const __half* h = reinterpret_cast<const __half*>(t);
-    return (T)((__half2float(h[tile_off_split(n, k, N, ld, false)]) + __half2float(h[tile_off_split(n, k, N, ld, true)])) * sc);
-  }
+  if (fmt == TILE_F32) return (T)reinterpret_cast<const float*>(t)[tile_off(n, k, N, ld, true)];
   const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(t);
   if (fmt == TILE_BF16HI) return (T)__bfloat162float(b[tile_off_hi(n, k, N, ld)]);
   return (T)(__bfloat162float(b[tile_off_split(n, k, N, ld, false)]) + __bfloat162float(b[tile_off_split(n, k, N, ld, true)]));
 }
 
 template <typename T, typename A>
-__global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __restrict__ tiles, const float* __restrict__ tsc, const T* __restrict__ Y,
+__global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __restrict__ tiles, const T* __restrict__ Y,
                                                       const A* __restrict__ Ic, const int* __restrict__ cls,
                                                       A* __restrict__ eb, int ncls, int ntrip, int nO, int N,
                                                       int npairs, int ld, int fmt, int ts) {
@@ -404,7 +398,6 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
   const int nrows = (N + nty - 1) / nty;
   const size_t tile_sz = (size_t)N * ld * (fmt == TILE_BF16HI ? 2 : sizeof(T));
   const unsigned char* tbase = tiles + ((size_t)iz * ncls + c) * ntrip * tile_sz;
-  const float* sc = fmt == TILE_FP16 ? tsc + ((size_t)iz * ncls + c) * N : nullptr;
   // Z-building role: thread -> (e = tid & 15, m = tid >> 4)
   const int ze = tid & 15, zm = tid >> 4;
   const int e_z = e0 + ze;
@@ -442,7 +435,7 @@ __global__ void __launch_bounds__(256) r2_simt_kernel(const unsigned char* __res
         const int h = (idx / kMB) & 1;
         const int n = idx / (2 * kMB);
         const int m = m0 + mm;
-        Asb[(h * N + n) * (kMB + 1) + mm] = (m < N) ? tile_get<T>(tile, n, h * N + m, N, ld, fmt, sc ? sc[n] : 1.f) : (T)0;
+        Asb[(h * N + n) * (kMB + 1) + mm] = (m < N) ? tile_get<T>(tile, n, h * N + m, N, ld, fmt) : (T)0;
       }
       __syncthreads();
 #pragma unroll 4
@@ -1053,7 +1046,7 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   if (!s3_done) {
     const size_t smem = sizeof(A) * (size_t)kMB * 2 * kCW * 4 + sizeof(T) * (size_t)2 * N * (kMB + 1);
     r2_simt_kernel<T, A><<<dim3(nchunk * ts, c->ncls, nz), 256, smem, c->stream>>>(
-        (const unsigned char*)tb.tiles, tb.tsc, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(),
+        (const unsigned char*)tb.tiles, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(),
         nO, N, c->npairs, tb.ld, tb.fmt, ts);
   }
   stage_end(c, ST_S3, e0);

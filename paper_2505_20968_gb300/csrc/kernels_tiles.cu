@@ -38,7 +38,6 @@
 #include <algorithm>
 #include <cstdio>
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include "prd_internal.h"
 #include "device_common.cuh"
 
@@ -523,18 +522,15 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) r3_kernel(R3Params p, floa
 // so that the large dispersion parts that cancel between Zeeman components
 // of one J level are summed once, in FP64, before rounding to the storage type.
 // One CTA per (row n, class, height); formats of the stored element (n, k):
-//   TILE_PLAIN  T, rows of ld (tiled: the FP32 K-step layout of tile_off)
-//   TILE_FP16   FP16 planes hi = rn(s v), lo = rn(s v - hi), s a power of two per (class, n) that
-//               brings the row's largest element over all tiles of the class to [2^13, 2^14);
-//               tsc[c][n] = 1/s
+//   TILE_PLAIN  T, rows of ld
+//   TILE_F32    FP32 in the K-step layout of tile_off
 //   TILE_BF16   bf16 planes (BF16x3), TILE_BF16HI the hi plane alone (BF16x2)
 constexpr int kSplitThreads = 128;
 
 template <typename T>
 __global__ void __launch_bounds__(kSplitThreads) group_split_kernel(const double* __restrict__ src, T* __restrict__ dst,
-                                                                    float* __restrict__ tsc, const int* __restrict__ grp,
-                                                                    int ncls, int ntrip, int ngrp, int N, int ld,
-                                                                    int tiled, int fmt) {
+                                                                    const int* __restrict__ grp, int ncls, int ntrip,
+                                                                    int ngrp, int N, int ld, int fmt) {
   const int n = blockIdx.x, c = blockIdx.y, z = blockIdx.z, nti = ngrp + ntrip;
   const size_t rowlen = (size_t)2 * N * N;             // one FP64 scratch tile: N rows of 2N
   src += ((size_t)z * ncls + c) * ntrip * rowlen + (size_t)n * 2 * N;
@@ -550,34 +546,9 @@ __global__ void __launch_bounds__(kSplitThreads) group_split_kernel(const double
     }
     for (int g = 0; g < ngrp; ++g) mean[g] = cnt[g] ? mean[g] / cnt[g] : 0.0;
   };
-  double scale = 1.0;
-  if (fmt == TILE_FP16) {
-    double m = 0.0, mean[2];
-    for (int k = threadIdx.x; k < 2 * N; k += kSplitThreads) {
-      means(k, mean);
-      for (int g = 0; g < ngrp; ++g) m = fmax(m, fabs(mean[g]));
-      for (int t = 0; t < ntrip; ++t) m = fmax(m, fabs(src[t * rowlen + k] - mean[grp[t]]));
-    }
-    __shared__ double red[kSplitThreads / 32];
-    for (int x = 16; x > 0; x >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, x));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    m = red[0];
-    for (int w = 1; w < kSplitThreads / 32; ++w) m = fmax(m, red[w]);
-    // exponent kept where the scale and its inverse are normal FP32 numbers
-    const int e = (m > 0.0 && m < 1e300) ? min(120, max(-120, 13 - ilogb(m))) : 0;
-    scale = ldexp(1.0, e);
-    if (threadIdx.x == 0) tsc[((size_t)z * ncls + c) * N + n] = (float)ldexp(1.0, -e);
-  }
   auto store = [&](int ti, int k, double v) {
-    if (fmt == TILE_PLAIN) {
-      dst[(t0 + ti) * tsz + tile_off(n, k, N, ld, tiled != 0)] = (T)v;
-    } else if (fmt == TILE_FP16) {
-      __half* t = reinterpret_cast<__half*>(dst) + (t0 + ti) * tsz * 2;
-      const double w = v * scale;
-      const __half hi = __float2half_rn((float)w);
-      t[tile_off_split(n, k, N, ld, false)] = hi;
-      t[tile_off_split(n, k, N, ld, true)] = __float2half_rn((float)(w - (double)__half2float(hi)));
+    if (fmt <= TILE_F32) {
+      dst[(t0 + ti) * tsz + tile_off(n, k, N, ld, fmt == TILE_F32)] = (T)v;
     } else if (fmt == TILE_BF16) {
       __nv_bfloat16* t = reinterpret_cast<__nv_bfloat16*>(dst) + (t0 + ti) * tsz * 2;
       const float w = (float)v;
@@ -656,9 +627,9 @@ struct TileGen {
   }
   // Stored tiles (group means, then deviations) of the heights z0 .. z0 + n - 1 from their rows in scr
   template <typename T>
-  int split(Ctx* c, int n, T* dst, int ld, int tiled, int fmt, float* tsc = nullptr) {
+  int split(Ctx* c, int n, T* dst, int ld, int fmt) {
     group_split_kernel<T><<<dim3(p.N, p.ncls, n), kSplitThreads, 0, c->stream>>>(
-        (const double*)scr.p, dst, tsc, (const int*)grp.p, p.ncls, p.ntrip, c->ngrp, p.N, ld, tiled, fmt);
+        (const double*)scr.p, dst, (const int*)grp.p, p.ncls, p.ntrip, c->ngrp, p.N, ld, fmt);
     PRD_CUDA_TRY(c, cudaPeekAtLastError());
     return PRD_OK;
   }
@@ -693,13 +664,12 @@ int launch_tiles(Ctx* c) {
     // their group mean, so their errors must be far below the storage epsilon
     if ((rc = g.rows(c, z0, n, (double*)g.scr.p))) break;
     if (c->prec == PRD_FP64) {
-      rc = g.split<double>(c, n, (double*)c->tiles.p + z0 * ztile, c->ld(), c->tiled(), TILE_PLAIN);
+      rc = g.split<double>(c, n, (double*)c->tiles.p + z0 * ztile, c->ld(), TILE_PLAIN);
     } else {
-      rc = g.split<float>(c, n, (float*)((char*)c->tiles.p + z0 * ztile * c->tile_esz()), c->ld(), 1, c->tile_fmt(),
-                          c->tile_scale.p ? (float*)c->tile_scale.p + (size_t)z0 * c->ncls * N : nullptr);
+      rc = g.split<float>(c, n, (float*)((char*)c->tiles.p + z0 * ztile * c->tile_esz()), c->ld(), c->tile_fmt());
       if (!rc && c->has64)
         rc = g.split<double>(c, n, (double*)c->tiles64.p + (size_t)z0 * c->ncls * c->ntile() * N * c->ld64(), c->ld64(),
-                             0, TILE_PLAIN);
+                             TILE_PLAIN);
     }
   }
   if (!rc) {
@@ -746,8 +716,8 @@ int los_tiles_angles(Ctx* c, LosTiles* t, const std::vector<double>& thetas) {
 int los_tiles_gen(Ctx* c, LosTiles* t, int z0, int n, void* out) {
   int rc = t->g.rows(c, z0, n, (double*)t->g.scr.p);
   if (rc) return rc;
-  return c->prec == PRD_FP64 ? t->g.split<double>(c, n, (double*)out, c->ld(), c->tiled(), TILE_PLAIN)
-                             : t->g.split<float>(c, n, (float*)out, c->ld(), c->tiled(), TILE_PLAIN);
+  return c->prec == PRD_FP64 ? t->g.split<double>(c, n, (double*)out, c->ld(), TILE_PLAIN)
+                             : t->g.split<float>(c, n, (float*)out, c->ld(), TILE_F32);
 }
 
 // Angle-averaged tiles and R_III incident weights of the unmagnetised J-level

@@ -34,7 +34,7 @@ constexpr int kAAThetaNodes = 48;
 // backward M_{r+1} = g_r - cp[r] M_{r+2}; the reciprocal pivots, and 6/h.
 enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpIden = 7, kSp6h = 8, kSpTabs = 9 };
 // Storage of the context's R_II tiles (kernels_tiles.cu, group_split_kernel)
-enum TileFmt { TILE_PLAIN = 0, TILE_FP16 = 1, TILE_BF16 = 2, TILE_BF16HI = 3 };
+enum TileFmt { TILE_PLAIN = 0, TILE_F32 = 1, TILE_BF16 = 2, TILE_BF16HI = 3 };
 // dynamic shared memory a CTA may have (opt-in limit of the device)
 constexpr int kMaxSmem = 227 * 1024;
 
@@ -121,7 +121,6 @@ struct Ctx {
   double refine_floor = 3e-5;  // FP32 refinement: floor of the inner GMRES relative tolerance
   int ld64() const { return (2 * nnu + 3) / 4 * 4; }
   DBuf tiles;        // [z][c][t][n][2N], format tile_fmt()
-  DBuf tile_scale;   // [z][c][n] power-of-two scale to undo (float; TILE_FP16 only)
   DBuf Y;            // [z][pair][t][16]    complex (T2)
   DBuf r3w;          // [z][q3][N] complex  (T2)  R_III incident weights
   DBuf r3in;         // [z][o'][q3][4] complex: w_o' * I_j(o'; ku, kv, kl)
@@ -195,11 +194,11 @@ struct Ctx {
   bool tc_ready = false;
   int use_tc = 0;
   long long tc_spin = 0;   // poll limit of the contraction's pipeline waits (0: the default)
-  int tc_bf16 = 0;         // contraction products: 0 split-FP16, 1 split-BF16 (BF16x3)
+  int tc_bf16 = 0;         // contraction products: 0 FP32 level (BF16x6), 1 split-BF16 (BF16x3)
   bool split_tiles = false;   // PRD_FP32_BF16X3/X2: R_II tiles stored as bf16 planes (tile_off_split)
   bool hi_only = false;       // PRD_FP32_BF16X2: the hi plane only (tile_off_hi), two products
   int tile_fmt() const {
-    return prec == PRD_FP64 ? TILE_PLAIN : (hi_only ? TILE_BF16HI : (split_tiles ? TILE_BF16 : TILE_FP16));
+    return prec == PRD_FP64 ? TILE_PLAIN : (hi_only ? TILE_BF16HI : (split_tiles ? TILE_BF16 : TILE_F32));
   }
   // bytes of one stored tile element (tile_bytes / elements of the padded layout)
   size_t tile_esz() const { return hi_only ? 2 : esz; }
@@ -297,14 +296,20 @@ int r2_tc_prepare(Ctx* c);
 int apply_prepare(Ctx* c);   // attributes of the per-apply kernels (once per setup)
 int adjoint_prepare(Ctx* c);
 // Contributions of the tensor-core contraction to the rows of eps_bar, added as a row is read:
-// those of the entries list[ptr[o]] .. (ent NULL: none); an entry has G parts [g][z][entry][N] in
-// ent, and where its work item (z * nwork + record) is split, (zs - 1) G more in tail.
+// those of the entries list[ptr[o]] .. (ent NULL: none).  An entry has one part in ent, [z][entry]
+// [N] rows, and for the rows from n0 on G - 1 more, [G - 1][z][entry][N - n0] behind it (add_off);
+// where its work item (z * nwork + record) is split, (zs - 1) times the same in tail, with
+// [item - split0][place in the record] in place of [z][entry].
 struct RowAdds {
   const float4 *ent = nullptr, *tail = nullptr;
   const int* ptr = nullptr;
   const int2* list = nullptr;    // (entry, record * 32 + its place in the record)
-  int nent = 0, G = 1, zs = 1, split0 = 0, nwork = 0, nsplit = 0;
+  int nent = 0, G = 1, n0 = 0, zs = 1, split0 = 0, nwork = 0, nsplit = 0;
 };
+// Place of part g of row n of the idx-th of `count` entries
+__host__ __device__ inline size_t add_off(int g, int idx, int count, int N, int n0, int n) {
+  return g == 0 ? (size_t)idx * N + n : (size_t)count * N + ((size_t)(g - 1) * count + idx) * (N - n0) + (n - n0);
+}
 RowAdds r2_tc_adds(const Ctx* c);
 int r2_tc_launch(Ctx* c, const float* Ic);   // contributions to c->tc_ent, added up by the frame change back
 // drop the captured solver graphs (options, tables or workspace changed)

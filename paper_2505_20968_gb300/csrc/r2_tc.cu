@@ -15,17 +15,15 @@
 // held the kernel at 2000 clocks a step of 16 columns and 200 rows, against the 630 in
 // which HBM delivers it.
 //
-// Operands are pairs of 16-bit planes, v = hi + lo, and a product is hi hi + hi lo + lo hi in
-// FP32: FP16 planes scaled by powers of two (one per tile row, one per incident direction
-// and Stokes parameter, from their largest element; undone exactly in FP32), which hold an
-// FP32 value to 2^-24 of itself down to 2^-17 of the row's largest element and to 2^-40
-// of that below, leaving <= 3 * 2^-24 a product.  TF32 products left 3 * 2^-22 at half the
-// rate.  BF16 contexts use bf16 planes, unscaled.
+// Here the tiles are stored as bf16 planes (PRD_FP32_BF16X3: hi and lo, PRD_FP32_BF16X2: hi alone), the
+// operands of the products as they land; r2_tc32.cu has the same contraction for FP32 tiles.
+// v = hi + lo, and a product is hi hi + hi lo + lo hi (2^-15 of it left out) in FP32.
 //
 // The entries' contributions go to a buffer of their own and are added per output, in a fixed
-// order, where the frame change back reads its rows: repeated applies agree to the bit
-// (added with atomics they differed by the order the classes finished in, which far-wing
-// optical depths amplify a thousandfold), and 20 us of atomics an apply (8 heights) go.
+// order, where the frame change back reads its rows: the sums of repeated applies agree to the
+// bit (added with atomics they differed by the order the classes finished in, which far-wing
+// optical depths amplify a thousandfold; R_III's moments are still FP64 atomics, whose order moves
+// their last bits), and 20 us of atomics an apply (8 heights) go.
 //
 // Roles (640 threads): warp 0 streams the tile into a ring of K step pairs with two bulk
 // asynchronous copies a step (the planes are stored pre-swizzled, step by step) and owns the
@@ -34,52 +32,29 @@
 // while Y is applied to the other.  Every mbarrier wait is bounded; on expiry the CTA
 // records an error flag, drains what it issued and returns.
 //
-// What shaped it, in turn (contraction of Mg II 8 heights x 64 directions x 200 frequencies):
-// the products' order above 2795 -> 1515 us; products issued by an elected lane of a uniform
-// warp 1200; K steps in pairs and 16 Y warps of 8 entries each instead of 8 of 16 1100; bare
+// What shaped it, in turn (contraction of Mg II 8 heights x 64 directions x 200 frequencies, both
+// planes in FP16): the products' order above 2795 -> 1515 us; products issued by an elected lane of a
+// uniform warp 1200; K steps in pairs and 16 Y warps of 8 entries each instead of 8 of 16 1100; bare
 // poll loops in the products' warp 967.  HBM alone takes 722, the copies without products
-// 804, the products without copies or Y about 800 (shared memory feeds them at 100 bytes a
-// clock); the rest is their overlap, the operand's build (7 us a CTA) and a last wave.
-// Measured (operator apply, FP32; before: the operand formed per K step by builder warps, TF32 x3;
-// the frame changes and R_III of the apply also got faster): that problem 3398 -> 1152 us (its
-// contraction 954), H I 4 x 96 x 150 2681 -> 949, H I angle-averaged 8 x 64 x 91 12476 -> 382,
-// Mg II 10 x 16 x 27 262 -> 79; BF16x3, Mg II 4 x 64 x 163, 1316 -> 591 us.
+// 804, the products without copies or Y about 800; the rest is their overlap, the operand's build
+// (7 us a CTA) and a last wave.
+// Measured (operator apply, BF16x3, Mg II 4 x 64 x 163; before: the operand formed per K step by builder
+// warps): 1316 -> 580 us.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-#include "prd_internal.h"
 #include "device_common.cuh"
-#include "ring.h"
+#include "r2_tc.cuh"
 
 namespace prd {
 
 namespace tc {
 
-constexpr int kStagesMax = 8;                 // tile ring depth: 2..8, the most that fit beside the rest
-constexpr int kKC = 16;                       // columns of a K step (32-byte rows per plane)
-constexpr int kSteps = 2;                     // K steps per stage: a stage's waits and commits cost the
-                                              // issuing warps some 300 clocks, a step's products 400
-constexpr int kMaxE = 32;                     // output entries per CTA
-constexpr int kMaxIn = 32;                    // incident directions per CTA (128 operand rows)
-constexpr int kPlane = 4 * kMaxIn * 32;       // bytes of one K step of one I~ plane
-constexpr int kEpiWarps = 16;
-constexpr int kEV = kMaxE / (kEpiWarps / 4);   // entries of a Y warp (4 warps share a lane quarter)
-constexpr int kEpi = 32 * kEpiWarps;          // threads of the Y warps
-constexpr int kThreads = 128 + kEpi;          // warps 0, 1: copies, products (2, 3 fill their warpgroup)
+// warps 0, 1: copies, products (2, 3 fill their warpgroup); then the Y warps
+constexpr int kThreads = 128 + kEpi;
 // registers a thread: launched with 96, the first warpgroup gives up what the Y warps'
 // accumulators need (128 * 32 + 512 * 112 = 640 * 96)
 constexpr int kRegsFew = 32, kRegsMany = 112;
-constexpr int kYS = 36;                       // floats of a staged pair: Re [j][i], -Im [j][i], 4 of padding (banks)
-constexpr int kYBytes = 2 * kMaxE * kYS * 4;  // one tile's Y (two buffers)
-constexpr int kRec = 4 + 32 + 64 + 32;        // ints of a work record
-constexpr int kAuxBytes = 2048;               // work record, column scales, barriers, TMEM slot, abort flag
-__host__ __device__ constexpr int rows16(int N) { return (N + 15) / 16 * 16; }
-// Tiles per pass: up to 64 (32) rows, two (four) tiles share the 128 accumulator rows, each
-// with its own lane quarters and Y, so a small tile does not leave most of a product
-// and of the Y warps idle.
-__host__ __device__ constexpr int tiles_per_pass(int N) { return N <= 32 ? 4 : (N <= 64 ? 2 : 1); }
 __host__ __device__ constexpr int plane_bytes(int N) { return (N <= 64 ? 128 : rows16(N)) * 32; }
 __host__ __device__ constexpr int step_bytes(int N, bool hi) { return plane_bytes(N) * (hi ? 1 : 2); }
 // Shared memory of one CTA: the tile ring, the resident I~ operand (two planes), two Y
@@ -89,173 +64,10 @@ __host__ __device__ constexpr int step_bytes(int N, bool hi) { return plane_byte
 __host__ __device__ constexpr int smem_bytes(int N, int st, bool hi) {
   return st * kSteps * step_bytes(N, hi) + rows16(N) / kKC * 2 * kPlane + 2 * tiles_per_pass(N) * kYBytes + kAuxBytes + 1024;
 }
-constexpr int kSpin = 1 << 24;                // bounded waits (default limit of the pipeline waits; drains)
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\tselp.b32 %0, 1, 0, P;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// the same without the suspension of try_wait
-__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred P;\n\tmbarrier.test_wait.parity.shared::cta.b64 P, [%1], %2;\n\tselp.b32 %0, 1, 0, P;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded pipeline wait of at most `limit` polls; returns false (and raises the
-// CTA abort flag) on expiry or when another role has aborted, which it looks at
-// between bursts of polls
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, int limit) {
-  bool r = mbar_try(b, parity);
-  for (int n = 1; !r && n < limit && !*abort_flag;) {
-    const int m = min(n + 64, limit);
-    for (; n < m && !r; ++n) r = mbar_try(b, parity);
-  }
-  if (!r) *abort_flag = 1;
-  return r;
-}
-// the same by a converged warp
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag, int limit) {
-  const bool r = mbar_wait(b, parity, abort_flag, limit);
-  return __all_sync(0xffffffffu, r);
-}
-
-// bulk asynchronous copy global -> shared (16-byte aligned ends, size a multiple
-// of 16) with an L2 eviction-priority policy
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-      ::"r"(smem_u32(dst)), "l"((uint64_t)src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
-      : "memory");
-}
-// the tiles are streamed once per apply: first out of L2, so that I~ and Y stay resident
-__device__ __forceinline__ uint64_t policy_evict_first() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-// 16-bit operands (kind::f16, both of one type), FP32 accumulation, K = 16 per instruction
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-      ::"r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-// shared-memory matrix descriptor: K-major, 32-byte swizzle (rows of 16 values),
-// 8-row groups 256 B apart
-__device__ __forceinline__ uint64_t sdesc32(const void* p) {
-  const uint64_t addr = (smem_u32(p) & 0x3FFFF) >> 4;
-  const uint64_t lbo = 1;            // unused for swizzled K-major
-  const uint64_t sbo = 256 >> 4;
-  return addr | (lbo << 16) | (sbo << 32) | (1ull << 46) | (6ull << 61);
-}
-// byte offset of the 4 values of k-group g (k = 4g .. 4g + 3, g < 4) of `row` in a
-// K-major 32-byte-swizzled operand: the 16-byte half (g >> 1) is exchanged with
-// the other in rows whose bit 2 is set
-__device__ __forceinline__ uint32_t swz32(int row, int g) {
-  return (uint32_t)row * 32u + (uint32_t)(((g >> 1) ^ ((row >> 2) & 1)) * 16) + (uint32_t)(g & 1) * 8u;
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-
-
-// Four values split into planes of the operand type: hi = rn(v), lo = rn(v - hi).
-template <bool BF>
-__device__ __forceinline__ void split4(float4 v, uint2& hi, uint2& lo) {
-  if constexpr (BF) {
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-    const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-    const __nv_bfloat162 l0 = __floats2bfloat162_rn(v.x - f0.x, v.y - f0.y);
-    const __nv_bfloat162 l1 = __floats2bfloat162_rn(v.z - f1.x, v.w - f1.y);
-    hi = {*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1)};
-    lo = {*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1)};
-  } else {
-    const __half2 h0 = __floats2half2_rn(v.x, v.y), h1 = __floats2half2_rn(v.z, v.w);
-    const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
-    const __half2 l0 = __floats2half2_rn(v.x - f0.x, v.y - f0.y), l1 = __floats2half2_rn(v.z - f1.x, v.w - f1.y);
-    hi = {*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1)};
-    lo = {*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1)};
-  }
-}
-
-// one lane of a converged warp (the same one every time)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
-  return r != 0;
-}
-
-struct Params {
-  const unsigned char* tiles;   // [z][class][tile] pre-swizzled K steps of [plane][N][16]
-  const float* tsc;     // [z][class][N] power-of-two scale to undo per tile row (NULL: none)
-  const float* Y;       // [z][pair][ntile][16][2]
-  const float* Ic;      // [z][o][N][4]
-  const int* work;      // [item][kRec]: class, entries, incident directions, first entry, then of each entry its
-                        // slots (a | b << 8 | pairs << 16) and its pairs' indices, and the direction of each slot
-  float4* ent;          // [G][z][entry][N] contributions of the entries
-  float4* tail;         // [(part - 1) * G][item - split0][kMaxE][N] those of the further parts of split items
-  int* err;
-  int ncls, ntile, nO, N, npairs, ld, nent, nz, nwork;
-  int split0, zs;       // work items from split0 on have their tiles split between zs CTAs
-  int nst;              // tile stages
-  int spin;             // poll limit of the pipeline waits (the drains keep kSpin)
-};
-
-// barrier over the Y warps only (named barrier 1), returning whether v holds on all of
-// them (keeps their loop exits uniform, so none waits at the barrier for one that left)
-__device__ __forceinline__ bool epi_all(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\tselp.b32 %0, 1, 0, q;\n\t}\n"
-      : "=r"(r)
-      : "r"((uint32_t)v), "n"(kEpi)
-      : "memory");
-  return r != 0;
-}
-
-// four TMEM columns of the warp's 32 lanes; the values are there after tmem_wait
-__device__ __forceinline__ void tmem_ld4(float (&w)[4], uint32_t addr) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3])
-               : "r"(addr));
-}
-template <int K>
-__device__ __forceinline__ void tmem_wait(float (&w)[K][4]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;");
-  // the values pass through here, so that no use of them moves above the wait
-#pragma unroll
-  for (int k = 0; k < K; ++k) asm volatile("" : "+f"(w[k][0]), "+f"(w[k][1]), "+f"(w[k][2]), "+f"(w[k][3]));
-}
 
 // NB: row blocks of 128 (N <= 128: 1, else 2).  G: tiles per pass (1, or 2 or 4 where N is
-// small).  BF: bf16 planes, else scaled FP16.  HI: the
-// tiles hold the hi plane alone (BF16x2: products hi hi + hi lo(I~)).  CONV: FP16 tiles
-// contracted with bf16 products (PRD_OPT_CONTRACTION): warp 1 re-splits each landed step
-// in place before its products.
-template <int NB, int G, bool BF, bool HI, bool CONV>
+// small).  HI: the tiles hold the hi plane alone (BF16x2: products hi hi + hi lo(I~)).
+template <int NB, int G, bool HI>
 __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   // 1024-byte aligned base, derived by offset so that the compiler keeps the
@@ -268,8 +80,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   unsigned char* Iop = sm + nst * kSteps * SA;   // [K step][hi | lo][128 rows][32 bytes]
   float* Ys = (float*)(Iop + KH * 2 * kPlane);   // [buffer][tile of the pass][entry][pair][kYS]
   int* rec = (int*)((unsigned char*)Ys + 2 * G * kYBytes);
-  float* colinv = (float*)(rec + kRec);          // scale to undo per operand row (o', j)
-  uint64_t* full = (uint64_t*)(((uintptr_t)(colinv + 4 * kMaxIn) + 7) & ~(uintptr_t)7);
+  uint64_t* full = (uint64_t*)(((uintptr_t)(rec + kRec) + 7) & ~(uintptr_t)7);
   uint64_t* empty = full + kStagesMax;
   uint64_t* accfull = empty + kStagesMax;        // [half] products of the half complete
   uint64_t* accfree = accfull + 2;               // [half] Y applied
@@ -331,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       const int pl = lane & 1, c2 = (lane >> 1) & 1, g = lane >> 2;
       const unsigned char* src = p.tiles + (((size_t)iz * p.ncls + c) * p.ntile + t0 + g) * KCH * sbytes + c2 * sbytes + pl * pbytes;
       unsigned char* dst = sm + c2 * SA + pl * PA + g * (4096 / G);
-      int j = 0, left = t1 - t0;                     // step pair of the pass; tiles left
+      int j = 0, left = t1 - t0;                     // stage of the pass; tiles left
       filled = ring_produce(
           iters, nst, [&](int s, uint32_t par) { return mbar_wait_warp(&empty[s], par, abort_flag, p.spin); },
           [&](int s) {
@@ -353,8 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       // ---------------- products: the warp runs uniformly (waits by all lanes, descriptors in
       // uniform registers) and an elected lane issues; a loop of one lane issued a product
       // every 160 clocks, three times what it takes to execute
-      const uint32_t ty = BF ? 1u : 0u;
-      const uint32_t idesc = (1u << 4) | (ty << 7) | (ty << 10) | ((uint32_t)(rows16(4 * ns) >> 3) << 17) | ((128u >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(rows16(4 * ns) >> 3) << 17) | ((128u >> 4) << 24);
       const uint64_t a0 = sdesc32(sm), b0 = sdesc32(Iop);    // the address field counts 16 bytes
       // A stage's waits are kept to a bare poll loop, without a vote on their outcome or a look
       // at the abort flag (either cost 100 to 200 clocks a stage in this warp of few
@@ -398,30 +208,8 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
                 return limit > 0;
               },
               [&](int s, bool landed) {
-                if constexpr (CONV) {
-                  for (int i = landed ? lane : kSteps * (PA / 16); i < kSteps * (PA / 16); i += 32) {
-                    unsigned char* A = sm + s * kSteps * SA + (i >= PA / 16 ? SA : 0);
-                    const int e = i >= PA / 16 ? i - PA / 16 : i;
-                    uint4 h4 = reinterpret_cast<uint4*>(A)[e], l4 = reinterpret_cast<uint4*>(A + PA)[e];
-                    uint32_t* hp = &h4.x;
-                    uint32_t* lp = &l4.x;
-#pragma unroll
-                    for (int q = 0; q < 4; q += 2) {
-                      const float2 a = __half22float2(*reinterpret_cast<__half2*>(hp + q)), b = __half22float2(*reinterpret_cast<__half2*>(lp + q));
-                      const float2 x = __half22float2(*reinterpret_cast<__half2*>(hp + q + 1)), f = __half22float2(*reinterpret_cast<__half2*>(lp + q + 1));
-                      uint2 hi, lo;
-                      split4<true>(make_float4(a.x + b.x, a.y + b.y, x.x + f.x, x.y + f.y), hi, lo);
-                      hp[q] = hi.x; hp[q + 1] = hi.y;
-                      lp[q] = lo.x; lp[q + 1] = lo.y;
-                    }
-                    reinterpret_cast<uint4*>(A)[e] = h4;
-                    reinterpret_cast<uint4*>(A + PA)[e] = l4;
-                  }
-                  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                  __syncwarp();
-                }
-                if (kc == 0 || kc + 1 == KH)   // orders the products behind the Y warps' reads of the accumulators
-                  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // orders the products behind the Y warps' reads of the accumulators
+                if (kc == 0 || kc + 1 == KH) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t as = a0 + (uint64_t)((uint32_t)(s * kSteps * SA) >> 4);
                 if (elect_one() && landed) {
                   int h2 = h, k2 = kc;
@@ -432,9 +220,9 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
 #pragma unroll
                     for (int b = 0; b < NB; ++b) {
                       const uint32_t d = tmem + (uint32_t)(h2 * NB + b) * 128u;
-                      mma_f16(d, ah + b * 256, bh, idesc, k2 > 0 ? 1u : 0u);
-                      mma_f16(d, ah + b * 256, bl, idesc, 1u);
-                      if constexpr (!HI) mma_f16(d, al + b * 256, bh, idesc, 1u);
+                      mma_bf16(d, ah + b * 256, bh, idesc, k2 > 0 ? 1u : 0u);
+                      mma_bf16(d, ah + b * 256, bl, idesc, 1u);
+                      if constexpr (!HI) mma_bf16(d, al + b * 256, bh, idesc, 1u);
                     }
                     if (++k2 == KH) {
                       mma_commit(&accfull[h2]);
@@ -481,59 +269,11 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
 #pragma unroll
     for (int k = 0; k < GY; ++k) ya[k] = yb[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     load_y(0);
-    // I~ operand: a warp per incident direction; the scale of each of its 4 rows brings
-    // the largest element to [2^13, 2^14)
-    for (int sl = warp - 4; sl < ns; sl += kEpiWarps) {
-      const float4* src = reinterpret_cast<const float4*>(p.Ic) + ((size_t)iz * p.nO + sdir[sl]) * N;
-      float sc[4] = {1.f, 1.f, 1.f, 1.f};
-      if constexpr (!BF) {
-        float m[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int k = lane; k < N; k += 32) {
-          const float4 v = src[k];
-          m[0] = fmaxf(m[0], fabsf(v.x)); m[1] = fmaxf(m[1], fabsf(v.y));
-          m[2] = fmaxf(m[2], fabsf(v.z)); m[3] = fmaxf(m[3], fabsf(v.w));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-#pragma unroll
-          for (int x = 16; x > 0; x >>= 1) m[j] = fmaxf(m[j], __shfl_xor_sync(0xffffffffu, m[j], x));
-          // 2^(13 - exponent), kept where it and its inverse are normal FP32 numbers
-          const int ex = (int)(__float_as_uint(m[j]) >> 23);          // biased exponent
-          const int e = (ex == 255 || m[j] == 0.f) ? 127 : min(253, max(1, 127 + 13 + 127 - ex));
-          sc[j] = __uint_as_float((uint32_t)e << 23);
-          if (lane == j) colinv[sl * 4 + j] = __uint_as_float((uint32_t)(254 - e) << 23);
-        }
-      } else if (lane < 4) {
-        colinv[sl * 4 + lane] = 1.f;
-      }
-      for (int g = lane; g < KH * 4; g += 32) {
-        float4 v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = 4 * g + k < N ? src[4 * g + k] : make_float4(0.f, 0.f, 0.f, 0.f);
-        unsigned char* dst = Iop + (g >> 2) * 2 * kPlane;
-        const float4 r[4] = {make_float4(v[0].x, v[1].x, v[2].x, v[3].x), make_float4(v[0].y, v[1].y, v[2].y, v[3].y),
-                             make_float4(v[0].z, v[1].z, v[2].z, v[3].z), make_float4(v[0].w, v[1].w, v[2].w, v[3].w)};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint2 hi, lo;
-          split4<BF>(make_float4(r[j].x * sc[j], r[j].y * sc[j], r[j].z * sc[j], r[j].w * sc[j]), hi, lo);
-          const uint32_t o = swz32(sl * 4 + j, g & 3);
-          *(uint2*)(dst + o) = hi;
-          *(uint2*)(dst + kPlane + o) = lo;
-        }
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    build_operand<2>(Iop, p.Ic, sdir, warp - 4, ns, iz, p.nO, N, KH);
     __syncwarp();
     if (lane == 0) mbar_arrive(iready);
-    bool ok = epi_all(true);                       // colinv is complete
+    bool ok = true;
 
-    float ci[4] = {1.f, 1.f, 1.f, 1.f};            // column scales of this thread's Y
-    if (ypair >= 0) {
-      const int info = vinfo[yp >> 1], sl = (yp & 1) ? (info >> 8) & 255 : info & 255;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) ci[j] = colinv[sl * 4 + j];
-    }
     // tile of the pass and row of this lane
     const int gt = q * G / 4, n0 = (q % (4 / G)) * 32 + lane;
     const bool live0 = (q % (4 / G)) * 32 < N, live1 = NB > 1 && 128 + q * 32 < N;
@@ -552,8 +292,8 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
         const int g = yg + 2 * k;
         if (g >= G) break;
         float* d = Yb + g * (kYBytes / 4) + yp * kYS + yi;             // [half][j][i]
-        d[0] = ya[k].x * ci[0]; d[4] = ya[k].z * ci[1]; d[8] = yb[k].x * ci[2]; d[12] = yb[k].z * ci[3];
-        d[16] = -ya[k].y * ci[0]; d[20] = -ya[k].w * ci[1]; d[24] = -yb[k].y * ci[2]; d[28] = -yb[k].w * ci[3];
+        d[0] = ya[k].x; d[4] = ya[k].z; d[8] = yb[k].x; d[12] = yb[k].z;
+        d[16] = -ya[k].y; d[20] = -ya[k].w; d[24] = -yb[k].y; d[28] = -yb[k].w;
       }
       ok = epi_all(ok);
       if (!ok) break;
@@ -609,14 +349,14 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
       for (int b = 0; b < NB; ++b) {
         const int n = b * 128 + n0;
         if (n >= N || (b > 0 && !live1)) continue;
-        const float sc = p.tsc ? p.tsc[((size_t)iz * p.ncls + c) * N + n] : 1.f;
 #pragma unroll
         for (int i = 0; i < kEV; ++i) {
           const int v = 4 * i + og;
           if (v < E) {
-            float4* dst = part == 0 ? p.ent + (((size_t)gt * p.nz + iz) * p.nent + rec[3] + v) * N
-                                    : p.tail + ((((size_t)(part - 1) * G + gt) * (p.nz * p.nwork - p.split0) + item - p.split0) * kMaxE + v) * N;
-            dst[n] = make_float4(acc[i][b][0] * sc, acc[i][b][1] * sc, acc[i][b][2] * sc, acc[i][b][3] * sc);
+            float4* dst = part == 0 ? p.ent + add_off(gt, iz * p.nent + rec[3] + v, p.nz * p.nent, N, 0, n)
+                                    : p.tail + (part - 1) * (size_t)G * p.nsplit * kMaxE * N +
+                                          add_off(gt, (item - p.split0) * kMaxE + v, p.nsplit * kMaxE, N, 0, n);
+            *dst = make_float4(acc[i][b][0], acc[i][b][1], acc[i][b][2], acc[i][b][3]);
           }
         }
       }
@@ -640,28 +380,31 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
 
 }  // namespace tc
 
-// Tile stages for N rows: the most (<= kStagesMax) whose shared memory fits.
-static int r2_tc_stages(int N, bool hi) {
-  for (int st = tc::kStagesMax; st >= 2; --st)
-    if (tc::smem_bytes(N, st, hi) <= kMaxSmem) return st;
-  return 0;
-}
-
-// The kernel of a context's tile format and products for N rows.
+// The kernel of a context's tiles (bf16 planes) for N rows.
 using R2Kernel = void (*)(tc::Params);
 template <int NB, int G>
-static R2Kernel r2_tc_pick(const Ctx* c) {
-  if (c->hi_only) return tc::r2_tc_kernel<NB, G, true, true, false>;
-  if (c->split_tiles) return tc::r2_tc_kernel<NB, G, true, false, false>;
-  if (c->tc_bf16) return tc::r2_tc_kernel<NB, G, true, false, true>;
-  return tc::r2_tc_kernel<NB, G, false, false, false>;
+static R2Kernel r2_tc_pick(bool hi) {
+  return hi ? tc::r2_tc_kernel<NB, G, true> : tc::r2_tc_kernel<NB, G, false>;
 }
 static R2Kernel r2_tc_pick(const Ctx* c) {
   switch (tc::tiles_per_pass(c->nnu)) {
-    case 4: return r2_tc_pick<1, 4>(c);
-    case 2: return r2_tc_pick<1, 2>(c);
-    default: return c->nnu <= 128 ? r2_tc_pick<1, 1>(c) : r2_tc_pick<2, 1>(c);
+    case 4: return r2_tc_pick<1, 4>(c->hi_only);
+    case 2: return r2_tc_pick<1, 2>(c->hi_only);
+    default: return c->nnu <= 128 ? r2_tc_pick<1, 1>(c->hi_only) : r2_tc_pick<2, 1>(c->hi_only);
   }
+}
+
+// Tile stages for N rows: the most (<= kStagesMax) whose shared memory fits.
+static int r2_tc_stages(const Ctx* c) {
+  if (!c->split_tiles) return r2_f32_stages(c->nnu);
+  for (int st = tc::kStagesMax; st >= 2; --st)
+    if (tc::smem_bytes(c->nnu, st, c->hi_only) <= kMaxSmem) return st;
+  return 0;
+}
+// Rows from which a pass takes several tiles, and how many
+static void r2_tc_packed(const Ctx* c, int* n0, int* G) {
+  *n0 = !c->split_tiles && c->nnu > 128 ? 128 : 0;
+  *G = tc::tiles_per_pass(c->nnu - *n0);
 }
 
 // Work records of the contraction: every class's outputs cut into entries of at most two
@@ -736,7 +479,7 @@ int r2_tc_prepare(Ctx* c) {
     PRD_CUDA_TRY(c, cudaMemset(c->tc_err.p, 0, sizeof(int)));
   }
   if (c->prec != PRD_FP32) return PRD_OK;
-  if (!c->tiled() || c->nnu > 224 || r2_tc_stages(c->nnu, c->hi_only) < 2)
+  if (!c->tiled() || c->nnu > 224 || r2_tc_stages(c) < 2)
     return fail(c, PRD_E_ARG, "tensor-core contraction needs FP32 tiles and N small enough for two tile stages "
                               "beside the resident I~ (N <= 224)");
   std::vector<int> work, eo;
@@ -763,19 +506,18 @@ int r2_tc_prepare(Ctx* c) {
   // directions 812 -> 779, angle-averaged 512 items 309 -> 272.
   const int items = c->tc_nwork * c->nz, rest = items % c->nsm;
   c->tc_split0 = items - rest;
-  const int G = tc::tiles_per_pass(c->nnu);
-  c->tc_zs = rest ? std::max(1, std::min(c->ntile() / std::max(4, 2 * G), c->nsm / rest)) : 1;
+  int n0, G;
+  r2_tc_packed(c, &n0, &G);
+  const size_t rows = c->nnu + (size_t)(G - 1) * (c->nnu - n0);   // stored per entry (RowAdds)
+  c->tc_zs = rest ? std::max(1, std::min(c->ntile() / std::max(4, 2 * tc::tiles_per_pass(c->nnu)), c->nsm / rest)) : 1;
   int rc;
   if ((rc = upload(c, c->tc_work, work.data(), work.size() * sizeof(int))) ||
       (rc = upload(c, c->tc_lists, lists.data(), lists.size() * sizeof(int))) ||
-      (rc = dalloc(c, c->tc_ent, (size_t)G * c->nz * c->tc_nent * c->nnu * sizeof(float4))) ||
-      (rc = dalloc(c, c->tc_tail, std::max<size_t>(16, (size_t)(c->tc_zs - 1) * G * rest * tc::kMaxE * c->nnu * sizeof(float4)))))
+      (rc = dalloc(c, c->tc_ent, c->nz * c->tc_nent * rows * sizeof(float4))) ||
+      (rc = dalloc(c, c->tc_tail, std::max<size_t>(16, (size_t)(c->tc_zs - 1) * rest * tc::kMaxE * rows * sizeof(float4)))))
     return rc;
-  const int bf16 = c->tc_bf16;
-  for (c->tc_bf16 = 0; c->tc_bf16 < 2; ++c->tc_bf16)   // the kernels PRD_OPT_CONTRACTION chooses from
-    if (cudaFuncSetAttribute(r2_tc_pick(c), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) rc = PRD_E_CUDA;
-  c->tc_bf16 = bf16;
-  if (rc) return fail(c, rc, "shared memory of the tensor-core contraction");
+  if (c->split_tiles) PRD_CUDA_TRY(c, cudaFuncSetAttribute(r2_tc_pick(c), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+  else if ((rc = r2_f32_prepare(c))) return rc;
   PRD_CUDA_TRY(c, cudaMemset(c->tc_err.p, 0, sizeof(int)));
   c->tc_ready = true;
   return PRD_OK;
@@ -783,20 +525,23 @@ int r2_tc_prepare(Ctx* c) {
 
 RowAdds r2_tc_adds(const Ctx* c) {
   const int* lists = (const int*)c->tc_lists.p;
-  return RowAdds{(const float4*)c->tc_ent.p, (const float4*)c->tc_tail.p, lists, reinterpret_cast<const int2*>(lists + c->nO + 1 + (c->nO + 1) % 2),
-                 c->tc_nent, tc::tiles_per_pass(c->nnu), c->tc_zs, c->tc_split0, c->tc_nwork,
-                 (c->tc_nwork * c->nz - c->tc_split0)};
+  RowAdds a{(const float4*)c->tc_ent.p, (const float4*)c->tc_tail.p, lists, reinterpret_cast<const int2*>(lists + c->nO + 1 + (c->nO + 1) % 2),
+            c->tc_nent, 1, 0, c->tc_zs, c->tc_split0, c->tc_nwork, c->tc_nwork * c->nz - c->tc_split0};
+  r2_tc_packed(c, &a.n0, &a.G);
+  return a;
 }
 
 int r2_tc_launch(Ctx* c, const float* Ic) {
   // the deepest ring that fits, or the caller's (autotuned) depth if smaller
-  const int nmax = r2_tc_stages(c->nnu, c->hi_only);
+  const int nmax = r2_tc_stages(c);
   const int nst = c->tc_stages >= 2 ? std::min(c->tc_stages, nmax) : nmax;
-  tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->tile_scale.p, (const float*)c->Y.p, Ic,
-               (const int*)c->tc_work.p, (float4*)c->tc_ent.p, (float4*)c->tc_tail.p, (int*)c->tc_err.p, c->ncls,
-               c->ntile(), c->nO, c->nnu, c->npairs, c->ld(), c->tc_nent, c->nz, c->tc_nwork, c->tc_split0, c->tc_zs, nst, c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
-  const int smem = tc::smem_bytes(c->nnu, nst, c->hi_only);
-  r2_tc_pick(c)<<<c->tc_split0 + (c->tc_nwork * c->nz - c->tc_split0) * c->tc_zs, tc::kThreads, smem, c->stream>>>(p);
+  const int items = c->tc_nwork * c->nz, nsplit = items - c->tc_split0, grid = c->tc_split0 + nsplit * c->tc_zs;
+  tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->Y.p, Ic, (const int*)c->tc_work.p, (float4*)c->tc_ent.p,
+               (float4*)c->tc_tail.p, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu, c->npairs, c->ld(), c->tc_nent,
+               c->nz, c->tc_nwork, c->tc_split0, nsplit, c->tc_zs, nst, 0,
+               c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
+  if (c->split_tiles) r2_tc_pick(c)<<<grid, tc::kThreads, tc::smem_bytes(c->nnu, nst, c->hi_only), c->stream>>>(p);
+  else r2_f32_launch(c, p, grid);
   PRD_CUDA_TRY(c, cudaPeekAtLastError());
   return PRD_OK;
 }

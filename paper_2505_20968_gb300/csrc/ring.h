@@ -46,6 +46,15 @@ PRD_RING_FN int ring_produce(int iters, int n, W&& wait_empty, F&& fill) {
   return it;
 }
 
+// Producer, before the ring's memory is laid out anew: waits until the consumer has given back
+// every stage of the `iters` filled; false when a wait gives up.
+template <class W>
+PRD_RING_FN bool ring_close(int iters, int n, W&& wait_empty) {
+  for (int k = iters > n ? iters - n : 0; k < iters; ++k)
+    if (!wait_empty(k % n, (unsigned)(k / n) & 1u)) return false;
+  return true;
+}
+
 // Consumer: takes the next stage.  wait_full(s, parity, limit): bounded wait of at most `limit`
 // polls, false when it gives up; use(s, landed): works on the stage and gives it back if it has
 // landed, does neither otherwise.  After a wait that gave up nothing is waited for or taken.

@@ -3,7 +3,8 @@ consumer thread run the header's rules against a model of the barriers (phases, 
 arrivals, bytes in flight) in which copies land late and any wait may give up, taking turns at
 random.  Checked in every trial, whether or not a wait gave up: "full" is armed once a phase, no
 copy starts while another fills its stage or its products read it, a stage is read only after its
-copies have landed, and none is in flight after the drain.  Two planted mistakes, a consumer that
+copies have landed, none is in use once the producer has closed the ring, and none in flight
+after the drain.  Two planted mistakes, a consumer that
 gives stages back after a wait that gave up and a producer that does not drain, are found by
 the same checks."""
 import os
@@ -106,6 +107,11 @@ static const char* trial(int n, int iters, int polls_p, int polls_c, unsigned se
           w.copying[s] += 1;
           w.step(0);
         });
+    // the ring's memory may be laid out anew
+    if (filled == iters &&
+        prd::ring_close(iters, n, [&](int s, unsigned par) { return w.wait(0, w.empty[s], par, polls_p, true); }))
+      for (int s = 0; s < n; ++s)
+        if (w.copying[s] || w.reading[s]) w.fault("ring closed with a stage in use");
     w.end(0);
   });
   std::thread cons([&] {
