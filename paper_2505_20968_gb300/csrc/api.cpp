@@ -90,12 +90,12 @@ void stage_begin(Ctx* c, int stage, cudaEvent_t* out) {
   *out = e;
 }
 
-void stage_end(Ctx* c, int stage, cudaEvent_t start) {
+void stage_end(Ctx* c, int stage, cudaEvent_t start, bool count) {
   if (!c->prof || !start) return;
   cudaEvent_t e;
   if (cudaEventCreate(&e) != cudaSuccess) return;
   cudaEventRecord(e, c->stream);
-  c->ev_pending.push_back({stage, {start, e}});
+  c->ev_pending.push_back({2 * stage + (count ? 1 : 0), {start, e}});
 }
 
 void stage_collect(Ctx* c) {
@@ -103,8 +103,8 @@ void stage_collect(Ctx* c) {
     float ms = 0.f;
     if (cudaEventSynchronize(p.second.second) == cudaSuccess &&
         cudaEventElapsedTime(&ms, p.second.first, p.second.second) == cudaSuccess) {
-      c->stage_ms[p.first] += ms;
-      c->stage_n[p.first] += 1;
+      c->stage_ms[p.first >> 1] += ms;
+      c->stage_n[p.first >> 1] += p.first & 1;
     }
     cudaEventDestroy(p.second.first);
     cudaEventDestroy(p.second.second);
@@ -135,6 +135,8 @@ static int setup(Ctx* c) {
     c->ready = true;
     return PRD_OK;
   }
+  // the contraction's workspace, so that the sizes below are weighed against what it leaves
+  if ((rc = r2_tc_prepare(c))) return rc;
   // memory check for the tiles
   const size_t tile_bytes = (size_t)c->nz * c->ncls * c->ntile() * c->nnu * c->ld() * c->tile_esz();
   size_t fr = 0, tot = 0;
@@ -160,7 +162,6 @@ static int setup(Ctx* c) {
   if ((rc = build_device_tables(c))) return rc;
   if ((rc = dalloc(c, c->gm_t, nvec(c) * c->esz))) return rc;
   if ((rc = launch_tiles(c))) return rc;
-  if ((rc = r2_tc_prepare(c))) return rc;
   if ((rc = compute_normalisation(c))) return rc;
   if ((rc = launch_precond_setup(c))) return rc;
   PRD_CUDA_TRY(c, cudaStreamSynchronize(c->stream));

@@ -214,9 +214,17 @@ static int allow_smem(Ctx* c, K kern) {
 
 template <typename T>
 static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt, const double* fI, T* out, int nO,
-                          const RowAdds& add = RowAdds()) {
-  const double* sp = (const double*)c->sp.p;
-  const int nz = c->nz, N = c->nnu;
+                          const RowAdds& add = RowAdds(), int z0 = 0, int nz = 0) {
+  // all heights, or the nz from z0 on
+  if (!nz) nz = c->nz;
+  const int N = c->nnu;
+  const size_t pt = (size_t)z0 * nO * N;
+  const double* sp = (const double*)c->sp.p + (size_t)z0 * kSpTabs * N;
+  y += 4 * pt;
+  out += 4 * pt;
+  kidx += pt;
+  tt += pt;
+  if (fI) fI += pt;
   if (nz * nO <= kSplFew)
     spline_kernel<T, 1><<<dim3(nO, nz), kSplThreads, SplineSmem<T, 1>::bytes(N), c->stream>>>(y, add, kidx, tt, sp, fI, out, nO, N);
   else
@@ -1025,13 +1033,11 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
   const int ts = std::is_same<A, double>::value
                      ? std::max(1, std::min(c->ntile(), 4 * c->nsm / (nchunk * c->ncls * nz))) : 1;
   bool s3_done = false;   // the tensor-core or double-float contraction ran
-  RowAdds add;            // what the tensor cores contribute to eps_bar
+  int zc = nz;            // heights of a launch of S3 + S4 and S6
   if constexpr (std::is_same<T, float>::value && std::is_same<A, float>::value) {
     if (c->use_tc && c->tc_ready && !t64) {
-      int rc = r2_tc_launch(c, Ic);
-      if (rc) return rc;
-      add = r2_tc_adds(c);
-      s3_done = true;
+      zc = c->tc_zc;
+      s3_done = true;       // below, with S6
     }
   }
   if constexpr (std::is_same<T, double>::value && std::is_same<A, double>::value) {
@@ -1049,11 +1055,25 @@ static int sigma_T(Ctx* c, const A* x, A* eps, bool normalised, A* eb_ext = null
         (const unsigned char*)tb.tiles, (const T*)tb.Y, Ic, (const int*)c->cls_dev.p, eb, c->ncls, c->ntile(),
         nO, N, c->npairs, tb.ld, tb.fmt, ts);
   }
-  stage_end(c, ST_S3, e0);
-  // S6
-  stage_begin(c, ST_S6, &e0);
-  launch_spline<A>(c, eb, (const int*)c->ibk.p, (const double*)c->tbk.p, normalised ? (const double*)c->f.p : nullptr,
-                   eps, nO, add);
+  for (int z0 = 0; z0 < nz; z0 += zc) {
+    const int n = std::min(zc, nz - z0);
+    RowAdds add;            // what the tensor cores contribute to eps_bar
+    if constexpr (std::is_same<T, float>::value && std::is_same<A, float>::value) {
+      if (c->use_tc && c->tc_ready && !t64) {
+        if (z0 > 0) stage_begin(c, ST_S3, &e0);
+        int rc = r2_tc_launch(c, Ic, z0, n);
+        if (rc) return rc;
+        add = r2_tc_adds(c, n);
+      }
+    }
+    const bool last = z0 + n == nz;
+    stage_end(c, ST_S3, e0, last);
+    // S6
+    stage_begin(c, ST_S6, &e0);
+    launch_spline<A>(c, eb, (const int*)c->ibk.p, (const double*)c->tbk.p, normalised ? (const double*)c->f.p : nullptr,
+                     eps, nO, add, z0, n);
+    if (!last) stage_end(c, ST_S6, e0, false);
+  }
   // continuum scattering (App. A) joins the normalised emissivity; the
   // Kirchhoff factor is computed from the line alone (normalised = false)
   if (normalised && c->has_cont())

@@ -190,7 +190,8 @@ struct Ctx {
   int tc_nwork = 0;
   DBuf tc_ent, tc_tail;   // contributions of the records' entries, and of split items' further parts (r2_tc.cu)
   DBuf tc_lists;     // entries of each output direction: [nO + 1] starts, then (entry, place) pairs
-  int tc_nent = 0, tc_split0 = 0, tc_zs = 1;
+  int tc_nent = 0;
+  int tc_zc = 1;     // heights whose contributions tc_ent holds: heights of one contraction launch
   bool tc_ready = false;
   int use_tc = 0;
   long long tc_spin = 0;   // poll limit of the contraction's pipeline waits (0: the default)
@@ -206,7 +207,7 @@ struct Ctx {
   // stage timing (prd_set_profiling): events on the ctx stream around each stage
   bool prof = false;
   std::vector<cudaEvent_t> ev_pool;
-  std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pending;
+  std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_pending;   // stage * 2 + count
   double stage_ms[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   long long stage_n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 
@@ -310,8 +311,10 @@ struct RowAdds {
 __host__ __device__ inline size_t add_off(int g, int idx, int count, int N, int n0, int n) {
   return g == 0 ? (size_t)idx * N + n : (size_t)count * N + ((size_t)(g - 1) * count + idx) * (N - n0) + (n - n0);
 }
-RowAdds r2_tc_adds(const Ctx* c);
-int r2_tc_launch(Ctx* c, const float* Ic);   // contributions to c->tc_ent, added up by the frame change back
+// contributions of the heights z0 .. z0 + n - 1 (n <= tc_zc) to c->tc_ent, and what the frame change
+// back of these heights adds up
+int r2_tc_launch(Ctx* c, const float* Ic, int z0, int n);
+RowAdds r2_tc_adds(const Ctx* c, int n);
 // drop the captured solver graphs (options, tables or workspace changed)
 void invalidate_graphs(Ctx* c);
 // Lockstep rounds of a batched solve (solver.cu): every context of the batch
@@ -327,7 +330,7 @@ int r2_tc_check_error(Ctx* c);
 enum Stage { ST_S1 = 0, ST_S5 = 1, ST_S3 = 2, ST_S6 = 3, ST_S7 = 4, ST_PRE = 5 };
 // Begin / end a timed stage (no-ops unless profiling is on).
 void stage_begin(Ctx* c, int stage, cudaEvent_t* out);
-void stage_end(Ctx* c, int stage, cudaEvent_t start);
+void stage_end(Ctx* c, int stage, cudaEvent_t start, bool count = true);   // count: ends one run of the stage
 void stage_collect(Ctx* c);
 
 // Offset of tile element (row n, column k in [0, 2N): Re | Im halves) within

@@ -93,13 +93,13 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
   const int past = max((int)blockIdx.x - p.split0, 0);
   const int item = min((int)blockIdx.x, p.split0) + past / p.zs;
   const int nparts = item >= p.split0 ? p.zs : 1, part = item >= p.split0 ? past % p.zs : 0;
-  const int iz = item / p.nwork;
+  const int zl = item / p.nwork, iz = p.z0 + zl;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // uniform
   const int et = threadIdx.x - 128;              // index among the Y threads
   constexpr uint32_t tm_cols = NB * 256u;
   const int t0 = p.ntile * part / nparts, t1 = p.ntile * (part + 1) / nparts;
 
-  for (int i = threadIdx.x; i < kRec; i += kThreads) rec[i] = p.work[(size_t)(item - iz * p.nwork) * kRec + i];
+  for (int i = threadIdx.x; i < kRec; i += kThreads) rec[i] = p.work[(size_t)(item - zl * p.nwork) * kRec + i];
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);        // armed by the producer with the bytes of the tile copy
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) r2_tc_kernel(Params p) {
         for (int i = 0; i < kEV; ++i) {
           const int v = 4 * i + og;
           if (v < E) {
-            float4* dst = part == 0 ? p.ent + add_off(gt, iz * p.nent + rec[3] + v, p.nz * p.nent, N, 0, n)
+            float4* dst = part == 0 ? p.ent + add_off(gt, zl * p.nent + rec[3] + v, p.nz * p.nent, N, 0, n)
                                     : p.tail + (part - 1) * (size_t)G * p.nsplit * kMaxE * N +
                                           add_off(gt, (item - p.split0) * kMaxE + v, p.nsplit * kMaxE, N, 0, n);
             *dst = make_float4(acc[i][b][0], acc[i][b][1], acc[i][b][2], acc[i][b][3]);
@@ -406,6 +406,21 @@ static void r2_tc_packed(const Ctx* c, int* n0, int* G) {
   *n0 = !c->split_tiles && c->nnu > 128 ? 128 : 0;
   *G = tc::tiles_per_pass(c->nnu - *n0);
 }
+
+// Every item takes about as long, one CTA per SM: whole waves of a launch's items run as they are, and
+// the tiles of the rest, the n items from split0 on, are split between zs CTAs each, on the SMs of a
+// last wave (at least 4 tiles, or two passes, a CTA).  On 152 SMs, contraction of Mg II 8 heights (768
+// items) 1000 -> 954 us, H I 4 heights x 96 directions 812 -> 779, angle-averaged 512 items 309 -> 272
+// (three FP16 products).
+struct R2Split {
+  int split0, n, zs;
+};
+static R2Split r2_tc_split(const Ctx* c, int nz) {
+  const int items = c->tc_nwork * nz, rest = items % c->nsm;
+  const int zs = rest ? std::min(c->ntile() / std::max(4, 2 * tc::tiles_per_pass(c->nnu)), c->nsm / rest) : 1;
+  return {items - rest, rest, std::max(1, zs)};
+}
+constexpr size_t kEntBytes = (size_t)256 << 20;
 
 // Work records of the contraction: every class's outputs cut into entries of at most two
 // incident directions each (an output with more, as all are in angle-averaged mode,
@@ -478,7 +493,7 @@ int r2_tc_prepare(Ctx* c) {
     if (rc) return rc;
     PRD_CUDA_TRY(c, cudaMemset(c->tc_err.p, 0, sizeof(int)));
   }
-  if (c->prec != PRD_FP32) return PRD_OK;
+  if (c->prec != PRD_FP32 || c->lambda_only) return PRD_OK;   // no contraction
   if (!c->tiled() || c->nnu > 224 || r2_tc_stages(c) < 2)
     return fail(c, PRD_E_ARG, "tensor-core contraction needs FP32 tiles and N small enough for two tile stages "
                               "beside the resident I~ (N <= 224)");
@@ -500,21 +515,24 @@ int r2_tc_prepare(Ctx* c) {
     l[0] = e;
     l[1] = place[e];
   }
-  // Every item takes about as long, one CTA per SM: whole waves of items run as they are, and the
-  // tiles of the rest are split between the SMs of a last wave (at least 4 tiles, or two passes, a
-  // CTA).  On 152 SMs, contraction of Mg II 8 heights (768 items) 1000 -> 954 us, H I 4 heights x 96
-  // directions 812 -> 779, angle-averaged 512 items 309 -> 272.
-  const int items = c->tc_nwork * c->nz, rest = items % c->nsm;
-  c->tc_split0 = items - rest;
+  // The contributions wait in tc_ent for the frame change back, at most kEntBytes of them or one height's
+  // (with all directions as partners an entry count grows as their square), so that they stay a
+  // small part of a context; more heights take several launches.
   int n0, G;
   r2_tc_packed(c, &n0, &G);
   const size_t rows = c->nnu + (size_t)(G - 1) * (c->nnu - n0);   // stored per entry (RowAdds)
-  c->tc_zs = rest ? std::max(1, std::min(c->ntile() / std::max(4, 2 * tc::tiles_per_pass(c->nnu)), c->nsm / rest)) : 1;
+  const size_t per = c->tc_nent * rows * sizeof(float4);
+  c->tc_zc = (int)std::max<size_t>(1, std::min<size_t>(c->nz, kEntBytes / per));
+  size_t tail = 16;
+  for (int n : {c->tc_zc, c->nz % c->tc_zc}) {
+    const R2Split s = r2_tc_split(c, n);
+    tail = std::max(tail, (size_t)(s.zs - 1) * s.n * tc::kMaxE * rows * sizeof(float4));
+  }
   int rc;
   if ((rc = upload(c, c->tc_work, work.data(), work.size() * sizeof(int))) ||
       (rc = upload(c, c->tc_lists, lists.data(), lists.size() * sizeof(int))) ||
-      (rc = dalloc(c, c->tc_ent, c->nz * c->tc_nent * rows * sizeof(float4))) ||
-      (rc = dalloc(c, c->tc_tail, std::max<size_t>(16, (size_t)(c->tc_zs - 1) * rest * tc::kMaxE * rows * sizeof(float4)))))
+      (rc = dalloc(c, c->tc_ent, c->tc_zc * per)) ||
+      (rc = dalloc(c, c->tc_tail, tail)))
     return rc;
   if (c->split_tiles) PRD_CUDA_TRY(c, cudaFuncSetAttribute(r2_tc_pick(c), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   else if ((rc = r2_f32_prepare(c))) return rc;
@@ -523,22 +541,24 @@ int r2_tc_prepare(Ctx* c) {
   return PRD_OK;
 }
 
-RowAdds r2_tc_adds(const Ctx* c) {
+RowAdds r2_tc_adds(const Ctx* c, int n) {
   const int* lists = (const int*)c->tc_lists.p;
+  const R2Split s = r2_tc_split(c, n);
   RowAdds a{(const float4*)c->tc_ent.p, (const float4*)c->tc_tail.p, lists, reinterpret_cast<const int2*>(lists + c->nO + 1 + (c->nO + 1) % 2),
-            c->tc_nent, 1, 0, c->tc_zs, c->tc_split0, c->tc_nwork, c->tc_nwork * c->nz - c->tc_split0};
+            c->tc_nent, 1, 0, s.zs, s.split0, c->tc_nwork, s.n};
   r2_tc_packed(c, &a.n0, &a.G);
   return a;
 }
 
-int r2_tc_launch(Ctx* c, const float* Ic) {
+int r2_tc_launch(Ctx* c, const float* Ic, int z0, int n) {
   // the deepest ring that fits, or the caller's (autotuned) depth if smaller
   const int nmax = r2_tc_stages(c);
   const int nst = c->tc_stages >= 2 ? std::min(c->tc_stages, nmax) : nmax;
-  const int items = c->tc_nwork * c->nz, nsplit = items - c->tc_split0, grid = c->tc_split0 + nsplit * c->tc_zs;
+  const R2Split s = r2_tc_split(c, n);
+  const int grid = s.split0 + s.n * s.zs;
   tc::Params p{(const unsigned char*)c->tiles.p, (const float*)c->Y.p, Ic, (const int*)c->tc_work.p, (float4*)c->tc_ent.p,
                (float4*)c->tc_tail.p, (int*)c->tc_err.p, c->ncls, c->ntile(), c->nO, c->nnu, c->npairs, c->ld(), c->tc_nent,
-               c->nz, c->tc_nwork, c->tc_split0, nsplit, c->tc_zs, nst, 0,
+               n, c->tc_nwork, z0, s.split0, s.n, s.zs, nst, 0,
                c->tc_spin > 0 ? (int)std::min<long long>(c->tc_spin, INT32_MAX) : tc::kSpin};
   if (c->split_tiles) r2_tc_pick(c)<<<grid, tc::kThreads, tc::smem_bytes(c->nnu, nst, c->hi_only), c->stream>>>(p);
   else r2_f32_launch(c, p, grid);

@@ -158,7 +158,8 @@ struct Params {
   float4* ent;          // contributions of the entries (RowAdds)
   float4* tail;         // those of the further parts of split items
   int* err;
-  int ncls, ntile, nO, N, npairs, ld, nent, nz, nwork;
+  int ncls, ntile, nO, N, npairs, ld, nent, nz, nwork;   // nz: heights of this launch
+  int z0;               // first height: the items count from it
   int split0, nsplit, zs;   // the nsplit work items from split0 on have their tiles split between zs CTAs
   int nst;              // tile stages
   int ring;             // bytes of the tile ring (FP32 tiles)

@@ -119,11 +119,11 @@ __global__ void __launch_bounds__(kThreads32, 1) r2_f32_kernel(Params p) {
   const int past = max((int)blockIdx.x - p.split0, 0);
   const int item = min((int)blockIdx.x, p.split0) + past / p.zs;
   const int nparts = item >= p.split0 ? p.zs : 1, part = item >= p.split0 ? past % p.zs : 0;
-  const int iz = item / p.nwork;
+  const int zl = item / p.nwork, iz = p.z0 + zl;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // uniform
   const int t0 = p.ntile * part / nparts, nt = p.ntile * (part + 1) / nparts - t0;   // this part's tiles
 
-  for (int i = threadIdx.x; i < kRec; i += kThreads32) rec[i] = p.work[(size_t)(item - iz * p.nwork) * kRec + i];
+  for (int i = threadIdx.x; i < kRec; i += kThreads32) rec[i] = p.work[(size_t)(item - zl * p.nwork) * kRec + i];
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2 * kStagesMax; ++s) {
       mbar_init(&full[s], 1);              // armed by the producer with the bytes of the copies
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kThreads32, 1) r2_f32_kernel(Params p) {
         for (int i = 0; i < kEV; ++i) {
           const int v = 4 * i + og;
           if (v < E) {
-            float4* dst = part == 0 ? p.ent + add_off(gt, iz * p.nent + rec[3] + v, p.nz * p.nent, N, n0, n)
+            float4* dst = part == 0 ? p.ent + add_off(gt, zl * p.nent + rec[3] + v, p.nz * p.nent, N, n0, n)
                                     : p.tail + (part - 1) * (size_t)p.nsplit * kMaxE * (N + (GX - 1) * (N - n0)) +
                                           add_off(gt, (item - p.split0) * kMaxE + v, p.nsplit * kMaxE, N, n0, n);
             *dst = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
