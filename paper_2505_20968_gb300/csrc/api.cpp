@@ -63,9 +63,8 @@ int upload(Ctx* c, DBuf& b, const void* host, size_t bytes) {
 
 static void free_all(Ctx* c) {
   DBuf* bufs[] = {&c->tiles, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab, &c->kt,
-                  &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk, &c->tin, &c->tbk, &c->cls_dev, &c->dmu,
-                  &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M, &c->pc_lii, &c->pc_eta,
-                  &c->pc_delo, &c->pc_qphi, &c->pc_x, &c->pc_r, &c->pc_v, &c->gm_t,
+                  &c->epsth, &c->f, &c->sp, &c->iin, &c->ibk, &c->tin, &c->tbk, &c->cls_dev, &c->dmu,
+                  &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M, &c->pc_lii, &c->pc_qphi, &c->pc_x, &c->pc_r, &c->pc_v, &c->gm_t,
                   &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_tail, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64, &c->r3out64,
                   &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw, &c->cont_sig,
                   &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S, &c->kt64, &c->epsth64};
@@ -75,8 +74,6 @@ static void free_all(Ctx* c) {
   c->tc_ready = false;
   for (DBuf* b : bufs) dfree(*b);
   for (auto& b : c->adj) dfree(b);
-  for (auto& b : c->krylov) dfree(b);
-  c->krylov.clear();
   for (auto& b : c->owned) dfree(b);
   c->owned.clear();
 }
@@ -379,10 +376,10 @@ int prd_workspace_bytes(const prd_ctx* ctx, int64_t* bytes) {
   if (!ctx || !bytes) return PRD_E_ARG;
   const Ctx* c = &ctx->c;
   const prd::DBuf* bufs[] = {&c->tiles, &c->Y, &c->r3w, &c->r3in, &c->r3out, &c->r3prof, &c->r3J, &c->r3ab,
-                             &c->kt, &c->kt64, &c->epsth64, &c->epsth, &c->f, &c->sp, &c->ugrid, &c->iin, &c->ibk,
+                             &c->kt, &c->kt64, &c->epsth64, &c->epsth, &c->f, &c->sp, &c->iin, &c->ibk,
                              &c->tin, &c->tbk,
                              &c->cls_dev, &c->scratch2, &c->scratch3, &c->pc_phi, &c->pc_M,
-                             &c->pc_lii, &c->pc_eta, &c->pc_delo, &c->gm_t, &c->dmu, &c->pc_qphi, &c->pc_x,
+                             &c->pc_lii, &c->gm_t, &c->dmu, &c->pc_qphi, &c->pc_x,
                              &c->pc_r, &c->pc_v, &c->tc_err, &c->tc_work, &c->tc_ent, &c->tc_tail, &c->tc_lists, &c->tiles64, &c->Y64, &c->r3w64, &c->r3in64,
                              &c->r3out64, &c->r3prof64, &c->r3ab64, &c->par, &c->eta_line, &c->cont_pw,
                              &c->cont_sig, &c->gk_V, &c->gk_r, &c->gk_w, &c->gk_cur, &c->gk_S};

@@ -390,18 +390,11 @@ int build_device_tables(Ctx* c) {
     std::vector<double> ones(npt, 1.0);
     if ((rc = upload(c, c->f, ones.data(), npt * 8))) return rc;   // FP64 in both modes
   }
-  // ---- preconditioner scalar formal-solver tables: eta1 and DELO weights
+  // ---- preconditioner: local DELO weight of S = eps/eta1
   {
-    std::vector<double> pe(npt), pd(npt * 3), lii(npt);
-    for (size_t i = 0; i < npt; ++i) {
-      pe[i] = eta[i];
-      pd[3 * i] = kt[10 * i + 7];
-      pd[3 * i + 1] = kt[10 * i + 8];
-      pd[3 * i + 2] = kt[10 * i + 9];
-      lii[i] = kt[10 * i + 9] / eta[i];     // local DELO weight of S = eps/eta1
-    }
-    if ((rc = upload_T(c, c->pc_eta, pe)) || (rc = upload_T(c, c->pc_delo, pd)) || (rc = upload_T(c, c->pc_lii, lii)))
-      return rc;
+    std::vector<double> lii(npt);
+    for (size_t i = 0; i < npt; ++i) lii[i] = kt[10 * i + 9] / eta[i];
+    if ((rc = upload_T(c, c->pc_lii, lii))) return rc;
     c->pc_lii_host = lii;
   }
   // ---- R_II contraction coefficients Y[z][pair][t][i][j] (complex)
@@ -493,15 +486,14 @@ int build_device_tables(Ctx* c) {
       return rc;
     if ((rc = dalloc(c, c->r3J, (size_t)nz * nuv * 2 * sizeof(double)))) return rc;
   }
-  // ---- spline tables: per height h, Thomas factors (cp, den), grid
+  // ---- spline tables
   {
-    std::vector<double> sp((size_t)nz * kSpTabs * N, 0.0), ug((size_t)nz * N);
+    std::vector<double> sp((size_t)nz * kSpTabs * N, 0.0), h(N);
     for (int iz = 0; iz < nz; ++iz) {
       const double* u = &c->u[(size_t)iz * N];
-      double* h = &sp[(size_t)iz * kSpTabs * N];
-      double *cp = h + kSpCp * N, *den = h + kSpDen * N, *k6 = h + kSpK6 * N;
-      double *e0 = h + kSpE0 * N, *e1 = h + kSpE1 * N, *cg = h + kSpCg * N;
-      double *iden = h + kSpIden * N, *s6 = h + kSp6h * N;
+      double* tab = &sp[(size_t)iz * kSpTabs * N];
+      double *cp = tab + kSpCp * N, *k6 = tab + kSpK6 * N, *e0 = tab + kSpE0 * N, *e1 = tab + kSpE1 * N;
+      double *cg = tab + kSpCg * N, *iden = tab + kSpIden * N, *s6 = tab + kSp6h * N;
       for (int i = 0; i < N - 1; ++i) {
         h[i] = u[i + 1] - u[i];
         k6[i] = h[i] * h[i] / 6.0;
@@ -512,17 +504,14 @@ int build_device_tables(Ctx* c) {
         const int i = r + 1;
         const double sub = (r > 0) ? h[i - 1] : 0.0;
         const double dn = 2.0 * (h[i - 1] + h[i]) - sub * (r > 0 ? cp[r - 1] : 0.0);
-        den[r] = dn;
         cp[r] = (r < m - 1) ? h[i] / dn : 0.0;
         cg[r] = sub / dn;
         iden[r] = 1.0 / dn;
         e0[r] = 6.0 / (h[i - 1] * dn);
         e1[r] = 6.0 / (h[i] * dn);
       }
-      for (int n = 0; n < N; ++n) ug[(size_t)iz * N + n] = u[n];
     }
     if ((rc = upload(c, c->sp, sp.data(), sp.size() * 8))) return rc;   // FP64 always
-    if ((rc = upload_T(c, c->ugrid, ug))) return rc;
     // interpolation points: in  = u_n - u_b(o) (observer -> comoving, Sect. 4.1)
     //                        back = u_n + u_b(o) (comoving -> observer)
     std::vector<int> iin(npt), ibk(npt);

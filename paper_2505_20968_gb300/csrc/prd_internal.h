@@ -28,11 +28,11 @@ constexpr int kWeidemanN64 = 36;   // Faddeeva expansion terms, FP64 paths
 constexpr int kAAThetaNodes = 48;
 
 // Spline tables of a height (natural cubic spline on its reduced-frequency grid), each of N
-// doubles: interval widths h, the Thomas factors of the second derivatives' tridiagonal system
-// (row r, node r + 1) cp and den, h^2/6, and the system divided by its pivots: right-hand side
+// doubles: h^2/6 and 6/h of the interval widths h, and the second derivatives' tridiagonal system
+// (row r, node r + 1) divided by its pivots: right-hand side
 // e1[r] (y_{r+2} - y_{r+1}) - e0[r] (y_{r+1} - y_r), forward g_r = rhs_r - cg[r] g_{r-1},
-// backward M_{r+1} = g_r - cp[r] M_{r+2}; the reciprocal pivots, and 6/h.
-enum SpTab { kSpH = 0, kSpCp = 1, kSpDen = 2, kSpK6 = 3, kSpE0 = 4, kSpE1 = 5, kSpCg = 6, kSpIden = 7, kSp6h = 8, kSpTabs = 9 };
+// backward M_{r+1} = g_r - cp[r] M_{r+2}; the reciprocal pivots.
+enum SpTab { kSpCp = 0, kSpK6 = 1, kSpE0 = 2, kSpE1 = 3, kSpCg = 4, kSpIden = 5, kSp6h = 6, kSpTabs = 7 };
 // Storage of the context's R_II tiles (kernels_tiles.cu, group_split_kernel)
 enum TileFmt { TILE_PLAIN = 0, TILE_F32 = 1, TILE_BF16 = 2, TILE_BF16HI = 3 };
 // dynamic shared memory a CTA may have (opt-in limit of the device)
@@ -107,8 +107,6 @@ struct Ctx {
   std::vector<double> Dmat;              // [z][3][ku][kl] dipole elements <ku|d_q|kl>
   std::vector<double> Rmag;              // [z][3][3] rows of the magnetic frame
   std::vector<double> Q;                 // [z][n][n] natural-spline 2nd-derivative map
-  std::vector<int> theta_node_cls;       // AA: unused
-  int n_aa_theta = 0;
   std::vector<double> aa_theta, aa_w;     // AA Theta rule
 
   // ---- device
@@ -143,7 +141,6 @@ struct Ctx {
   DBuf epsth;        // [z][o][n][4]
   DBuf f;            // [z][o][n]
   DBuf sp;           // spline tables [z][kSpTabs][N] (double), SpTab below
-  DBuf ugrid;        // [z][N] (T)
   DBuf iin, ibk;     // interpolation [z][o][n]: int k | flag, and t (T)  -> int2/ T pairs
   DBuf tin, tbk;
   DBuf cls_dev;      // cout_ptr, cout_dir, pair_ptr, pair_in  (int)
@@ -153,15 +150,12 @@ struct Ctx {
   DBuf pc_phi;       // [z][N][N] Phi_bar (double)
   DBuf pc_M;         // [z][N][N] Phi_bar (Id - A)^-1 (double)
   DBuf pc_lii;       // [z][o][n] Lambda_ii (T)
-  DBuf pc_eta;       // [z][o][n]: eta1 (T)  (scalar Lambda*)
-  DBuf pc_delo;      // [z][o][n][3] (T)
   DBuf pc_qphi;      // [z][N][N] spline second derivatives of Phi_bar's columns (double)
   DBuf pc_x, pc_r;   // [z][o][n] iterate and residual of the sweeps (double)
   DBuf pc_v;         // [2][z][N] eps* before the frame change back: values, spline second derivatives (double)
   std::vector<double> pc_lii_host;
   void* pc_w = nullptr;   // device angular weights (double), owned via `owned`
   // GMRES
-  std::vector<DBuf> krylov;
   DBuf gm_t;
   // GMRES workspace kept across solves (basis V[m+1], residual r, operator
   // output w, current basis vector, device state), and the Arnoldi step
@@ -290,7 +284,6 @@ int solve(Ctx* c, double tol, int max_iter, int restart, const void* x0, void* x
 int emergent(Ctx* c, const void* x, int nlos, const double* mu, const double* chi, void* out);
 int narrowband(Ctx* c, const void* x, int nlos, const double* mu, const double* chi, double lam0, double fwhm,
                double half, double* out);
-int upload_faddeeva_coeffs(Ctx* c);
 
 size_t nvec(const Ctx* c);   // 4*nz*nO*nnu
 int r2_tc_prepare(Ctx* c);
