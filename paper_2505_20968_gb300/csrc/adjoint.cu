@@ -233,11 +233,11 @@ __global__ void __launch_bounds__(256) r2_t_kernel(const double* __restrict__ ti
         const int mm = q / NC, col = q - mm * NC;
         const int m = m0 + mm, e = col >> 2, i = col & 3;
         double zr = 0.0, zi = 0.0;
-          for (int n = 0; n < N; ++n) {
-            const double gv = gs[((size_t)e * N + n) * 4 + i];
-            zr += T[(size_t)n * ld + m] * gv;
-            zi -= T[(size_t)n * ld + N + m] * gv;
-          }
+        for (int n = 0; n < N; ++n) {
+          const double gv = gs[((size_t)e * N + n) * 4 + i];
+          zr += T[(size_t)n * ld + m] * gv;
+          zi -= T[(size_t)n * ld + N + m] * gv;
+        }
         zs[q * 2] = zr;
         zs[q * 2 + 1] = zi;
       }

@@ -34,11 +34,10 @@ template <> struct V4<double> { using type = double4_16a; };
 // step: an FP32 apply of 8 x 64 rows of 200 points 3399 -> 2952 us, of 10 x 16 rows of
 // 27 points 262 -> 201 us, a preconditioner apply of 20 x 16 rows of 100 points
 // (four FP64 frame changes) 1097 -> 217 us.
-// R = 4 rows a CTA (16 recurrences in a warp) where there are rows enough for
+// R = 4 rows a CTA (16 recurrences in a warp) where there are more than four rows for
 // every SM, R = 1 below that, so that the right-hand sides and evaluations of a
 // small problem still spread over the chip.
 constexpr int kSplThreads = 128;
-constexpr int kSplFew = 4 * 152;                     // rows up to which a CTA takes one
 
 template <typename T, int R>
 struct SplineSmem {
@@ -225,7 +224,7 @@ static void launch_spline(Ctx* c, const T* y, const int* kidx, const double* tt,
   kidx += pt;
   tt += pt;
   if (fI) fI += pt;
-  if (nz * nO <= kSplFew)
+  if (nz * nO <= 4 * c->nsm)
     spline_kernel<T, 1><<<dim3(nO, nz), kSplThreads, SplineSmem<T, 1>::bytes(N), c->stream>>>(y, add, kidx, tt, sp, fI, out, nO, N);
   else
     spline_kernel<T, 4><<<dim3((nO + 3) / 4, nz), kSplThreads, SplineSmem<T, 4>::bytes(N), c->stream>>>(y, add, kidx, tt, sp, fI, out, nO, N);
@@ -1354,7 +1353,7 @@ static int emergent_T(Ctx* c, const T* x, int nlos, const double* mus, const dou
     launch_r3_out<T, A>(c, (const double*)Jw.p, (const T*)rout.p, (A*)ew_bar.p, 1, tb);
     // R_II: tiles of the heights for the LOS classes, zb heights at a time, then the contraction
     if (ncl > 1 && (rc = los_tiles_angles(c, lt, L.theta))) break;
-    const int tg = (size_t)nO * nz >= 608 ? nti : 1;
+    const int tg = nO * nz >= 4 * c->nsm ? nti : 1;      // enough CTAs for the SMs with all tiles in one
     for (int z0 = 0; z0 < nz && !rc; z0 += zb) {
       const int n = std::min(zb, nz - z0);
       if ((rc = los_tiles_gen(c, lt, z0, n, tiles.p))) break;
