@@ -12,6 +12,7 @@
 #include <type_traits>
 #include "prd_internal.h"
 #include "device_common.cuh"
+#include "ring.h"
 
 namespace prd {
 
@@ -789,7 +790,7 @@ __global__ void delo_kernel(const A* __restrict__ eps, const T* __restrict__ kt,
 // kDR points) with bulk asynchronous copies into a ring of kDStages heights;
 // the kDR consumer threads (one per ray) take their point from shared memory.
 // Needs an even frequency count (16-byte aligned slices).  Every wait is
-// bounded: on expiry the CTA stops, the producer drains its copies, and the
+// bounded: on expiry the CTA stops, its copies are drained, and the
 // error flag is raised (PRD_E_TIMEOUT through prd_device_status).
 constexpr int kDR = 128;                       // rays per CTA
 constexpr int kDStages = 8;                    // heights in flight per CTA
@@ -849,11 +850,12 @@ __global__ void __launch_bounds__(32 + kDR) delo_staged_kernel(const A* __restri
   }
   __syncthreads();
   auto row = [&](int p) { return ((size_t)(up ? p : nz - 1 - p) * nO + o) * N + n0; };
+  int filled = 0;                                // heights thread 0 has issued copies for
   if (threadIdx.x < 32) {
     if (threadIdx.x == 0) {
       const uint32_t bkt = (uint32_t)R * 10 * sizeof(T), bv = (uint32_t)R * 4 * sizeof(A), bp = (uint32_t)R * 24;
       const uint32_t bytes = bkt + bv + (x_sub ? bv : 0u) + (par ? bp : 0u);
-      int p = 0;
+      int& p = filled;
       for (; p < nz; ++p) {
         const int d = p % kDStages;
         if (p >= kDStages && !dbar_wait(&empty[d], ((p / kDStages) - 1) & 1, abort_flag)) break;
@@ -873,10 +875,6 @@ __global__ void __launch_bounds__(32 + kDR) delo_staged_kernel(const A* __restri
         if (x_sub) copy(st + L::kXs, x_sub + r0 * 4, bv);
         if (par) copy(st + L::kPar, par + r0 * 3, bp);
       }
-      if (*abort_flag)   // drain copies that were issued and may not have been consumed
-        for (int q = max(0, p - kDStages); q < p; ++q)
-          for (long long i = 0; i < kDSpin && !dbar_try(&full[q % kDStages], (q / kDStages) & 1); ++i) {
-          }
     }
   } else {
     const int r = threadIdx.x - 32;
@@ -922,7 +920,15 @@ __global__ void __launch_bounds__(32 + kDR) delo_staged_kernel(const A* __restri
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag && err) atomicExch(err, 1);
+  if (threadIdx.x == 0 && *abort_flag) {
+    // a wait gave up: copies that nobody has waited for may be in flight, also those of a producer
+    // that had already issued its last
+    ring_drain(filled, kDStages, [&](int d, uint32_t parity) {
+      for (long long i = 0; i < kDSpin && !dbar_try(&full[d], parity); ++i) {
+      }
+    });
+    if (err) atomicExch(err, 1);
+  }
 }
 
 template <typename T, typename A>
