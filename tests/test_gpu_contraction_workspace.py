@@ -1,5 +1,5 @@
 """The workspace of the tensor-core contraction: a small part of a context whatever the number of
-directions and heights (at most 256 MiB, or one height), there before the FP64 copy of the tiles
+directions and heights (at most 1 GiB, or one height), there before the FP64 copy of the tiles
 is weighed against free memory; problems of more heights than it holds take several launches,
 which agree with the CUDA-core contraction as one launch does (5e-6 of each height's largest
 emissivity, the bound between the two paths)."""
@@ -47,10 +47,10 @@ def test_workspace_comes_before_the_fp64_tiles():
 
 def test_heights_in_several_launches():
     from paper_2505_20968_gb300.binding import PRD
-    nz, nnu, nO = 31, 128, 96
+    nz, nnu, nO = 38, 224, 128
     per = nO * (nO // 2) * nnu * 16
-    assert 1 < (256 << 20) // per < nz
-    cfg = inputs.hi_lya(n_z=nz, n_core=nnu - 6, n_wing=6, n_mu_half=6, n_chi=8, seed=6, mode=inputs.MODE_AA)
+    assert 1 < (1 << 30) // per < nz
+    cfg = inputs.hi_lya(n_z=nz, n_core=nnu - 6, n_wing=6, n_mu_half=8, n_chi=8, seed=6, mode=inputs.MODE_AA)
     P = PRD(cfg, device=0)
     x = torch.from_numpy(inputs.seeded_vector(P.shape, 6, 0.1, 1.0)).to("cuda", torch.float32)
     out = P.apply_sigma(x)
