@@ -9,8 +9,9 @@
 // and three products, as contexts of bf16 planes do.
 //
 // What bounds it: the tensor pipe (64 clocks a product of 128 x 128 x 16) and shared memory,
-// which at 128 bytes a clock can feed both operands of one such product in just that time; and the
-// schedulers, which the split and Y share with the warp that issues the products.
+// which at 128 bytes a clock can feed both operands of one such product in just that time; beside
+// them the schedulers, which the split and Y share with the warp that issues the products (ncu, 4
+// heights of the problem below: tensor pipe 64 %, issue slots 55 %, HBM 47 % of the measured rate).
 // So the tile goes through registers into TMEM, the one place that a product can take its first
 // operand from without shared memory: four warps, a thread a row, read a landed FP32 step, split it
 // and store its planes as packed columns, and only I~ is read from shared memory.  TMEM
@@ -23,12 +24,14 @@
 // to shared memory for the products, 2350 us; through TMEM, 1570 with eight split warps in one step
 // each; remainders by mixed-precision fma and barriers looked at ahead 1530; hand-overs of four K
 // steps 1505; four split warps of two steps each (fewer instructions beside the products' warp)
-// 1455.  The products alone take 1140 to 1250 here (probe: 980), split, Y and copies without them 1270.
+// 1455; the look ahead in the middle of a turn 1420.  The products alone take 1140 to 1250 here
+// (a loop without other warps: 970), split, Y and copies without them 1270.
 // Without gain: fetching the tiles into L2 ahead (the ring is shallow, three stages, at 200
-// frequencies), Y's columns read an entry ahead, eight Y warps of 16 entries.
+// frequencies), Y's columns read an entry ahead, eight Y warps of 16 entries, a split group for each
+// slot, registers moved to the Y warps (setmaxnreg).
 // Measured, contraction (before: scaled FP16 pairs, three products; before that: three TF32 products of
-// an operand formed per K step): that problem 2795, 954, now 1455 us; H I 4 x 96 x 150 779 -> 826; H I
-// angle-averaged 8 x 64 x 91 272 -> 380; Mg II 10 x 16 x 27 24 -> 29.
+// an operand formed per K step): that problem 2795, 954, now 1420 us; H I 4 x 96 x 150 779 -> 816; H I
+// angle-averaged 8 x 64 x 91 272 -> 379; Mg II 10 x 16 x 27 24 -> 29.
 //
 // Roles (704 threads): warp 0 streams the tile into a ring of K step pairs (bulk copies) and owns the
 // TMEM allocation; warp 1 issues tcgen05.mma; warps 2-5 split; warps 6-21 stage I~ and Y and apply
@@ -222,7 +225,8 @@ __global__ void __launch_bounds__(kThreads32, 1) r2_f32_kernel(Params p) {
       if (!r) *abort_flag = 1;
       live = r;
     }
-    // A slot (four K steps) a turn, whose barrier is looked at a turn ahead.  What may come in
+    // A slot (four K steps) a turn, whose barrier is looked at in the middle of the turn before (at its
+    // start the slot is still being filled, and the wait cost 2 % more).  What may come in
     // the middle of a turn, the end of a half and the next one's wait for its accumulators, costs
     // no branch between the products: the commit is predicated, the wait taken at the turn's start
     // (branches a step cost 100 clocks a stage).  Halves of less than a turn (and a last turn of one
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(kThreads32, 1) r2_f32_kernel(Params p) {
     for (int it = 0; it < iters && live; it += 2) {
       const int cnt = min(2, iters - it);
       if (!__all_sync(0xffffffffu, ahead)) wait(&aready[sl], ph);
-      ahead = it + 2 < iters && mbar_test(&aready[sl ^ 1], ph ^ sl);
+      ahead = false;
       if (cnt == 2 && KH >= kTurn) {
         // a half's accumulators are free once Y has been applied to the pass before
         const bool starts = kc == 0, next = kc + kTurn > KH;
@@ -262,6 +266,7 @@ __global__ void __launch_bounds__(kThreads32, 1) r2_f32_kernel(Params p) {
         for (int v = 0; v < kTurn; ++v) {
           const bool wrap = kc + v >= KH;
           if (live && elect_one()) products(v, wrap ? h ^ 1 : h, wrap ? kc + v - KH : kc + v);
+          if (v == 1) ahead = it + 2 < iters && mbar_test(&aready[sl ^ 1], ph ^ sl);
         }
         kc += kTurn;
         if (kc >= KH) {
