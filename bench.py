@@ -33,7 +33,7 @@ UNIT = "applies/s"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 # layout tag of the contraction whose DRAM traffic profiles/traffic.json records;
 # the traffic figure is reported only while it matches the kernel that runs
-KERNEL_LAYOUT = "planes-v6"
+KERNEL_LAYOUT = "f32-v7"
 # what each value of --contraction multiplies on the tensor cores
 PRODUCTS = {"tf32x3": "bf16 planes x6, FP32 level", "bf16x3": "bf16 planes x3", "bf16x2": "bf16 hi plane x2"}
 N_PRODUCTS = {"tf32x3": 6.0, "bf16x3": 3.0, "bf16x2": 2.0}
@@ -406,24 +406,28 @@ def main():
     useful, n_theta_omega = useful_contraction_flops(P, n_t=n_t)
     peaks, src = _peaks()
     # The contraction runs six products of bf16 planes per FP32-level product (three or two for
-    # the bf16 precisions); streaming the tiles once still takes longer at the measured HBM rate
-    # than those products at the measured bf16 rate, so HBM bounds it.  `achieved` counts the tile
-    # bytes; `useful_tflops` the useful work F3 and `issued_frac` the products over the stored
-    # tiles (J-level means plus per-triple deviations, 20 per angle class) against the tensor peak.
+    # the bf16 precisions) and streams the tiles once; the longer of the two at the measured bf16 and
+    # HBM rates bounds it (FP32: the products).  `issued` counts the products over the stored tiles
+    # (J-level means plus per-triple deviations, 20 per angle class), `useful_tflops` the useful
+    # work F3 and `hbm` the tile bytes.
     achieved_tf = useful / (r2_ms * 1e-3) / 1e12
     issued_tf = N_PRODUCTS[args.contraction] * flops / (r2_ms * 1e-3) / 1e12
     achieved_gbs = tile_bytes / (r2_ms * 1e-3) / 1e9
+    kernel = "r2_f32_kernel" if args.contraction == "tf32x3" else "r2_tc_kernel"
+    tensor_bound = issued_tf / peaks["bf16_tflops"] > achieved_gbs / peaks["hbm_gbs"]
     traffic = None
     try:
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
             tr = json.load(f)
-        if tr.get("kernel") == "r2_tc_kernel" and tr.get("workload") == "mgii" and tr.get("layout") == KERNEL_LAYOUT:
+        if tr.get("kernel") == kernel and tr.get("workload") == "mgii" and tr.get("layout") == KERNEL_LAYOUT:
             traffic = tr.get("dram_bytes_per_launch")
     except (OSError, ValueError):
         pass
-    roofline = {"bound": "hbm", "kernel": f"r2_tc_kernel (S3+S4 R_II contraction, tcgen05, {PRODUCTS[args.contraction]})",
-                "achieved": achieved_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved_gbs / peaks["hbm_gbs"],
+    bound = ({"bound": "tensor", "achieved": issued_tf, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s issued",
+              "frac": issued_tf / peaks["bf16_tflops"]} if tensor_bound else
+             {"bound": "hbm", "achieved": achieved_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+              "frac": achieved_gbs / peaks["hbm_gbs"]})
+    roofline = {**bound, "kernel": f"{kernel} (S3+S4 R_II contraction, tcgen05, {PRODUCTS[args.contraction]})",
                 "useful_tflops": achieved_tf, "useful_frac": achieved_tf / peaks["bf16_tflops"],
                 "issued": issued_tf, "issued_frac": issued_tf / peaks["bf16_tflops"],
                 "peak_source": src, "traffic": traffic,
@@ -481,7 +485,7 @@ def main():
         sol16, info16 = Pb.solve(tol=args.solve_tol, max_iter=900, restart=200, check=False)
         torch.cuda.synchronize()
         modes["bf16x3"] = {"contraction_ms": b16_ms, "useful_tflops": useful / (b16_ms * 1e-3) / 1e12,
-                           "issued_frac_of_bf16_peak": N_PRODUCTS[args.contraction] * flops / (b16_ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
+                           "issued_frac_of_bf16_peak": N_PRODUCTS["bf16x3"] * flops / (b16_ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
                            "hbm_frac": tile_bytes / (b16_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                            "solve_seconds": time.time() - t0, "solve_applies": info16["iters"],
                            "solve_true_rel_res": info16["true_rel_res"], "rc": info16["rc"],

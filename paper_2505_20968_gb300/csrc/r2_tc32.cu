@@ -11,7 +11,7 @@
 // What bounds it: the tensor pipe (64 clocks a product of 128 x 128 x 16) and shared memory,
 // which at 128 bytes a clock can feed both operands of one such product in just that time; beside
 // them the schedulers, which the split and Y share with the warp that issues the products (ncu, 4
-// heights of the problem below: tensor pipe 64 %, issue slots 55 %, HBM 47 % of the measured rate).
+// heights of the problem below: tensor pipe 65 %, issue slots 56 %, HBM 45 % of the measured rate).
 // So the tile goes through registers into TMEM, the one place that a product can take its first
 // operand from without shared memory: four warps, a thread a row, read a landed FP32 step, split it
 // and store its planes as packed columns, and only I~ is read from shared memory.  TMEM
