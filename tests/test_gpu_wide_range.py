@@ -7,8 +7,8 @@ emissivity that spans as much, frequency by frequency made of the field near it.
 elastic collisions (no R_III, which spreads the core over the wings) every element is compared
 with its own size: perturbing the field by 1e-7 moves the elements by at most 1e-6 (evaluated
 with the oracle), FP32 tiles, field and frame changes are some ten such roundings and at most 240
-partial sums of 2^-23 a product chain; 1e-4 covers their product and is a hundredth of what a
-field or tile held to 2^-24 of its largest element would leave."""
+partial sums of 2^-23 a product chain; 1e-4 covers their product.  (Operands under one scale a row,
+which hold a value to 2^-38 of the row's largest, exceed it.)"""
 import numpy as np
 import pytest
 import torch
