@@ -16,6 +16,14 @@
 
 namespace prd {
 
+// (s, c) += x (x exact float); error-free two-sum of s and x into s, error into c
+__device__ __forceinline__ void dd_add(float& s, float& c, float x) {
+  const float t = s + x;
+  const float bb = t - s;
+  c += (s - (t - bb)) + (x - bb);
+  s = t;
+}
+
 // ------------------------------------------------------------------ splines
 template <typename T> struct V4;
 template <> struct V4<float> { using type = float4; };
@@ -83,7 +91,14 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
           V v = src[(size_t)r * N + i];
           if constexpr (sizeof(T) == 4) {
             if (add.ent) {
-              // the entries' parts, eight loads at a time, added in order
+              // the entries' parts, eight loads at a time, added in order; their rounding errors are kept
+              // and added last: the largest error against FP64 over eight grids of 27 to 200 points is
+              // 3.3e-7 to 5.3e-7 instead of 4.9e-7 to 7.4e-7, for 1 to 6 us of the frame change
+              float4 err = make_float4(0.f, 0.f, 0.f, 0.f);
+              auto sum = [&](float4 w) {
+                dd_add(v.x, err.x, w.x); dd_add(v.y, err.y, w.y);
+                dd_add(v.z, err.z, w.z); dd_add(v.w, err.w, w.w);
+              };
               const int e0 = add.ptr[o0 + r], e1 = add.ptr[o0 + r + 1], cnt = gridDim.y * add.nent;
               const int G = i >= add.n0 ? add.G : 1;
               for (int e = e0, p = 0; e < e1;) {
@@ -97,7 +112,7 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
                   }
                 }
 #pragma unroll
-                for (int q = 0; q < 8; ++q) { v.x += w[q].x; v.y += w[q].y; v.z += w[q].z; v.w += w[q].w; }
+                for (int q = 0; q < 8; ++q) sum(w[q]);
               }
               // and the further parts of this height's split items
               if (add.zs > 1 && (iz + 1) * add.nwork > add.split0) {
@@ -108,13 +123,13 @@ __global__ void __launch_bounds__(kSplThreads) spline_kernel(const T* __restrict
                   for (int g = 0; g < G; ++g) {
                     const float4* a = add.tail + add_off(g, it * 32 + (l & 31), add.nsplit * 32, N, add.n0, i);
 #pragma unroll 8
-                    for (int p = 0; p < add.zs - 1; ++p) {
-                      const float4 w = a[p * ps];
-                      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-                    }
+                    for (int p = 0; p < add.zs - 1; ++p) sum(a[p * ps]);
                   }
                 }
               }
+              // (a sum that overflowed has no rounding error: it stays the infinity that it is)
+              v.x += err.x == err.x ? err.x : 0.f; v.y += err.y == err.y ? err.y : 0.f;
+              v.z += err.z == err.z ? err.z : 0.f; v.w += err.w == err.w ? err.w : 0.f;
             }
           }
           ys[r * S + i] = v;
@@ -496,13 +511,6 @@ struct F2 { float hi, lo; };
 __device__ __forceinline__ F2 split2(double a) {
   const float h = (float)a;
   return {h, (float)(a - (double)h)};
-}
-// (s, c) += x (x exact float); error-free two-sum of s and x into s, error into c
-__device__ __forceinline__ void dd_add(float& s, float& c, float x) {
-  const float t = s + x;
-  const float bb = t - s;
-  c += (s - (t - bb)) + (x - bb);
-  s = t;
 }
 
 __global__ void __launch_bounds__(256) r2_dd_kernel(const double* __restrict__ tiles, const double* __restrict__ Y,
